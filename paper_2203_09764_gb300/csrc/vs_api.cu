@@ -403,7 +403,7 @@ extern "C" vs_status vs_centrifuge(vs_field *f, double omega, uint64_t seed) {
     // the centrifuged links are built in the original gauge from the labels
     if (f->gauge_on) return fail(VS_EINVAL, "vs_centrifuge: field in a random gauge (centrifuge first)");
     CK(cudaSetDevice(f->ctx->opt.device));
-    CK(launch_centrifuge(f->prec == VS_FP32, f->nc, f->g, f->ref, omega, seed, f->U, f->stream));
+    CK(launch_centrifuge(f->prec == VS_FP32, f->nc, f->g, f->ref, omega, seed, f->U, f->partials, f->stream));
     return VS_OK;
 }
 

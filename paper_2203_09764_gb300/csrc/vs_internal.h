@@ -130,8 +130,9 @@ cudaError_t launch_count_nonfinite(int prec, int nc, const Geo &g, const void *U
                                    cudaStream_t st);
 cudaError_t launch_current_labels(int prec, int nc, const Geo &g, const void *U, int8_t *out_lex,
                                   cudaStream_t st);
+// table: scratch of at least 294 doubles, 16-byte aligned
 cudaError_t launch_centrifuge(int prec, int nc, const Geo &g, const int8_t *ref, double omega,
-                              uint64_t seed, void *U, cudaStream_t st);
+                              uint64_t seed, void *U, double *table, cudaStream_t st);
 // mean over sites of S(x)/beta into *out (device double); partials: n_part doubles
 int action_partials(const Geo &g);
 cudaError_t launch_action(int prec, int nc, const Geo &g, const void *U, double *partials,

@@ -3,6 +3,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cmath>
+#include <type_traits>
 
 #include "vs_internal.h"
 #include "vs_stout.cuh"
@@ -52,41 +53,59 @@ __global__ void __launch_bounds__(kThreads) k_load_labels(Geo g, const int8_t *_
     }
 }
 
-// Links from FP64 host layout; the reference label is the sector of arg Tr U of the FP64 input.
-template <class T, int NC>
-__global__ void k_load_links(Geo g, const double *__restrict__ in, T *U, int8_t *ref) {
-    long long l = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (l >= 4ll * g.V) return;
-    int mu = (int)(l / g.V), s = (int)(l % g.V);
-    Pt p = site_of_lex(g, s);
-    int i = sidx(g, p);
-    const double *q = in + l * 18;
+// FP64 link matrices of the caller ([..][9] (re, im) pairs, 144 bytes per matrix)
+// pass through shared memory on their way in and out: a warp's global accesses
+// are then runs of 256 bytes, where one thread per matrix touches 32 sectors
+// 144 bytes apart with every 8-byte access (read at 32^3x64: 1.02 ms that way,
+// against the 0.27 ms that its 1.8 GB take at the copy rate).  The accesses stay
+// 8 bytes wide because the caller's pointer need not be aligned to more.  A
+// block takes kThreads consecutive sites of one direction (V is a multiple of
+// 256: every extent is a multiple of 4).
+template <class T>
+__device__ __forceinline__ M3<T> staged_matrix(const double *__restrict__ in, double *sm, double &tr, double &ti) {
+#pragma unroll
+    for (int k = 0; k < 18; ++k) sm[k * kThreads + threadIdx.x] = in[k * kThreads + threadIdx.x];
+    __syncthreads();
+    const double2 *q = reinterpret_cast<const double2 *>(sm) + 9 * threadIdx.x;
     M3<T> m;
-    double tr = 0, ti = 0;
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
-        m.re[k] = T(q[2 * k]);
-        m.im[k] = T(q[2 * k + 1]);
+        const double2 v = q[k];
+        m.re[k] = T(v.x);
+        m.im[k] = T(v.y);
+        if (k == 0) { tr = v.x; ti = v.y; }
+        if (k == 4 || k == 8) { tr += v.x; ti += v.y; }
     }
-    tr = q[0] + q[8] + q[16];
-    ti = q[1] + q[9] + q[17];
+    return m;
+}
+
+// Links from FP64 host layout; the reference label is the sector of arg Tr U of the FP64 input.
+template <class T, int NC>
+__global__ void __launch_bounds__(kThreads) k_load_links(Geo g, const double *__restrict__ in, T *U, int8_t *ref) {
+    __shared__ __align__(16) double sm[kThreads * 18];
+    const int mu = blockIdx.y, s0 = blockIdx.x * kThreads;
+    double tr, ti;
+    const M3<T> m = staged_matrix<T>(in + ((long long)mu * g.V + s0) * 18, sm, tr, ti);
+    const int i = sidx(g, site_of_lex(g, s0 + threadIdx.x));
     store_link<T, NC>(U, g.P, mu, i, m);
     ref[(long long)mu * g.P + i] = (int8_t)z3_label<double>(tr, ti);
 }
 
 template <class T, int NC>
-__global__ void k_read_links(Geo g, const T *__restrict__ U, double *out) {
-    long long l = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (l >= 4ll * g.V) return;
-    int mu = (int)(l / g.V), s = (int)(l % g.V);
-    Pt p = site_of_lex(g, s);
-    M3<T> m = load_link<T, NC>(U, g.P, mu, sidx(g, p));
-    double *q = out + l * 18;
+__global__ void __launch_bounds__(kThreads) k_read_links(Geo g, const T *__restrict__ U, double *out) {
+    __shared__ __align__(16) T sm[kThreads * 18];
+    const int mu = blockIdx.y, s0 = blockIdx.x * kThreads;
+    const M3<T> m = load_link<T, NC>(U, g.P, mu, sidx(g, site_of_lex(g, s0 + threadIdx.x)));
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
-        q[2 * k] = double(m.re[k]);
-        q[2 * k + 1] = double(m.im[k]);
+        T *q = sm + 18 * threadIdx.x + 2 * k;
+        if constexpr (sizeof(T) == 4) *reinterpret_cast<float2 *>(q) = make_float2(m.re[k], m.im[k]);
+        else *reinterpret_cast<double2 *>(q) = make_double2(m.re[k], m.im[k]);
     }
+    __syncthreads();
+    double *o = out + ((long long)mu * g.V + s0) * 18;
+#pragma unroll
+    for (int k = 0; k < 18; ++k) o[k * kThreads + threadIdx.x] = double(sm[k * kThreads + threadIdx.x]);
 }
 
 __global__ void k_read_labels(Geo g, const int8_t *__restrict__ ref, int8_t *out) {
@@ -135,63 +154,90 @@ __global__ void k_current_labels(Geo g, const T *__restrict__ U, int8_t *out) {
 // + n_nu(x-nu+mu)] so that sigma = m 2 pi / 18; delta = omega (sigma - lambda)
 // = omega pi (m - 6n) / 9.  Pair p = SplitMix64(seed, mu V + s) mod 3 picks
 // (j,k) = (0,1), (1,2), (2,0): phase j gets lambda + delta, phase k lambda - delta.
-// The phases take few values: pi (2n/3 + s omega k/9) with n in {-1, 0, 1},
-// k = m - 6n in [-24, 24], s = +-1 (k = 0 is the untouched phase 2n/3).  Each
-// block evaluates them once into shared memory with the same FP64 expressions
-// as the per-link form, so the links are bit-identical to it; values outside
-// the table (labels outside {-1, 0, 1}, only from device input) are evaluated
-// directly.
-constexpr int kCtabK = 24, kCtabN = 3 * (2 * kCtabK + 1) * 2;
+// The phases take few values: pi (2n/3 + omega k/9) with n in {-1, 0, 1} and
+// k = +-(m - 6n) in [-24, 24] (k = 0 is the untouched phase 2n/3).
+// k_centrifuge_table evaluates them once, with the same FP64 expressions as the
+// per-link form, so the links are bit-identical to it; values outside the table
+// (labels outside {-1, 0, 1}, only from device input) are evaluated directly.
+// The table is a kernel of its own: one warp per SM computes 32 entries in a
+// microsecond or two, where a table per block kept every SM's FP64 pipe busy for
+// ~10 us a block (0.16 of the 0.53 ms that the single kernel took at 32^3x64).
+constexpr int kCtabK = 24, kCtabN = 3 * (2 * kCtabK + 1);
 
-__device__ __forceinline__ double centrifuge_phase(double omega, int n, int k, bool neg) {
+__device__ __forceinline__ double2 centrifuge_phase(double omega, int n, int k) {
     const double delta = omega * (double)k / 9.0;   // in units of pi
-    const double ph = 2.0 * n / 3.0;
-    return neg ? ph - delta : ph + delta;
+    double2 v;
+    sincospi(2.0 * n / 3.0 + delta, &v.y, &v.x);
+    return v;
 }
 
+__global__ void k_centrifuge_table(double omega, double2 *tab) {   // (cos, sin) at (n + 1)(2K + 1) + k + K
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e < kCtabN) tab[e] = centrifuge_phase(omega, e / (2 * kCtabK + 1) - 1, e % (2 * kCtabK + 1) - kCtabK);
+}
+
+// One thread per site, its four links: 44 label reads at 21 positions, where a
+// thread per link read 19 labels at 13 positions four times over.  At 32^3x64
+// the links written (604 MB) take 0.09 ms at the copy rate.
 template <class T, int NC>
 __global__ void __launch_bounds__(kThreads) k_centrifuge(Geo g, const int8_t *__restrict__ ref, double omega,
-                                                          uint64_t seed, T *U) {
-    __shared__ double2 tab[kCtabN];   // (cos, sin) at ((n + 1)(2K + 1) + k + K) * 2 + neg
+                                                          uint64_t seed, T *U, const double2 *__restrict__ gtab) {
+    using T2 = typename std::conditional<sizeof(T) == 4, float2, double2>::type;
+    __shared__ T2 tab[kCtabN];
     for (int e = threadIdx.x; e < kCtabN; e += blockDim.x) {
-        const int q = e >> 1;
-        double sn, cs;
-        sincospi(centrifuge_phase(omega, q / (2 * kCtabK + 1) - 1, q % (2 * kCtabK + 1) - kCtabK, e & 1), &sn, &cs);
-        tab[e] = make_double2(cs, sn);
+        const double2 v = gtab[e];
+        tab[e].x = T(v.x);
+        tab[e].y = T(v.y);
     }
     __syncthreads();
-    for (long long l = (long long)blockIdx.x * blockDim.x + threadIdx.x; l < 4ll * g.V;
-         l += (long long)gridDim.x * blockDim.x) {
-        int mu = (int)(l / g.V), s = (int)(l % g.V);
-        Pt x = site_of_lex(g, s);
-        auto lab = [&](int d, const Pt &p) { return (int)ref[(long long)d * g.P + sidx(g, p)]; };
-        int m = 0;
+    for (int d = blockIdx.x * blockDim.x + threadIdx.x; d < g.V; d += gridDim.x * blockDim.x) {
+        const Pt x = site_of_index(g, d);
+        const int i = sidx(g, x), s = lexidx(g, x);
+        int dp[4], dm[4];
 #pragma unroll
-        for (int j = 1; j < 4; ++j) {
-            int nu = (mu + j) & 3;
-            Pt xpn = mv(g, x, nu, 1), xpm = mv(g, x, mu, 1), xmn = mv(g, x, nu, -1);
-            Pt xmnpm = mv(g, xmn, mu, 1);
-            m += lab(nu, x) + lab(mu, xpn) - lab(nu, xpm) - lab(nu, xmn) + lab(mu, xmn) + lab(nu, xmnpm);
+        for (int a = 0; a < 4; ++a) {
+            dp[a] = shift_delta(g, x, a, 1);
+            dm[a] = shift_delta(g, x, a, -1);
         }
-        const int n = lab(mu, x), k = m - 6 * n;
-        int pair = (int)(splitmix64(seed, (uint64_t)mu * (uint64_t)g.V + (uint64_t)s) % 3ull);
-        int jj = pair, kk = (pair + 1) % 3;
-        M3<T> z;
-        m3_zero(z);
+        const int8_t *lab[4] = {ref + i, ref + g.P + i, ref + 2 * g.P + i, ref + 3 * g.P + i};
+        int n[4], m[4];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const int kc = c == jj ? k : c == kk ? k : 0;
-            const bool neg = c == kk;
-            double2 v;
-            if (n >= -1 && n <= 1 && kc >= -kCtabK && kc <= kCtabK) {
-                v = tab[((n + 1) * (2 * kCtabK + 1) + kc + kCtabK) * 2 + neg];
-            } else {
-                sincospi(centrifuge_phase(omega, n, kc, neg), &v.y, &v.x);
+        for (int mu = 0; mu < 4; ++mu) {
+            n[mu] = lab[mu][0];
+            m[mu] = 0;
+        }
+#pragma unroll
+        for (int mu = 0; mu < 4; ++mu)
+#pragma unroll
+            for (int j = 1; j < 4; ++j) {
+                const int nu = (mu + j) & 3;
+                m[mu] += n[nu] + (int)lab[mu][dp[nu]] - (int)lab[nu][dp[mu]] - (int)lab[nu][dm[nu]] +
+                         (int)lab[mu][dm[nu]] + (int)lab[nu][dm[nu] + dp[mu]];
             }
-            z.re[4 * c] = T(v.x);
-            z.im[4 * c] = T(v.y);
+#pragma unroll
+        for (int mu = 0; mu < 4; ++mu) {
+            const int k = m[mu] - 6 * n[mu];
+            const uint64_t z64 = splitmix64(seed, (uint64_t)mu * (uint64_t)g.V + (uint64_t)s);
+            // z64 mod 3, with 2^32 = 1 (mod 3)
+            const int jj = (int)(((uint32_t)(z64 >> 32) % 3u + (uint32_t)z64 % 3u) % 3u), kk = jj == 2 ? 0 : jj + 1;
+            const bool in_tab = n[mu] >= -1 && n[mu] <= 1 && k >= -kCtabK && k <= kCtabK;
+            M3<T> z;
+            m3_zero(z);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const int kc = c == jj ? k : c == kk ? -k : 0;
+                if (in_tab) {
+                    const T2 v = tab[(n[mu] + 1) * (2 * kCtabK + 1) + kc + kCtabK];
+                    z.re[4 * c] = v.x;
+                    z.im[4 * c] = v.y;
+                } else {
+                    const double2 v = centrifuge_phase(omega, n[mu], kc);
+                    z.re[4 * c] = T(v.x);
+                    z.im[4 * c] = T(v.y);
+                }
+            }
+            store_link<T, NC>(U, g.P, mu, i, z);
         }
-        store_link<T, NC>(U, g.P, mu, sidx(g, x), z);
     }
 }
 
@@ -634,14 +680,12 @@ __global__ void k_haar(Geo g, uint64_t seed, T *U) {
 // lexicographic site order) as 18 reals per site in the link layout, then
 // U_mu(x) -> G(x) U_mu(x) G^dag(x + mu) for every link.
 template <class T>
-__global__ void k_store_gauge(Geo g, const double *__restrict__ Glex, T *Gs) {
-    int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= g.V) return;
-    const double *q = Glex + 18ll * s;
-    M3<T> m;
-#pragma unroll
-    for (int k = 0; k < 9; ++k) { m.re[k] = T(q[2 * k]); m.im[k] = T(q[2 * k + 1]); }
-    store_link<T, 18>(Gs, g.P, 0, sidx(g, site_of_lex(g, s)), m);
+__global__ void __launch_bounds__(kThreads) k_store_gauge(Geo g, const double *__restrict__ Glex, T *Gs) {
+    __shared__ __align__(16) double sm[kThreads * 18];
+    const int s0 = blockIdx.x * kThreads;
+    double tr, ti;
+    const M3<T> m = staged_matrix<T>(Glex + 18ll * s0, sm, tr, ti);
+    store_link<T, 18>(Gs, g.P, 0, sidx(g, site_of_lex(g, s0 + threadIdx.x)), m);
 }
 
 template <class T, int NC>
@@ -707,7 +751,7 @@ cudaError_t launch_load_labels(int prec, int nc, const Geo &g, const int8_t *lab
 
 cudaError_t launch_load_links(int prec, int nc, const Geo &g, const double *in, void *U, int8_t *ref,
                               cudaStream_t st) {
-    int b = nblocks(4ll * g.V);
+    const dim3 b(nblocks(g.V), 4);
     if (prec == 0) k_load_links<double, 18><<<b, kThreads, 0, st>>>(g, in, (double *)U, ref);
     else if (nc == 18) k_load_links<float, 18><<<b, kThreads, 0, st>>>(g, in, (float *)U, ref);
     else k_load_links<float, 12><<<b, kThreads, 0, st>>>(g, in, (float *)U, ref);
@@ -716,7 +760,7 @@ cudaError_t launch_load_links(int prec, int nc, const Geo &g, const double *in, 
 }
 
 cudaError_t launch_read_links(int prec, int nc, const Geo &g, const void *U, double *out, cudaStream_t st) {
-    int b = nblocks(4ll * g.V);
+    const dim3 b(nblocks(g.V), 4);
     if (prec == 0) k_read_links<double, 18><<<b, kThreads, 0, st>>>(g, (const double *)U, out);
     else if (nc == 18) k_read_links<float, 18><<<b, kThreads, 0, st>>>(g, (const float *)U, out);
     else k_read_links<float, 12><<<b, kThreads, 0, st>>>(g, (const float *)U, out);
@@ -756,12 +800,14 @@ cudaError_t launch_current_labels(int prec, int nc, const Geo &g, const void *U,
 }
 
 cudaError_t launch_centrifuge(int prec, int nc, const Geo &g, const int8_t *ref, double omega, uint64_t seed,
-                              void *U, cudaStream_t st) {
-    int b = std::min(nblocks(4ll * g.V), kTableGrid);
-    if (prec == 0) k_centrifuge<double, 18><<<b, kThreads, 0, st>>>(g, ref, omega, seed, (double *)U);
-    else if (nc == 18) k_centrifuge<float, 18><<<b, kThreads, 0, st>>>(g, ref, omega, seed, (float *)U);
-    else k_centrifuge<float, 12><<<b, kThreads, 0, st>>>(g, ref, omega, seed, (float *)U);
-    count_launches(1);
+                              void *U, double *table, cudaStream_t st) {
+    const int b = std::min(nblocks(g.V), kTableGrid);
+    double2 *tab = reinterpret_cast<double2 *>(table);
+    k_centrifuge_table<<<(kCtabN + 31) / 32, 32, 0, st>>>(omega, tab);
+    if (prec == 0) k_centrifuge<double, 18><<<b, kThreads, 0, st>>>(g, ref, omega, seed, (double *)U, tab);
+    else if (nc == 18) k_centrifuge<float, 18><<<b, kThreads, 0, st>>>(g, ref, omega, seed, (float *)U, tab);
+    else k_centrifuge<float, 12><<<b, kThreads, 0, st>>>(g, ref, omega, seed, (float *)U, tab);
+    count_launches(2);
     return cudaGetLastError();
 }
 
