@@ -125,7 +125,7 @@ uint64_t vs::field_footprint(const int32_t dims[4], int32_t precision, int32_t s
     const long long P = make_geo(dims).P;   // plane stride, with the layout's unused positions
     int nc = storage == VS_LINK12 ? 12 : 18;
     uint64_t links = (uint64_t)4 * nc * P * (precision == VS_FP64 ? 8 : 4);
-    return links + 8ull * P + 1216 * 8 + 4096 + (precision == VS_FP32 ? kDeferCap * sizeof(int) : 0);
+    return links + 8ull * P + kPartials * 8 + 256 + (precision == VS_FP32 ? kDeferCap * sizeof(int) : 0);
 }
 
 extern "C" vs_status vs_field_create(vs_ctx *c, const int32_t dims[4], int32_t precision, int32_t storage,
@@ -157,14 +157,14 @@ extern "C" vs_status vs_field_create(vs_ctx *c, const int32_t dims[4], int32_t p
     f->U = dev_alloc(c, field_bytes(f));
     f->ref = (int8_t *)dev_alloc(c, 4 * (size_t)f->g.P);
     f->cur = (int8_t *)dev_alloc(c, 4 * (size_t)f->g.P);
-    f->partials = (double *)dev_alloc(c, 1216 * sizeof(double) + 4096);
+    f->partials = (double *)dev_alloc(c, kPartials * sizeof(double) + 256);
     if (precision == VS_FP32) f->defer_idx = (int *)dev_alloc(c, kDeferCap * sizeof(int));
     if (!f->U || !f->ref || !f->cur || !f->partials || (precision == VS_FP32 && !f->defer_idx)) {
         vs_field_destroy(f);
         return fail(VS_ENOMEM, "vs_field_create: device allocation of %zu bytes failed", field_bytes(f));
     }
-    // scalars live after the partials: [1216 doubles][result double][counters...]
-    f->d_result = f->partials + 1216;
+    // scalars live after the partials: [kPartials doubles][result double][counters...], 18 words
+    f->d_result = f->partials + kPartials;
     f->d_counts = (unsigned long long *)(f->d_result + 1);      // 8 slots
     f->d_sweep = f->d_counts + 8;                               // kSweepSlots slots
     f->defer_n = (unsigned *)(f->d_sweep + kSweepSlots);        // 2 counters
@@ -979,8 +979,7 @@ extern "C" vs_status vs_observables(vs_field *f, vs_observables_out *out, double
         dSR = SR_site ? sc + V : nullptr;
         dq = q_site ? sc + 2 * V : nullptr;
     }
-    // 3 x 400 partials fit in the 1216 + 512 doubles after f->partials; results after them
-    double *res = f->partials + 1200;
+    double *res = f->partials + kPartials - 8;
     CK(launch_observables(f->prec == VS_FP32, f->nc, f->g, f->U, f->partials, res, dS, dSR, dq, f->stream));
     double h[3];
     CK(cudaMemcpyAsync(h, res, sizeof h, cudaMemcpyDeviceToHost, f->stream));
@@ -1011,8 +1010,7 @@ extern "C" vs_status vs_correlation(vs_field *f, const double *a, const double *
         da = sc;
         db = sc + V;
     }
-    // 3 x 400 partials, then the result and the three sums
-    double *res = f->partials + 1200;
+    double *res = f->partials + kPartials - 8;   // the result and the three sums
     CK(launch_correlation(da, db, (long long)V, f->partials, res, f->stream));
     double h[4];
     CK(cudaMemcpyAsync(h, res, sizeof h, cudaMemcpyDeviceToHost, f->stream));

@@ -39,7 +39,7 @@ struct vs_field {
     bool loaded = false;
     void *U = nullptr;
     int8_t *ref = nullptr;
-    int8_t *cur = nullptr;
+    int8_t *cur = nullptr;           // vortex check: label differences mod 3
     void *G = nullptr;              // random gauge transformation (18 reals per site)
     bool gauge_on = false;          // links are in the random gauge G
     double *partials = nullptr;

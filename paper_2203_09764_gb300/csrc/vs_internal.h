@@ -133,11 +133,14 @@ cudaError_t launch_current_labels(int prec, int nc, const Geo &g, const void *U,
 // table: scratch of at least 294 doubles, 16-byte aligned
 cudaError_t launch_centrifuge(int prec, int nc, const Geo &g, const int8_t *ref, double omega,
                               uint64_t seed, void *U, double *table, cudaStream_t st);
-// mean over sites of S(x)/beta into *out (device double); partials: n_part doubles
-int action_partials(const Geo &g);
+// Doubles of a field's scratch for block sums (the last 8 hold the results of
+// vs_observables and vs_correlation), the blocks of the action kernel, and those of
+// the observables and correlation kernels (three sums each).
+constexpr int kPartials = 1696, kActionBlocks = 1216, kObsBlocks = (kPartials - 8) / 3;
+// mean over sites of S(x)/beta into *out (device double); partials: kActionBlocks doubles
 cudaError_t launch_action(int prec, int nc, const Geo &g, const void *U, double *partials,
                           double *out, cudaStream_t st);
-// <S>/beta, <S_R>/beta and Q into out[0..2]; partials: 3 x 400 doubles;
+// <S>/beta, <S_R>/beta and Q into out[0..2]; partials: 3 x kObsBlocks doubles;
 // optional per-site densities in lexicographic order
 cudaError_t launch_observables(int prec, int nc, const Geo &g, const void *U, double *partials, double *out,
                                double *S_site, double *SR_site, double *q_site, cudaStream_t st);
@@ -146,9 +149,10 @@ cudaError_t launch_observables(int prec, int nc, const Geo &g, const void *U, do
 cudaError_t launch_correlation(const double *a, const double *b, long long n, double *partials, double *out,
                                cudaStream_t st);
 // counts[0] label diffs, counts[1] charge diffs, counts[2] near-boundary links;
-// margin_bits: min angular margin as the bit pattern of a non-negative double
+// margin_bits: min angular margin as the bit pattern of a non-negative double;
+// dz: scratch of one byte per link position (label differences mod 3)
 cudaError_t launch_vortex(int prec, int nc, const Geo &g, const void *U, const int8_t *ref,
-                          int8_t *cur, unsigned long long *counts,
+                          int8_t *dz, unsigned long long *counts,
                           unsigned long long *margin_bits, cudaStream_t st, const void *G = nullptr);
 // load the vortex-check kernels now (a first launch would, with lazy loading)
 cudaError_t preload_vortex_kernels();

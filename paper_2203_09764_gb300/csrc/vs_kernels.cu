@@ -137,13 +137,13 @@ __global__ void k_store_ref(Geo g, const int8_t *__restrict__ lab, int8_t *ref) 
     ref[(long long)mu * g.P + sidx(g, site_of_lex(g, s))] = lab[l];
 }
 
+// One thread per link, one direction per grid row; a label needs the link's
+// diagonal, so only the chunks that hold it are loaded (40 of 72 bytes).
 template <class T, int NC>
-__global__ void k_current_labels(Geo g, const T *__restrict__ U, int8_t *out) {
-    long long l = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (l >= 4ll * g.V) return;
-    int mu = (int)(l / g.V), s = (int)(l % g.V);
-    M3<T> m = load_link<T, NC>(U, g.P, mu, sidx(g, site_of_lex(g, s)));
-    out[l] = (int8_t)z3_label<T>(m.re[0] + m.re[4] + m.re[8], m.im[0] + m.im[4] + m.im[8]);
+__global__ void __launch_bounds__(kThreads) k_current_labels(Geo g, const T *__restrict__ U, int8_t *out) {
+    const int mu = blockIdx.y, s = blockIdx.x * kThreads + threadIdx.x;
+    const M3<T> m = load_link<T, NC>(U, g.P, mu, sidx(g, site_of_lex(g, s)));
+    out[(long long)mu * g.V + s] = (int8_t)z3_label<T>(m.re[0] + m.re[4] + m.re[8], m.im[0] + m.im[4] + m.im[8]);
 }
 
 // ---------------------------------------------------------------------------
@@ -265,31 +265,63 @@ __device__ __forceinline__ double block_sum(double v) {
     return v;
 }
 
+// Sum of a few values of the storage precision as FP64 would give it.  FP32: an
+// error-free transformation (Knuth's TwoSum), so that a site costs two
+// conversions instead of an FP64 operation per value (GB300's FP64 pipe takes a
+// warp instruction every 16 cycles; 18 per site were 60 us of k_action at
+// 32^3x64).
+template <class T> struct ShortSum;
+template <> struct ShortSum<double> {
+    double v = 0;
+    __device__ __forceinline__ void add(double x) { v += x; }
+    __device__ __forceinline__ double value() const { return v; }
+};
+template <> struct ShortSum<float> {
+    float hi = 0, lo = 0;
+    __device__ __forceinline__ void add(float x) {
+        const float s = hi + x, b = s - hi;
+        lo += (hi - (s - b)) + (x - b);
+        hi = s;
+    }
+    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+};
+
+// Blocks of the measurement kernels: kMeasThreads threads, one wave of resident
+// blocks, grid-stride over the sites.  Both are bound by the latency and the
+// L1/L2 rate of their link loads (1.5 and 6 KB per site), so what counts is warps
+// per SM: 16 for the action (120 registers), 12 for the observables (168), where
+// blocks of 256 threads left 8.  Per call at 32^3x64, FP32: action 395 -> 213 us
+// (five blocks per SM spill: 295), observables 1174 -> 842 us (four: 958).
+constexpr int kMeasThreads = 128, kActionPerSM = 4, kObsPerSM = 3;
+
 template <class T, int NC>
-__global__ void __launch_bounds__(kThreads) k_action(Geo g, const T *__restrict__ U, double *partials) {
+__global__ void __launch_bounds__(kMeasThreads, sizeof(T) == 4 ? kActionPerSM : 2)
+    k_action(Geo g, const T *__restrict__ U, double *partials) {
     double acc = 0;
     for (int d = blockIdx.x * blockDim.x + threadIdx.x; d < g.V; d += gridDim.x * blockDim.x) {
         const Pt x = site_of_index(g, d);
         const int i = sidx(g, x);
-#pragma unroll
+        ShortSum<T> tr;
+#pragma unroll 1
         for (int mu = 0; mu < 3; ++mu) {
-            M3<T> Umu = load_link<T, NC>(U, g.P, mu, i);
-            Pt xm = mv(g, x, mu, 1);
-#pragma unroll
+            const M3<T> Umu = load_link<T, NC>(U, g.P, mu, i);
+            const int im = i + shift_delta(g, x, mu, 1);
+#pragma unroll 1
             for (int nu = mu + 1; nu < 4; ++nu) {
-                Pt xn = mv(g, x, nu, 1);
                 // P = (U_mu(x) U_nu(x+mu)) (U_nu(x) U_mu(x+nu))^dag
-                M3<T> X = m3_mul(Umu, load_link<T, NC>(U, g.P, nu, sidx(g, xm)));
-                M3<T> Y = m3_mul(load_link<T, NC>(U, g.P, nu, i), load_link<T, NC>(U, g.P, mu, sidx(g, xn)));
+                const M3<T> X = m3_mul(Umu, load_link<T, NC>(U, g.P, nu, im));
+                const M3<T> Y = m3_mul(load_link<T, NC>(U, g.P, nu, i),
+                                       load_link<T, NC>(U, g.P, mu, i + shift_delta(g, x, nu, 1)));
                 // Re Tr(X Y^dag) in the storage precision: the FP32 products
                 // already carry FP32 rounding, and an FP64 dot (18 conversions
                 // and FMAs on the slow FP64 pipe) made this kernel FP64-bound
                 T re = T(0);
 #pragma unroll
                 for (int k = 0; k < 9; ++k) re = fma(X.re[k], Y.re[k], fma(X.im[k], Y.im[k], re));
-                acc += 3.0 - (double)re;
+                tr.add(re);
             }
         }
+        acc += 18.0 - tr.value();
     }
     double b = block_sum(acc);
     if (threadIdx.x == 0) partials[blockIdx.x] = b;
@@ -304,82 +336,104 @@ __global__ void __launch_bounds__(kThreads) k_action(Geo g, const T *__restrict_
 // (the eps-sum of Eq. 1LTopQ collapsed to its three pairings x 8 / (32 pi^2)).
 // ---------------------------------------------------------------------------
 
-template <class T, int NC>
-__device__ __forceinline__ M3<T> clover_F(const Geo &g, const T *__restrict__ U, const Pt &x, int i, int mu,
-                                          int nu, T &plaq_retr) {
-    const Pt xpm = mv(g, x, mu, 1), xpn = mv(g, x, nu, 1), xmm = mv(g, x, mu, -1), xmn = mv(g, x, nu, -1);
-    const int ipm = sidx(g, xpm), ipn = sidx(g, xpn), imm = sidx(g, xmm), imn = sidx(g, xmn);
-    const int ipnmm = sidx(g, mv(g, xpn, mu, -1)), immmn = sidx(g, mv(g, xmm, nu, -1));
-    const int imnpm = sidx(g, mv(g, xmn, mu, 1));
-    M3<T> C, L;
-    // leaf 1: +mu +nu -mu -nu
-    L = m3_mul(load_link<T, NC>(U, g.P, mu, i), load_link<T, NC>(U, g.P, nu, ipm));
-    L = m3_mul_nd(L, load_link<T, NC>(U, g.P, mu, ipn));
-    L = m3_mul_nd(L, load_link<T, NC>(U, g.P, nu, i));
-    plaq_retr = L.re[0] + L.re[4] + L.re[8];
-    C = L;
-    // leaf 2: +nu -mu -nu +mu
-    L = m3_mul_nd(load_link<T, NC>(U, g.P, nu, i), load_link<T, NC>(U, g.P, mu, ipnmm));
-    L = m3_mul_nd(L, load_link<T, NC>(U, g.P, nu, imm));
-    m3_madd(C, L, load_link<T, NC>(U, g.P, mu, imm));
-    // leaf 3: -mu -nu +mu +nu
-    L = m3_mul_dn(load_link<T, NC>(U, g.P, mu, imm), m3_dag(load_link<T, NC>(U, g.P, nu, immmn)));
-    L = m3_mul(L, load_link<T, NC>(U, g.P, mu, immmn));
-    m3_madd(C, L, load_link<T, NC>(U, g.P, nu, imn));
-    // leaf 4: -nu +mu +nu -mu
-    L = m3_mul_dn(load_link<T, NC>(U, g.P, nu, imn), load_link<T, NC>(U, g.P, mu, imn));
-    L = m3_mul(L, load_link<T, NC>(U, g.P, nu, imnpm));
-    L = m3_mul_nd(L, load_link<T, NC>(U, g.P, mu, i));
-    for (int k = 0; k < 9; ++k) { C.re[k] += L.re[k]; C.im[k] += L.im[k]; }
-    // F = (C - C^dag) / (2i) / 4, traceless
-    M3<T> F;
+// D(y) = B(y) - B'(y) for the link U_mu(y) and the plane (mu, nu), the two paths
+// that close it into the leaf above and (its conjugate) the leaf below:
+//   B  = U_nu(y+mu) U_mu^dag(y+nu) U_nu^dag(y)
+//   B' = U_nu^dag(y+mu-nu) U_mu^dag(y-nu) U_nu(y-nu)
+// iy: position of y; dm: shift to y+mu; dn, db: shifts to y+nu and y-nu.
+// retr: Re Tr(W B) for the plaquette W = U_mu(y), if wanted.
+template <class T, int NC, bool TRACE>
+__device__ __forceinline__ M3<T> clover_arms(const Geo &g, const T *__restrict__ U, int mu, int nu, int iy, int dm,
+                                             int dn, int db, const M3<T> *W, T &retr) {
+    M3<T> D = m3_mul_nd(m3_mul_nd(load_link<T, NC>(U, g.P, nu, iy + dm), load_link<T, NC>(U, g.P, mu, iy + dn)),
+                        load_link<T, NC>(U, g.P, nu, iy));
+    if constexpr (TRACE) {
+        T re = T(0);
 #pragma unroll
-    for (int j = 0; j < 3; ++j)
+        for (int j = 0; j < 3; ++j)
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const T dr = C.re[3 * j + k] - C.re[3 * k + j], di = C.im[3 * j + k] + C.im[3 * k + j];
-            F.re[3 * j + k] = T(0.125) * di;
-            F.im[3 * j + k] = -T(0.125) * dr;
-        }
-    const T tr = (F.re[0] + F.re[4] + F.re[8]) / T(3);
-    F.re[0] -= tr;
-    F.re[4] -= tr;
-    F.re[8] -= tr;
-    return F;
+            for (int k = 0; k < 3; ++k)
+                re = fma(W->re[3 * j + k], D.re[3 * k + j], fma(-W->im[3 * j + k], D.im[3 * k + j], re));
+        retr = re;
+    }
+    // U_nu^dag U_mu^dag = (U_mu U_nu)^dag
+    M3<T> E = m3_dag(m3_mul(load_link<T, NC>(U, g.P, mu, iy + db), load_link<T, NC>(U, g.P, nu, iy + dm + db)));
+#pragma unroll
+    for (int k = 0; k < 9; ++k) { E.re[k] = -E.re[k]; E.im[k] = -E.im[k]; }
+    m3_madd(D, E, load_link<T, NC>(U, g.P, nu, iy + db));
+    return D;
 }
 
-// Tr(A B) for Hermitian A, B: sum_jk A_jk conj(B_jk), real, in the storage
+// F_munu(x) by its diagonal h[0..2] and upper entries h[3..8] (re, im): the four
+// leaves pair up as U_mu(x) D(x) and D(x-mu) U_mu(x-mu), each minus its adjoint
+// (10 products for a plane instead of 12 leaf by leaf).
+template <class T, int NC>
+__device__ __forceinline__ void clover_F(const Geo &g, const T *__restrict__ U, const Pt &x, int i, int mu, int nu,
+                                         T h[9], T &plaq_retr) {
+    const int pm = shift_delta(g, x, mu, 1), mm = shift_delta(g, x, mu, -1);
+    const int pn = shift_delta(g, x, nu, 1), mn = shift_delta(g, x, nu, -1);
+    M3<T> C;
+    {
+        const M3<T> Um = load_link<T, NC>(U, g.P, mu, i);
+        const M3<T> D = clover_arms<T, NC, true>(g, U, mu, nu, i, pm, pn, mn, &Um, plaq_retr);
+        C = m3_mul(Um, D);
+    }
+    {
+        T none;
+        const M3<T> D = clover_arms<T, NC, false>(g, U, mu, nu, i + mm, -mm, pn, mn, nullptr, none);
+        m3_madd(C, D, load_link<T, NC>(U, g.P, mu, i + mm));
+    }
+    // F = (C - C^dag) / (2i) / 4, traceless
+    const T tr = (C.im[0] + C.im[4] + C.im[8]) / T(3);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) h[j] = T(0.25) * (C.im[4 * j] - tr);
+    h[3] = T(0.125) * (C.im[1] + C.im[3]); h[4] = T(0.125) * (C.re[3] - C.re[1]);
+    h[5] = T(0.125) * (C.im[2] + C.im[6]); h[6] = T(0.125) * (C.re[6] - C.re[2]);
+    h[7] = T(0.125) * (C.im[5] + C.im[7]); h[8] = T(0.125) * (C.re[7] - C.re[5]);
+}
+
+// Tr(A B) for Hermitian A, B by diagonal and upper entries, in the storage
 // precision (its FP32 inputs already carry FP32 rounding; an FP64 dot made the
 // kernel FP64-bound); the sums over sites run in FP64.
 template <class T>
-__device__ __forceinline__ T tr_herm(const M3<T> &A, const M3<T> &B) {
-    T s = T(0);
+__device__ __forceinline__ T tr_herm(const T a[9], const T b[9]) {
+    T s = T(0), o = T(0);
 #pragma unroll
-    for (int k = 0; k < 9; ++k) s += A.re[k] * B.re[k] + A.im[k] * B.im[k];
-    return s;
+    for (int k = 0; k < 3; ++k) s = fma(a[k], b[k], s);
+#pragma unroll
+    for (int k = 3; k < 9; ++k) o = fma(a[k], b[k], o);
+    return fma(T(2), o, s);
 }
 
 template <class T, int NC>
-__global__ void __launch_bounds__(kThreads) k_observables(Geo g, const T *__restrict__ U, double *partials,
-                                                           double *S_site, double *SR_site, double *q_site) {
+__global__ void __launch_bounds__(kMeasThreads, sizeof(T) == 4 ? kObsPerSM : 2)
+    k_observables(Geo g, const T *__restrict__ U, double *partials, double *S_site, double *SR_site,
+                  double *q_site) {
     double aS = 0, aSR = 0, aQ = 0;
-    const int pairs[3][4] = {{0, 1, 2, 3}, {0, 2, 1, 3}, {0, 3, 1, 2}};
-    const double sgn[3] = {1.0, -1.0, 1.0};
     for (int d = blockIdx.x * blockDim.x + threadIdx.x; d < g.V; d += gridDim.x * blockDim.x) {
         const Pt x = site_of_index(g, d);
         const int i = sidx(g, x);
-        double s = 0, sr = 0, q = 0;
-        for (int pp = 0; pp < 3; ++pp) {
-            T r1, r2;
-            const M3<T> Fa = clover_F<T, NC>(g, U, x, i, pairs[pp][0], pairs[pp][1], r1);
-            const M3<T> Fb = clover_F<T, NC>(g, U, x, i, pairs[pp][2], pairs[pp][3], r2);
-            s += (3.0 - (double)r1) + (3.0 - (double)r2);
-            sr += (double)tr_herm(Fa, Fa) + (double)tr_herm(Fb, Fb);
-            q += sgn[pp] * (double)tr_herm(Fa, Fb);
+        ShortSum<T> ss, ssr, sq;
+        // the pairings (01, 23), (02, 13), (03, 12) with signs +, -, +, one plane
+        // at a time so that the clover code exists once
+        T fa[9];
+#pragma unroll 1
+        for (int p = 0; p < 6; ++p) {
+            const int j = (p >> 1) + 1;                       // the partner of direction 0
+            const int mu = p & 1 ? (j == 1 ? 2 : 1) : 0, nu = p & 1 ? (j == 3 ? 2 : 3) : j;
+            T f[9], re;
+            clover_F<T, NC>(g, U, x, i, mu, nu, f, re);
+            ss.add(re);
+            ssr.add(tr_herm(f, f));
+            if (p & 1) {
+                const T qq = tr_herm(fa, f);
+                sq.add(j == 2 ? -qq : qq);
+            }
+#pragma unroll
+            for (int k = 0; k < 9; ++k) fa[k] = f[k];
         }
-        s *= 2.0 / 72.0;
-        sr /= 72.0;
-        q /= 4.0 * 9.869604401089358;
+        const double s = (18.0 - ss.value()) * (2.0 / 72.0), sr = ssr.value() / 72.0,
+                     q = sq.value() / (4.0 * 9.869604401089358);
         const int lx = lexidx(g, x);
         if (S_site) S_site[lx] = s;
         if (SR_site) SR_site[lx] = sr;
@@ -462,71 +516,84 @@ __global__ void k_correlation_finish(const double *__restrict__ partials, int nb
 // Vortex check
 // ---------------------------------------------------------------------------
 
-__device__ __forceinline__ void count_warp(unsigned long long *ctr, bool pred) {
-    unsigned b = __ballot_sync(0xffffffffu, pred);
-    if ((threadIdx.x & 31) == 0 && b) atomicAdd(ctr, (unsigned long long)__popc(b));
-}
-
-template <class T, int NC>
-__global__ void k_vortex_links(Geo g, const T *__restrict__ U, const int8_t *__restrict__ ref,
-                               int8_t *cur, unsigned long long *counts, unsigned long long *mbits,
-                               const T *__restrict__ G) {
-    long long l = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    bool diff = false, near = false;
+// One thread per site, its four links.  dz: per link (current - reference label)
+// mod 3 in {0, 1, 2}, all that the charges need.  A warp's smallest margin goes
+// to the global minimum only if it is below the value read there: with one
+// 64-bit atomicMin per warp of links, all to one address, this kernel took
+// 0.21 ms at 32^3x64 whatever it read.  Without a gauge only the diagonals are
+// loaded (40 of 72 bytes per FP32 link, 335 MB: 0.05 ms at the copy rate).
+template <class T, int NC, bool GAUGE>
+__global__ void __launch_bounds__(kThreads) k_vortex_links(Geo g, const T *__restrict__ U,
+                                                            const int8_t *__restrict__ ref, int8_t *dz,
+                                                            unsigned long long *counts, unsigned long long *mbits,
+                                                            const T *__restrict__ G) {
+    const Pt x = site_of_index(g, blockIdx.x * kThreads + threadIdx.x);   // V is a multiple of kThreads
+    const int i = sidx(g, x);
+    int n_diff = 0, n_near = 0;
     double margin = 1e300;
-    if (l < 4ll * g.V) {
-        const int mu = (int)(l / g.V);
-        const Pt x = site_of_index(g, (int)(l % g.V));
-        const int i = sidx(g, x);
-        M3<T> m = load_link<T, NC>(U, g.P, mu, i);
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) {
+        const M3<T> m = load_link<T, NC>(U, g.P, mu, i);
         T a, b;
-        vp_trace<T>(G, g.P, i, G ? sidx(g, mv(g, x, mu, 1)) : i, m, a, b);
-        int lab = z3_label<T>(a, b);
-        cur[(long long)mu * g.P + i] = (int8_t)lab;
-        diff = lab != ref[(long long)mu * g.P + i];
+        if constexpr (GAUGE) vp_trace<T>(G, g.P, i, i + shift_delta(g, x, mu, 1), m, a, b);
+        else vp_trace<T>((const T *)nullptr, g.P, i, i, m, a, b);
+        const int d = z3_label<T>(a, b) - (int)ref[(long long)mu * g.P + i];
+        dz[(long long)mu * g.P + i] = (int8_t)((d % 3 + 3) % 3);
+        n_diff += d != 0;
         // angular distance of arg Tr U from the nearest sector edge (+-pi/3,
         // pi), in the field's precision: an FP32 trace is itself rounded to
         // ~1e-7, and an FP64 atan2 per link made this kernel FP64-bound
+        double mg;
         if constexpr (sizeof(T) == 4) {
             const float argf = atan2f(b + 0.0f, a);
             const float pi3f = 1.04719755f;
-            margin = (double)fminf(fminf(fabsf(argf - pi3f), fabsf(argf + pi3f)), 3.14159265f - fabsf(argf));
+            mg = (double)fminf(fminf(fabsf(argf - pi3f), fabsf(argf + pi3f)), 3.14159265f - fabsf(argf));
         } else {
-            double arg = atan2((double)b + 0.0, (double)a);
+            const double arg = atan2((double)b + 0.0, (double)a);
             const double pi3 = 1.0471975511965976;
-            margin = fmin(fmin(fabs(arg - pi3), fabs(arg + pi3)), 3.141592653589793 - fabs(arg));
+            mg = fmin(fmin(fabs(arg - pi3), fabs(arg + pi3)), 3.141592653589793 - fabs(arg));
         }
-        near = margin < 1e-5;
+        n_near += mg < 1e-5;
+        margin = fmin(margin, mg);
     }
-    count_warp(&counts[0], diff);
-    count_warp(&counts[2], near);
+    if (__any_sync(0xffffffffu, n_diff | n_near)) {
+        n_diff = __reduce_add_sync(0xffffffffu, n_diff);
+        n_near = __reduce_add_sync(0xffffffffu, n_near);
+        if ((threadIdx.x & 31) == 0) {
+            if (n_diff) atomicAdd(&counts[0], (unsigned long long)n_diff);
+            if (n_near) atomicAdd(&counts[2], (unsigned long long)n_near);
+        }
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) margin = fmin(margin, __shfl_xor_sync(0xffffffffu, margin, o));
-    if ((threadIdx.x & 31) == 0 && margin < 1e300)
-        atomicMin(mbits, (unsigned long long)__double_as_longlong(margin));
-}
-
-// centre charge p = n_mu(x) + n_nu(x+mu) - n_mu(x+nu) - n_nu(x) mod 3 in {-1,0,1}
-__device__ __forceinline__ int charge(const Geo &g, const int8_t *lab, const Pt &x, int i, int mu, int nu) {
-    int p = lab[(long long)mu * g.P + i] + lab[(long long)nu * g.P + sidx(g, mv(g, x, mu, 1))]
-          - lab[(long long)mu * g.P + sidx(g, mv(g, x, nu, 1))] - lab[(long long)nu * g.P + i];
-    p = ((p % 3) + 3) % 3;
-    return p == 2 ? -1 : p;
-}
-
-__global__ void k_vortex_charges(Geo g, const int8_t *__restrict__ ref, const int8_t *__restrict__ cur,
-                                 unsigned long long *counts) {
-    const int dn = blockIdx.x * blockDim.x + threadIdx.x;
-    int nd = 0;
-    if (dn < g.V) {
-        const Pt x = site_of_index(g, dn);
-        const int i = sidx(g, x);
-        for (int mu = 0; mu < 4; ++mu)
-            for (int nu = mu + 1; nu < 4; ++nu)
-                nd += charge(g, cur, x, i, mu, nu) != charge(g, ref, x, i, mu, nu);
+    if ((threadIdx.x & 31) == 0 && margin < 1e300) {
+        const unsigned long long bits = (unsigned long long)__double_as_longlong(margin);
+        if (bits < *(volatile unsigned long long *)mbits) atomicMin(mbits, bits);
     }
+}
+
+// Plaquettes whose centre charge p = n_mu(x) + n_nu(x+mu) - n_mu(x+nu) - n_nu(x)
+// (mod 3) differs from the reference: those whose label differences dz do not
+// cancel mod 3.  Where no label differs (every check of a vortex-preserving run)
+// no charge can, and the kernel ends on the count that k_vortex_links left.
+__global__ void __launch_bounds__(kThreads) k_vortex_charges(Geo g, const int8_t *__restrict__ dz,
+                                                              unsigned long long *counts) {
+    if (counts[0] == 0) return;
+    const Pt x = site_of_index(g, blockIdx.x * kThreads + threadIdx.x);
+    const int i = sidx(g, x);
+    int here[4], nd = 0;
+    const int8_t *lab[4] = {dz + i, dz + g.P + i, dz + 2 * g.P + i, dz + 3 * g.P + i};
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) nd += __shfl_xor_sync(0xffffffffu, nd, o);
+    for (int mu = 0; mu < 4; ++mu) here[mu] = lab[mu][0];
+    int dp[4];
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) dp[mu] = shift_delta(g, x, mu, 1);
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu)
+#pragma unroll
+        for (int nu = mu + 1; nu < 4; ++nu)
+            nd += (here[mu] + (int)lab[nu][dp[mu]] - (int)lab[mu][dp[nu]] - here[nu] + 6) % 3 != 0;
+    nd = __reduce_add_sync(0xffffffffu, nd);
     if ((threadIdx.x & 31) == 0 && nd) atomicAdd(&counts[1], (unsigned long long)nd);
 }
 
@@ -791,7 +858,7 @@ cudaError_t launch_read_labels(const Geo &g, const int8_t *ref, int8_t *out, cud
 }
 
 cudaError_t launch_current_labels(int prec, int nc, const Geo &g, const void *U, int8_t *out, cudaStream_t st) {
-    int b = nblocks(4ll * g.V);
+    const dim3 b(nblocks(g.V), 4);
     if (prec == 0) k_current_labels<double, 18><<<b, kThreads, 0, st>>>(g, (const double *)U, out);
     else if (nc == 18) k_current_labels<float, 18><<<b, kThreads, 0, st>>>(g, (const float *)U, out);
     else k_current_labels<float, 12><<<b, kThreads, 0, st>>>(g, (const float *)U, out);
@@ -811,17 +878,27 @@ cudaError_t launch_centrifuge(int prec, int nc, const Geo &g, const int8_t *ref,
     return cudaGetLastError();
 }
 
-int action_partials(const Geo &g) {
-    int b = nblocks(g.V);
-    return b < 1216 ? b : 1216;
+// One wave of the resident blocks of a measurement kernel, at most `most` (its partials).
+template <class K>
+static int meas_blocks(K kernel, const Geo &g, int most) {
+    int dev = 0, n_sm = 0, per_sm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kMeasThreads, 0);
+    const int wave = std::max(1, n_sm * std::max(per_sm, 1));
+    return std::min(nblocks(g.V, kMeasThreads), std::min(wave, most));
 }
 
 cudaError_t launch_action(int prec, int nc, const Geo &g, const void *U, double *partials, double *out,
                           cudaStream_t st) {
-    int b = action_partials(g);
-    if (prec == 0) k_action<double, 18><<<b, kThreads, 0, st>>>(g, (const double *)U, partials);
-    else if (nc == 18) k_action<float, 18><<<b, kThreads, 0, st>>>(g, (const float *)U, partials);
-    else k_action<float, 12><<<b, kThreads, 0, st>>>(g, (const float *)U, partials);
+    int b = 0;
+    const auto run = [&](auto kernel, auto *links) {
+        b = meas_blocks(kernel, g, kActionBlocks);
+        kernel<<<b, kMeasThreads, 0, st>>>(g, links, partials);
+    };
+    if (prec == 0) run(k_action<double, 18>, (const double *)U);
+    else if (nc == 18) run(k_action<float, 18>, (const float *)U);
+    else run(k_action<float, 12>, (const float *)U);
     // <S>/beta = (1/V) sum_x (2/72) sum_{mu<nu} (3 - Re Tr P)
     k_sum_partials<<<1, 1024, 0, st>>>(partials, b, 2.0 / 72.0 / (double)g.V, out);
     count_launches(2);
@@ -830,25 +907,14 @@ cudaError_t launch_action(int prec, int nc, const Geo &g, const void *U, double 
 
 cudaError_t launch_observables(int prec, int nc, const Geo &g, const void *U, double *partials, double *out,
                                double *S_site, double *SR_site, double *q_site, cudaStream_t st) {
-    // one balanced wave: as many blocks as are resident at once (the kernel's
-    // registers allow one or two per SM), at most 400 (the partials buffer)
-    int b = nblocks(g.V), dev = 0, n_sm = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    if (prec == 0)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_observables<double, 18>, kThreads, 0);
-    else if (nc == 18)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_observables<float, 18>, kThreads, 0);
-    else
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_observables<float, 12>, kThreads, 0);
-    const int wave = std::max(1, n_sm * std::max(per_sm, 1));
-    b = std::min(b, std::min(wave, 400));
-    if (prec == 0)
-        k_observables<double, 18><<<b, kThreads, 0, st>>>(g, (const double *)U, partials, S_site, SR_site, q_site);
-    else if (nc == 18)
-        k_observables<float, 18><<<b, kThreads, 0, st>>>(g, (const float *)U, partials, S_site, SR_site, q_site);
-    else
-        k_observables<float, 12><<<b, kThreads, 0, st>>>(g, (const float *)U, partials, S_site, SR_site, q_site);
+    int b = 0;
+    const auto run = [&](auto kernel, auto *links) {
+        b = meas_blocks(kernel, g, kObsBlocks);
+        kernel<<<b, kMeasThreads, 0, st>>>(g, links, partials, S_site, SR_site, q_site);
+    };
+    if (prec == 0) run(k_observables<double, 18>, (const double *)U);
+    else if (nc == 18) run(k_observables<float, 18>, (const float *)U);
+    else run(k_observables<float, 12>, (const float *)U);
     k_sum_partials3<<<1, 1024, 0, st>>>(partials, b, 1.0 / (double)g.V, out);
     count_launches(2);
     return cudaGetLastError();
@@ -865,27 +931,33 @@ cudaError_t launch_correlation(const double *a, const double *b, long long n, do
 
 cudaError_t preload_vortex_kernels() {
     cudaFuncAttributes a;
-    cudaError_t e = cudaFuncGetAttributes(&a, k_vortex_links<double, 18>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_vortex_links<float, 18>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_vortex_links<float, 12>);
+    cudaError_t e = cudaFuncGetAttributes(&a, k_vortex_links<double, 18, false>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_vortex_links<float, 18, false>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_vortex_links<float, 12, false>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_vortex_links<double, 18, true>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_vortex_links<float, 18, true>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_vortex_links<float, 12, true>);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_vortex_charges);
     return e;
 }
 
-cudaError_t launch_vortex(int prec, int nc, const Geo &g, const void *U, const int8_t *ref, int8_t *cur,
+template <class T, int NC>
+static void vortex_links(const Geo &g, const void *U, const int8_t *ref, int8_t *dz, unsigned long long *counts,
+                         unsigned long long *mbits, cudaStream_t st, const void *G) {
+    const int b = nblocks(g.V);
+    if (G)
+        k_vortex_links<T, NC, true><<<b, kThreads, 0, st>>>(g, (const T *)U, ref, dz, counts, mbits, (const T *)G);
+    else
+        k_vortex_links<T, NC, false><<<b, kThreads, 0, st>>>(g, (const T *)U, ref, dz, counts, mbits, nullptr);
+}
+
+cudaError_t launch_vortex(int prec, int nc, const Geo &g, const void *U, const int8_t *ref, int8_t *dz,
                           unsigned long long *counts, unsigned long long *mbits, cudaStream_t st,
                           const void *G) {
-    int b = nblocks(4ll * g.V);
-    if (prec == 0)
-        k_vortex_links<double, 18><<<b, kThreads, 0, st>>>(g, (const double *)U, ref, cur, counts, mbits,
-                                                           (const double *)G);
-    else if (nc == 18)
-        k_vortex_links<float, 18><<<b, kThreads, 0, st>>>(g, (const float *)U, ref, cur, counts, mbits,
-                                                          (const float *)G);
-    else
-        k_vortex_links<float, 12><<<b, kThreads, 0, st>>>(g, (const float *)U, ref, cur, counts, mbits,
-                                                          (const float *)G);
-    k_vortex_charges<<<nblocks(g.V), kThreads, 0, st>>>(g, ref, cur, counts);
+    if (prec == 0) vortex_links<double, 18>(g, U, ref, dz, counts, mbits, st, G);
+    else if (nc == 18) vortex_links<float, 18>(g, U, ref, dz, counts, mbits, st, G);
+    else vortex_links<float, 12>(g, U, ref, dz, counts, mbits, st, G);
+    k_vortex_charges<<<nblocks(g.V), kThreads, 0, st>>>(g, dz, counts);
     count_launches(2);
     return cudaGetLastError();
 }
