@@ -259,7 +259,7 @@ __global__ void __launch_bounds__(VS_RING_THREADS, RECT ? VS_RING_MINB : 4) k_fl
 template <class T, int NC>
 cudaError_t launch_ape_tpl(bool rect, int mu, const ApeParams &p, cudaStream_t st) {
     if (p.n_threads <= 0) return cudaSuccess;
-    if constexpr (sizeof(T) == 4 && VS_RING) {
+    if constexpr (sizeof(T) == 4) {
         if (rect) {   // annealed classes and simultaneous sweeps alike
             const int rb = (p.n_threads + VS_RING_THREADS - 1) / VS_RING_THREADS;
             constexpr int sm = ring6_smem_bytes<NC>();
@@ -284,7 +284,7 @@ cudaError_t launch_ape_tpl(bool rect, int mu, const ApeParams &p, cudaStream_t s
     const int blocks = (p.n_threads + threads - 1) / threads;
 #define VS_LAUNCH(R, M) k_ape<T, NC, R, M><<<blocks, threads, 0, st>>>(p)
     if (rect) {
-        switch (mu) {
+        if constexpr (sizeof(T) == 8) switch (mu) {
             case 0: VS_LAUNCH(true, 0); break;
             case 1: VS_LAUNCH(true, 1); break;
             case 2: VS_LAUNCH(true, 2); break;
@@ -306,7 +306,7 @@ cudaError_t launch_ape_tpl(bool rect, int mu, const ApeParams &p, cudaStream_t s
 template <class T, int NC>
 cudaError_t launch_flow_tpl(bool rect, int mu, const FlowParams &p, cudaStream_t st) {
     if (p.n_threads <= 0) return cudaSuccess;
-    if constexpr (sizeof(T) == 4 && VS_RING) {
+    if constexpr (sizeof(T) == 4) {
         const int rb = (p.n_threads + VS_RING_THREADS - 1) / VS_RING_THREADS;
         constexpr int sm = ring6_smem_bytes<NC>();
         static std::atomic<unsigned long long> attr_set{0};
@@ -339,28 +339,29 @@ cudaError_t launch_flow_tpl(bool rect, int mu, const FlowParams &p, cudaStream_t
 #undef VS_LAUNCH
         count_launches(1);
         return cudaGetLastError();
-    }
-    const int threads = VS_SUBSWEEP_THREADS;
-    const int blocks = (p.n_threads + threads - 1) / threads;
-#define VS_LAUNCH(R, M) k_flow_stage<T, NC, R, M><<<blocks, threads, 0, st>>>(p)
-    if (rect) {
-        switch (mu) {
-            case 0: VS_LAUNCH(true, 0); break;
-            case 1: VS_LAUNCH(true, 1); break;
-            case 2: VS_LAUNCH(true, 2); break;
-            default: VS_LAUNCH(true, 3); break;
-        }
     } else {
-        switch (mu) {
-            case 0: VS_LAUNCH(false, 0); break;
-            case 1: VS_LAUNCH(false, 1); break;
-            case 2: VS_LAUNCH(false, 2); break;
-            default: VS_LAUNCH(false, 3); break;
+        const int threads = VS_SUBSWEEP_THREADS;
+        const int blocks = (p.n_threads + threads - 1) / threads;
+#define VS_LAUNCH(R, M) k_flow_stage<T, NC, R, M><<<blocks, threads, 0, st>>>(p)
+        if (rect) {
+            switch (mu) {
+                case 0: VS_LAUNCH(true, 0); break;
+                case 1: VS_LAUNCH(true, 1); break;
+                case 2: VS_LAUNCH(true, 2); break;
+                default: VS_LAUNCH(true, 3); break;
+            }
+        } else {
+            switch (mu) {
+                case 0: VS_LAUNCH(false, 0); break;
+                case 1: VS_LAUNCH(false, 1); break;
+                case 2: VS_LAUNCH(false, 2); break;
+                default: VS_LAUNCH(false, 3); break;
+            }
         }
-    }
 #undef VS_LAUNCH
-    count_launches(1);
-    return cudaGetLastError();
+        count_launches(1);
+        return cudaGetLastError();
+    }
 }
 
 }  // namespace vs

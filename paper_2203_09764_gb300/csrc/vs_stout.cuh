@@ -21,7 +21,7 @@
 // Exponential: exp(rho Q) = exp(i H) with H = -i rho Q Hermitian traceless.
 // Cayley-Hamilton, H^3 = tau H + delta I with tau = Tr(H^2)/2, delta = det H,
 // so H^n = a_n I + b_n H + c_n H^2 with a_{n+1} = delta c_n,
-// b_{n+1} = a_n + tau c_n, c_{n+1} = b_n, and
+// b_{n+1} = a_n + tau c_n, c_{n+1} = b_n (so c alone satisfies a recurrence), and
 //   exp(iH) = f0 I + f1 H + f2 H^2,  f_j = sum_n i^n (a_n, b_n, c_n)_j / n!.
 // The scalar series converges like |H|^n / n! with no cancellation for
 // |H| <= 1 and needs no eigenvalues, so it has no degeneracy problem.
@@ -211,32 +211,32 @@ __device__ __forceinline__ bool ch_exp_coeffs(R h00, R h11, R h22, R h01r, R h01
     const R pr = h01r * h12r - h01i * h12i, pi = h01r * h12i + h01i * h12r;
     const R delta = h00 * h11 * h22 + R(2) * (pr * h02r + pi * h02i) - h00 * a12 - h11 * a02 - h22 * a01;
     const R r2 = R(2) * tau;
-    R f0r = 1, f0i = 0, f1r = 0, f1i = 0, f2r = 0, f2i = 0;
-    R a = 1, b = 0, c = 0, bound = 1;
+    // c_n alone, c_{n+1} = tau c_{n-1} + delta c_{n-2} (b_n = c_{n+1}, a_n = delta c_{n-1}
+    // for n >= 1): f2 = sum i^n c_n / n!, f1 = sum i^n c_{n+1} / n!, and
+    // (f0 - 1) / delta = sum i^n c_{n-1} / n!, five operations per term.
+    R s0r = 0, s0i = 0, f1r = 0, f1i = 0, f2r = 0, f2i = 0;
+    R cm = 0, c = 0, cp = 1, w = 1, bound = 1;        // c_{n-1}, c_n, c_{n+1} at n = 1; 1 / n!
     const R eps = Tol<R>::eps();
 #pragma unroll
     for (int g4 = 0; g4 < GROUPS; ++g4) {
         const int n = 4 * g4 + 1;
-        R na, nb, nc, inv;
-        inv = R(1) / R(n);                        // i^n = i
-        na = delta * c * inv; nb = (a + tau * c) * inv; nc = b * inv;
-        a = na; b = nb; c = nc;
-        f0i += a; f1i += b; f2i += c;
-        inv = R(1) / R(n + 1);                    // i^n = -1
-        na = delta * c * inv; nb = (a + tau * c) * inv; nc = b * inv;
-        a = na; b = nb; c = nc;
-        f0r -= a; f1r -= b; f2r -= c;
-        inv = R(1) / R(n + 2);                    // i^n = -i
-        na = delta * c * inv; nb = (a + tau * c) * inv; nc = b * inv;
-        a = na; b = nb; c = nc;
-        f0i -= a; f1i -= b; f2i -= c;
-        inv = R(1) / R(n + 3);                    // i^n = 1
-        na = delta * c * inv; nb = (a + tau * c) * inv; nc = b * inv;
-        a = na; b = nb; c = nc;
-        f0r += a; f1r += b; f2r += c;
+        R next;
+        w *= R(1) / R(n);                             // i^n = i
+        s0i = fma(w, cm, s0i); f1i = fma(w, cp, f1i); f2i = fma(w, c, f2i);
+        next = fma(tau, c, delta * cm); cm = c; c = cp; cp = next;
+        w *= R(1) / R(n + 1);                         // i^n = -1
+        s0r = fma(-w, cm, s0r); f1r = fma(-w, cp, f1r); f2r = fma(-w, c, f2r);
+        next = fma(tau, c, delta * cm); cm = c; c = cp; cp = next;
+        w *= R(1) / R(n + 2);                         // i^n = -i
+        s0i = fma(-w, cm, s0i); f1i = fma(-w, cp, f1i); f2i = fma(-w, c, f2i);
+        next = fma(tau, c, delta * cm); cm = c; c = cp; cp = next;
+        w *= R(1) / R(n + 3);                         // i^n = 1
+        s0r = fma(w, cm, s0r); f1r = fma(w, cp, f1r); f2r = fma(w, c, f2r);
+        next = fma(tau, c, delta * cm); cm = c; c = cp; cp = next;
         bound *= r2 * r2 * (R(1) / (R(n) * R(n + 1) * R(n + 2) * R(n + 3)));
         if (bound < eps) break;
     }
+    const R f0r = fma(delta, s0r, R(1)), f0i = delta * s0i;
     f[0] = f0r; f[1] = f0i; f[2] = f1r; f[3] = f1i; f[4] = f2r; f[5] = f2i;
     return r2 <= rmax * rmax;
 }
@@ -337,8 +337,11 @@ __device__ __forceinline__ M3<T> stout_candidate(const M3<T> &sig, const M3<T> &
     return m3_mul(Mx, Ux);
 }
 
+// Threads of the plain-load kernels (FP64, and FP32 APE on plaquette staples).  128
+// and not 256: an FP64 thread holds up to 255 registers, two blocks of 128 fit an SM
+// as one of 256 does, and the last, partial layer of blocks is half as long.
 #ifndef VS_SUBSWEEP_THREADS
-#define VS_SUBSWEEP_THREADS 256
+#define VS_SUBSWEEP_THREADS 128
 #endif
 #ifndef VS_SUBSWEEP_MINB
 #define VS_SUBSWEEP_MINB (512 / VS_SUBSWEEP_THREADS)
@@ -499,26 +502,23 @@ __global__ void __launch_bounds__(32) k_redecide(SubsweepParams a) {
     }
 }
 
-// One thread per link of the colour class (or of direction MU when colour < 0).
-// FP32: at most 65536 / (VS_SUBSWEEP_THREADS * VS_SUBSWEEP_MINB) registers per
-// thread (128 by default), so VS_SUBSWEEP_MINB blocks fit on an SM (16 warps).
-template <class T, int NC, bool RECT, int MU>
-__global__ void __launch_bounds__(VS_SUBSWEEP_THREADS, sizeof(T) == 4 ? VS_SUBSWEEP_MINB : 1)
-    k_subsweep(SubsweepParams a) {
+// FP64 with plaquette staples: one thread per link of the colour class (or of
+// direction MU when colour < 0), for launches that fill the chip several times.
+template <int MU>
+__global__ void __launch_bounds__(VS_SUBSWEEP_THREADS) k_subsweep(SubsweepParams a) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const bool active = t < a.n_threads;
-    Update<T> u;
+    Update<double> u;
     if (active) {
         const Geo &g = a.g;
         Pt x = a.colour >= 0 ? class_site<MU>(g, a.colour, t) : dir_site<MU>(g, t);
         const int i = sidx(g, x);
-        const T *Us = static_cast<const T *>(a.Usrc);
-        const T c0 = sizeof(T) == 4 ? T(a.c0_f) : T(a.c0), c1 = sizeof(T) == 4 ? T(a.c1_f) : T(a.c1);
-        M3<T> sig = staple_sum<T, NC, RECT, MU>(g, Us, x, c0, c1);
-        M3<T> Ux = load_link<T, NC>(Us, g.P, MU, i);
-        stout_store<T, NC, MU>(a, x, i, sig, Ux, u);
+        const double *Us = static_cast<const double *>(a.Usrc);
+        M3<double> sig = staple_sum<double, 18, false, MU>(g, Us, x, a.c0, a.c1);
+        M3<double> Ux = load_link<double, 18>(Us, g.P, MU, i);
+        stout_store<double, 18, MU>(a, x, i, sig, Ux, u);
     }
-    count_update<T>(a.counters, u);
+    count_update<double>(a.counters, u);
 }
 
 // ---------------------------------------------------------------------------
@@ -530,9 +530,6 @@ __global__ void __launch_bounds__(VS_SUBSWEEP_THREADS, sizeof(T) == 4 ? VS_SUBSW
 // the thread's stream; every slot index is known at compile time.
 // ---------------------------------------------------------------------------
 
-#ifndef VS_RING
-#define VS_RING 1
-#endif
 #ifndef VS_RING_THREADS
 #define VS_RING_THREADS 128
 #endif

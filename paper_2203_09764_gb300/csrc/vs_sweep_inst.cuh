@@ -20,11 +20,11 @@ void launch_redecide(int mu, const SubsweepParams &p, cudaStream_t st) {
     count_launches(1);
 }
 
-template <class T, int NC>
+// FP32 class launches: the cp.async link-ring kernels.
+template <int NC>
 cudaError_t launch_subsweep_tpl(bool rect, int mu, const SubsweepParams &p, cudaStream_t st) {
     if (p.n_threads <= 0) return cudaSuccess;
-    if constexpr (sizeof(T) == 4 && VS_RING) {
-        // FP32: the cp.async link-ring kernels
+    {
         if (rect) {
             const int rb = (p.n_threads + VS_RING_THREADS - 1) / VS_RING_THREADS;
             constexpr int sm = ring6_smem_bytes<NC>();
@@ -66,39 +66,12 @@ cudaError_t launch_subsweep_tpl(bool rect, int mu, const SubsweepParams &p, cuda
             return cudaGetLastError();
         }
     }
-    const int threads = VS_SUBSWEEP_THREADS;
-    const int blocks = (p.n_threads + threads - 1) / threads;
-#define VS_LAUNCH(R, M) k_subsweep<T, NC, R, M><<<blocks, threads, 0, st>>>(p)
-    if (rect) {
-        switch (mu) {
-            case 0: VS_LAUNCH(true, 0); break;
-            case 1: VS_LAUNCH(true, 1); break;
-            case 2: VS_LAUNCH(true, 2); break;
-            default: VS_LAUNCH(true, 3); break;
-        }
-    } else {
-        switch (mu) {
-            case 0: VS_LAUNCH(false, 0); break;
-            case 1: VS_LAUNCH(false, 1); break;
-            case 2: VS_LAUNCH(false, 2); break;
-            default: VS_LAUNCH(false, 3); break;
-        }
-    }
-#undef VS_LAUNCH
-    count_launches(1);
-    if constexpr (sizeof(T) == 4) {
-        if (p.defer_idx) {
-            if (rect) launch_redecide<NC, true>(mu, p, st);
-            else launch_redecide<NC, false>(mu, p, st);
-        }
-    }
-    return cudaGetLastError();
 }
 
 template <class T, int NC>
 cudaError_t launch_aus_tpl(bool rect, int mu, const AusParams &p, cudaStream_t st) {
     if (p.n_threads <= 0) return cudaSuccess;
-    if constexpr (sizeof(T) == 4 && VS_RING) {
+    if constexpr (sizeof(T) == 4) {
         // FP32: the link-ring kernels
         if (rect) {
             const int rb = (p.n_threads + VS_RING_THREADS - 1) / VS_RING_THREADS;
@@ -138,28 +111,29 @@ cudaError_t launch_aus_tpl(bool rect, int mu, const AusParams &p, cudaStream_t s
             count_launches(1);
             return cudaGetLastError();
         }
-    }
-    const int threads = VS_SUBSWEEP_THREADS;
-    const int blocks = (p.n_threads + threads - 1) / threads;
-#define VS_LAUNCH(R, M) k_aus<T, NC, R, M><<<blocks, threads, 0, st>>>(p)
-    if (rect) {
-        switch (mu) {
-            case 0: VS_LAUNCH(true, 0); break;
-            case 1: VS_LAUNCH(true, 1); break;
-            case 2: VS_LAUNCH(true, 2); break;
-            default: VS_LAUNCH(true, 3); break;
-        }
     } else {
-        switch (mu) {
-            case 0: VS_LAUNCH(false, 0); break;
-            case 1: VS_LAUNCH(false, 1); break;
-            case 2: VS_LAUNCH(false, 2); break;
-            default: VS_LAUNCH(false, 3); break;
+        const int threads = VS_SUBSWEEP_THREADS;
+        const int blocks = (p.n_threads + threads - 1) / threads;
+#define VS_LAUNCH(R, M) k_aus<T, NC, R, M><<<blocks, threads, 0, st>>>(p)
+        if (rect) {
+            switch (mu) {
+                case 0: VS_LAUNCH(true, 0); break;
+                case 1: VS_LAUNCH(true, 1); break;
+                case 2: VS_LAUNCH(true, 2); break;
+                default: VS_LAUNCH(true, 3); break;
+            }
+        } else {
+            switch (mu) {
+                case 0: VS_LAUNCH(false, 0); break;
+                case 1: VS_LAUNCH(false, 1); break;
+                case 2: VS_LAUNCH(false, 2); break;
+                default: VS_LAUNCH(false, 3); break;
+            }
         }
-    }
 #undef VS_LAUNCH
-    count_launches(1);
-    return cudaGetLastError();
+        count_launches(1);
+        return cudaGetLastError();
+    }
 }
 
 }  // namespace vs
