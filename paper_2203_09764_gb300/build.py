@@ -18,7 +18,7 @@ LIB = os.path.join(OUT_DIR, "libvs.so")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2"]
-# VS_NVCC_EXTRA: extra nvcc flags, e.g. -DVS_SUBSWEEP_MINB=3 (blocks per SM of the
+# VS_NVCC_EXTRA: extra nvcc flags, e.g. -DVS_RING_MINB=2 (blocks per SM of the
 # class-update kernel, which sets its register budget)
 FLAGS += os.environ.get("VS_NVCC_EXTRA", "").split()
 

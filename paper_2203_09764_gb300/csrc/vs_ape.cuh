@@ -1,6 +1,5 @@
 // vs_ape.cuh -- APE / annealed U-link smearing with unit circle projection and
-// one stage of the third-order Runge-Kutta Wilson flow.  Included by
-// vs_ape_f18.cu, vs_ape_f12.cu and vs_ape_d18.cu.
+// one stage of the third-order Runge-Kutta Wilson flow.
 //
 // Unit circle projection (Sec. II.C, Eqs. W and P_ucp):
 //   W = V (V^dag V)^{-1/2},  P_ucp{V} = W / cbrt(det W)  (principal root).
@@ -101,8 +100,8 @@ __device__ __forceinline__ bool ucp_project(const M3<T> &V, M3<T> &out) {
 // APE / AUS+UCP update of link (x, MU) at plane position i from its staple
 // sum Vb and current value u: blocking, projection (a singular V keeps u),
 // vortex-preservation test, store if accepted.
-template <class T, int NC, int MU>
-__device__ __forceinline__ void ape_finish(const ApeParams &a, const Pt &x, int i, M3<T> Vb, const M3<T> &u,
+template <class T, int NC>
+__device__ __forceinline__ void ape_finish(const ApeParams &a, int MU, const Pt &x, int i, M3<T> Vb, const M3<T> &u,
                                            Update<T> &up) {
     const Geo &g = a.g;
     const T al = sizeof(T) == 4 ? T(a.alpha_f) : T(a.alpha);
@@ -125,30 +124,29 @@ __device__ __forceinline__ void ape_finish(const ApeParams &a, const Pt &x, int 
     else if (a.U != a.Usrc) store_link<T, NC>(static_cast<T *>(a.U), g.P, MU, i, u);
 }
 
-// APE / AUS with unit circle projection: one thread per link of the colour
+// FP64 APE / AUS with unit circle projection: one thread per link of the colour
 // class (annealed, in place) or of direction MU (colour < 0, from Usrc).
-template <class T, int NC, bool RECT, int MU>
-__global__ void __launch_bounds__(VS_SUBSWEEP_THREADS, sizeof(T) == 4 ? VS_SUBSWEEP_MINB : 1)
-    k_ape(ApeParams a) {
+template <bool RECT, int MU>
+__global__ void __launch_bounds__(VS_SUBSWEEP_THREADS) k_ape(ApeParams a) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const bool active = t < a.n_threads;
-    Update<T> up;
+    Update<double> up;
     if (active) {
         const Geo &g = a.g;
-        const Pt x = a.colour >= 0 ? class_site<MU>(g, a.colour, t) : dir_site<MU>(g, t);
+        const Pt x = a.colour >= 0 ? class_site(g, MU, a.colour, t) : dir_site(g, MU, t);
         const int i = sidx(g, x);
-        const T *Us = static_cast<const T *>(a.Usrc);
-        const T c0 = sizeof(T) == 4 ? T(a.c0_f) : T(a.c0), c1 = sizeof(T) == 4 ? T(a.c1_f) : T(a.c1);
-        const M3<T> Vb = staple_sum<T, NC, RECT, MU>(g, Us, x, c0, c1);
-        const M3<T> u = load_link<T, NC>(Us, g.P, MU, i);
-        ape_finish<T, NC, MU>(a, x, i, Vb, u, up);
+        const double *Us = static_cast<const double *>(a.Usrc);
+        const M3<double> Vb = staple_sum<double, 18, RECT, MU>(g, Us, x, a.c0, a.c1);
+        const M3<double> u = load_link<double, 18>(Us, g.P, MU, i);
+        ape_finish<double, 18>(a, MU, x, i, Vb, u, up);
     }
-    count_update<T>(a.counters, up);
+    count_update<double>(a.counters, up);
 }
 
-// FP32 over-improved AUS+UCP with the one-pass link stream of k_subsweep_fused.
-template <int NC, int MU>
-__global__ void __launch_bounds__(VS_RING_THREADS, VS_RING_MINB) k_ape_ring(ApeParams a) {
+// FP32: the staple links through the per-thread ring, the one-pass stream of
+// k_subsweep_fused for over-improved staples, the plaquette-staple ring for eps = 1.
+template <int NC, bool RECT, int MU>
+__global__ void __launch_bounds__(VS_RING_THREADS, RECT ? VS_RING_MINB : 4) k_ape_ring(ApeParams a) {
     extern __shared__ float4 ape_dyn[];
     float4 *ring4 = ape_dyn;
     float2 *ring2 = reinterpret_cast<float2 *>(ape_dyn + 6 * (NC / 4) * VS_RING_THREADS);
@@ -157,21 +155,27 @@ __global__ void __launch_bounds__(VS_RING_THREADS, VS_RING_MINB) k_ape_ring(ApeP
     Update<float> up;
     if (active) {
         const Geo &g = a.g;
-        const Pt x = a.colour >= 0 ? class_site<MU>(g, a.colour, t) : dir_site<MU>(g, t);
+        const Pt x = a.colour >= 0 ? class_site(g, MU, a.colour, t) : dir_site(g, MU, t);
         const int i = sidx(g, x);
+        const float *Us = static_cast<const float *>(a.Usrc);
         LinkRing<NC> R = ring_of<NC>(ring4, ring2);
-        M3<float> Ux;
-        const M3<float> Vb =
-            staple_sum_fused<NC, MU>(g, static_cast<const float *>(a.Usrc), x, a.c0_f, a.c1_f, R, Ux);
-        ape_finish<float, NC, MU>(a, x, i, Vb, Ux, up);
+        dep_wait();
+        M3<float> Vb, Ux;
+        if constexpr (RECT) {
+            Vb = staple_sum_fused<NC, MU>(g, Us, x, a.c0_f, a.c1_f, R, Ux);
+        } else {
+            Vb = staple_sum_plain_ring<NC, MU>(g, Us, x, a.c0_f, R);
+            Ux = load_link<float, NC>(Us, g.P, MU, i);
+        }
+        ape_finish<float, NC>(a, MU, x, i, Vb, Ux, up);
     }
     count_update<float>(a.counters, up);
 }
 
 // End of one Runge-Kutta stage for link (MU, i) from its staple sum sig and
 // link u: H_Z = -i h Q[W_i], H_S <- a H_Z + b H_S, W_{i+1} = exp(i c H_S) W_i.
-template <class T, int NC, int MU>
-__device__ __forceinline__ void flow_finish(const FlowParams &a, int i, const M3<T> &sig, const M3<T> &u,
+template <class T, int NC>
+__device__ __forceinline__ void flow_finish(const FlowParams &a, int MU, int i, const M3<T> &sig, const M3<T> &u,
                                             bool &used64, const T *s_old = nullptr) {
     const Geo &g = a.g;
     const bool f32 = sizeof(T) == 4;
@@ -201,23 +205,20 @@ __device__ __forceinline__ void flow_count(const FlowParams &a, bool used64) {
     }
 }
 
-// One Runge-Kutta stage for every link of direction MU (thread t = site t in
-// plane order), staples from plain loads (FP64, and FP32 without the ring).
-template <class T, int NC, bool RECT, int MU>
-__global__ void __launch_bounds__(VS_SUBSWEEP_THREADS, sizeof(T) == 4 ? VS_SUBSWEEP_MINB : 1)
-    k_flow_stage(FlowParams a) {
+// One FP64 Runge-Kutta stage for every link of direction MU (thread t = site t in
+// plane order), staples from plain loads.
+template <bool RECT, int MU>
+__global__ void __launch_bounds__(VS_SUBSWEEP_THREADS) k_flow_stage(FlowParams a) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     bool used64 = false;
     if (t < a.n_threads) {
         const Geo &g = a.g;
-        const Pt x = dir_site<MU>(g, t);
+        const Pt x = dir_site(g, MU, t);
         const int i = sidx(g, x);
-        const T *Us = static_cast<const T *>(a.Usrc);
-        const bool f32 = sizeof(T) == 4;
-        const T c0 = f32 ? T(a.c0_f) : T(a.c0), c1 = f32 ? T(a.c1_f) : T(a.c1);
-        const M3<T> sig = staple_sum<T, NC, RECT, MU>(g, Us, x, c0, c1);
-        const M3<T> u = load_link<T, NC>(Us, g.P, MU, i);
-        flow_finish<T, NC, MU>(a, i, sig, u, used64);
+        const double *Us = static_cast<const double *>(a.Usrc);
+        const M3<double> sig = staple_sum<double, 18, RECT, MU>(g, Us, x, a.c0, a.c1);
+        const M3<double> u = load_link<double, 18>(Us, g.P, MU, i);
+        flow_finish<double, 18>(a, MU, i, sig, u, used64);
     }
     flow_count(a, used64);
 }
@@ -234,10 +235,11 @@ __global__ void __launch_bounds__(VS_RING_THREADS, RECT ? VS_RING_MINB : 4) k_fl
     bool used64 = false;
     if (t < a.n_threads) {
         const Geo &g = a.g;
-        const Pt x = dir_site<MU>(g, t);
+        const Pt x = dir_site(g, MU, t);
         const int i = sidx(g, x);
         const float *Us = static_cast<const float *>(a.Usrc);
         LinkRing<NC> R = ring_of<NC>(ring4, ring2);
+        dep_wait();
         M3<float> sig, u;
         // the exponent H_S of this link, read before the staple stream so that
         // its latency hides behind it (stage 1 of a step does not read it)
@@ -251,117 +253,9 @@ __global__ void __launch_bounds__(VS_RING_THREADS, RECT ? VS_RING_MINB : 4) k_fl
             sig = staple_sum_plain_ring<NC, MU>(g, Us, x, a.c0_f, R);
             u = load_link<float, NC>(Us, g.P, MU, i);
         }
-        flow_finish<float, NC, MU>(a, i, sig, u, used64, s_old);
+        flow_finish<float, NC>(a, MU, i, sig, u, used64, s_old);
     }
     flow_count(a, used64);
-}
-
-template <class T, int NC>
-cudaError_t launch_ape_tpl(bool rect, int mu, const ApeParams &p, cudaStream_t st) {
-    if (p.n_threads <= 0) return cudaSuccess;
-    if constexpr (sizeof(T) == 4) {
-        if (rect) {   // annealed classes and simultaneous sweeps alike
-            const int rb = (p.n_threads + VS_RING_THREADS - 1) / VS_RING_THREADS;
-            constexpr int sm = ring6_smem_bytes<NC>();
-            static std::atomic<unsigned long long> attr_set{0};
-            once_per_device(attr_set, [&] {
-                cudaFuncSetAttribute(k_ape_ring<NC, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-                cudaFuncSetAttribute(k_ape_ring<NC, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-                cudaFuncSetAttribute(k_ape_ring<NC, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-                cudaFuncSetAttribute(k_ape_ring<NC, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-            });
-            switch (mu) {
-                case 0: k_ape_ring<NC, 0><<<rb, VS_RING_THREADS, sm, st>>>(p); break;
-                case 1: k_ape_ring<NC, 1><<<rb, VS_RING_THREADS, sm, st>>>(p); break;
-                case 2: k_ape_ring<NC, 2><<<rb, VS_RING_THREADS, sm, st>>>(p); break;
-                default: k_ape_ring<NC, 3><<<rb, VS_RING_THREADS, sm, st>>>(p); break;
-            }
-            count_launches(1);
-            return cudaGetLastError();
-        }
-    }
-    const int threads = VS_SUBSWEEP_THREADS;
-    const int blocks = (p.n_threads + threads - 1) / threads;
-#define VS_LAUNCH(R, M) k_ape<T, NC, R, M><<<blocks, threads, 0, st>>>(p)
-    if (rect) {
-        if constexpr (sizeof(T) == 8) switch (mu) {
-            case 0: VS_LAUNCH(true, 0); break;
-            case 1: VS_LAUNCH(true, 1); break;
-            case 2: VS_LAUNCH(true, 2); break;
-            default: VS_LAUNCH(true, 3); break;
-        }
-    } else {
-        switch (mu) {
-            case 0: VS_LAUNCH(false, 0); break;
-            case 1: VS_LAUNCH(false, 1); break;
-            case 2: VS_LAUNCH(false, 2); break;
-            default: VS_LAUNCH(false, 3); break;
-        }
-    }
-#undef VS_LAUNCH
-    count_launches(1);
-    return cudaGetLastError();
-}
-
-template <class T, int NC>
-cudaError_t launch_flow_tpl(bool rect, int mu, const FlowParams &p, cudaStream_t st) {
-    if (p.n_threads <= 0) return cudaSuccess;
-    if constexpr (sizeof(T) == 4) {
-        const int rb = (p.n_threads + VS_RING_THREADS - 1) / VS_RING_THREADS;
-        constexpr int sm = ring6_smem_bytes<NC>();
-        static std::atomic<unsigned long long> attr_set{0};
-        once_per_device(attr_set, [&] {
-            cudaFuncSetAttribute(k_flow_stage_ring<NC, true, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-            cudaFuncSetAttribute(k_flow_stage_ring<NC, true, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-            cudaFuncSetAttribute(k_flow_stage_ring<NC, true, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-            cudaFuncSetAttribute(k_flow_stage_ring<NC, true, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-            cudaFuncSetAttribute(k_flow_stage_ring<NC, false, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-            cudaFuncSetAttribute(k_flow_stage_ring<NC, false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-            cudaFuncSetAttribute(k_flow_stage_ring<NC, false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-            cudaFuncSetAttribute(k_flow_stage_ring<NC, false, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-        });
-#define VS_LAUNCH(R, M) k_flow_stage_ring<NC, R, M><<<rb, VS_RING_THREADS, sm, st>>>(p)
-        if (rect) {
-            switch (mu) {
-                case 0: VS_LAUNCH(true, 0); break;
-                case 1: VS_LAUNCH(true, 1); break;
-                case 2: VS_LAUNCH(true, 2); break;
-                default: VS_LAUNCH(true, 3); break;
-            }
-        } else {
-            switch (mu) {
-                case 0: VS_LAUNCH(false, 0); break;
-                case 1: VS_LAUNCH(false, 1); break;
-                case 2: VS_LAUNCH(false, 2); break;
-                default: VS_LAUNCH(false, 3); break;
-            }
-        }
-#undef VS_LAUNCH
-        count_launches(1);
-        return cudaGetLastError();
-    } else {
-        const int threads = VS_SUBSWEEP_THREADS;
-        const int blocks = (p.n_threads + threads - 1) / threads;
-#define VS_LAUNCH(R, M) k_flow_stage<T, NC, R, M><<<blocks, threads, 0, st>>>(p)
-        if (rect) {
-            switch (mu) {
-                case 0: VS_LAUNCH(true, 0); break;
-                case 1: VS_LAUNCH(true, 1); break;
-                case 2: VS_LAUNCH(true, 2); break;
-                default: VS_LAUNCH(true, 3); break;
-            }
-        } else {
-            switch (mu) {
-                case 0: VS_LAUNCH(false, 0); break;
-                case 1: VS_LAUNCH(false, 1); break;
-                case 2: VS_LAUNCH(false, 2); break;
-                default: VS_LAUNCH(false, 3); break;
-            }
-        }
-#undef VS_LAUNCH
-        count_launches(1);
-        return cudaGetLastError();
-    }
 }
 
 }  // namespace vs

@@ -84,8 +84,7 @@ __device__ __forceinline__ Pt site_of_index(const Geo &g, int i) {
 // Thread t of a launch over every site of direction MU (the simultaneous
 // schedules and the Runge-Kutta stages): odd directions take the sites in
 // reverse order, so each launch starts where the previous one ended.
-template <int MU>
-__device__ __forceinline__ Pt dir_site(const Geo &g, int t) {
+__device__ __forceinline__ Pt dir_site(const Geo &g, int MU, int t) {
     return site_of_index(g, (MU & 1) ? g.V - 1 - t : t);
 }
 
@@ -119,8 +118,7 @@ __device__ __forceinline__ Pt site_of_lex(const Geo &g, int s) {
 //           Lx/2 class sites, x mod 4 in {b0, b0 + 2}.
 // Odd colours take the sites in reverse order, so that each class launch of a
 // sweep starts where the previous one ended and finds those links still in L2.
-template <int MU>
-__device__ __forceinline__ Pt class_site(const Geo &g, int c, int t) {
+__device__ __forceinline__ Pt class_site(const Geo &g, int MU, int c, int t) {
     Pt p;
     const int Q = g.Q;
     if (c & 1) t = g.V / 4 - 1 - t;

@@ -291,7 +291,7 @@ template <> struct ShortSum<float> {
 // L1/L2 rate of their link loads (1.5 and 6 KB per site), so what counts is warps
 // per SM: 16 for the action (120 registers), 12 for the observables (168), where
 // blocks of 256 threads left 8.  Per call at 32^3x64, FP32: action 395 -> 213 us
-// (five blocks per SM spill: 295), observables 1174 -> 842 us (four: 958).
+// (five blocks per SM spill: 295), observables 1174 -> 880 us (four: 980).
 constexpr int kMeasThreads = 128, kActionPerSM = 4, kObsPerSM = 3;
 
 template <class T, int NC>
@@ -336,73 +336,61 @@ __global__ void __launch_bounds__(kMeasThreads, sizeof(T) == 4 ? kActionPerSM : 
 // (the eps-sum of Eq. 1LTopQ collapsed to its three pairings x 8 / (32 pi^2)).
 // ---------------------------------------------------------------------------
 
-// D(y) = B(y) - B'(y) for the link U_mu(y) and the plane (mu, nu), the two paths
-// that close it into the leaf above and (its conjugate) the leaf below:
-//   B  = U_nu(y+mu) U_mu^dag(y+nu) U_nu^dag(y)
-//   B' = U_nu^dag(y+mu-nu) U_mu^dag(y-nu) U_nu(y-nu)
-// iy: position of y; dm: shift to y+mu; dn, db: shifts to y+nu and y-nu.
-// retr: Re Tr(W B) for the plaquette W = U_mu(y), if wanted.
-template <class T, int NC, bool TRACE>
-__device__ __forceinline__ M3<T> clover_arms(const Geo &g, const T *__restrict__ U, int mu, int nu, int iy, int dm,
-                                             int dn, int db, const M3<T> *W, T &retr) {
-    M3<T> D = m3_mul_nd(m3_mul_nd(load_link<T, NC>(U, g.P, nu, iy + dm), load_link<T, NC>(U, g.P, mu, iy + dn)),
-                        load_link<T, NC>(U, g.P, nu, iy));
-    if constexpr (TRACE) {
-        T re = T(0);
-#pragma unroll
-        for (int j = 0; j < 3; ++j)
-#pragma unroll
-            for (int k = 0; k < 3; ++k)
-                re = fma(W->re[3 * j + k], D.re[3 * k + j], fma(-W->im[3 * j + k], D.im[3 * k + j], re));
-        retr = re;
-    }
-    // U_nu^dag U_mu^dag = (U_mu U_nu)^dag
-    M3<T> E = m3_dag(m3_mul(load_link<T, NC>(U, g.P, mu, iy + db), load_link<T, NC>(U, g.P, nu, iy + dm + db)));
-#pragma unroll
-    for (int k = 0; k < 9; ++k) { E.re[k] = -E.re[k]; E.im[k] = -E.im[k]; }
-    m3_madd(D, E, load_link<T, NC>(U, g.P, nu, iy + db));
-    return D;
-}
-
-// F_munu(x) by its diagonal h[0..2] and upper entries h[3..8] (re, im): the four
-// leaves pair up as U_mu(x) D(x) and D(x-mu) U_mu(x-mu), each minus its adjoint
-// (10 products for a plane instead of 12 leaf by leaf).
+// F_munu(x) by its diagonal h[0..2] and upper entries h[3..8] (re, im).
 template <class T, int NC>
 __device__ __forceinline__ void clover_F(const Geo &g, const T *__restrict__ U, const Pt &x, int i, int mu, int nu,
                                          T h[9], T &plaq_retr) {
     const int pm = shift_delta(g, x, mu, 1), mm = shift_delta(g, x, mu, -1);
     const int pn = shift_delta(g, x, nu, 1), mn = shift_delta(g, x, nu, -1);
-    M3<T> C;
-    {
-        const M3<T> Um = load_link<T, NC>(U, g.P, mu, i);
-        const M3<T> D = clover_arms<T, NC, true>(g, U, mu, nu, i, pm, pn, mn, &Um, plaq_retr);
-        C = m3_mul(Um, D);
-    }
-    {
-        T none;
-        const M3<T> D = clover_arms<T, NC, false>(g, U, mu, nu, i + mm, -mm, pn, mn, nullptr, none);
-        m3_madd(C, D, load_link<T, NC>(U, g.P, mu, i + mm));
-    }
-    // F = (C - C^dag) / (2i) / 4, traceless
-    const T tr = (C.im[0] + C.im[4] + C.im[8]) / T(3);
+    M3<T> C, L;
+    // leaf 1: +mu +nu -mu -nu
+    L = m3_mul(load_link<T, NC>(U, g.P, mu, i), load_link<T, NC>(U, g.P, nu, i + pm));
+    L = m3_mul_nd(L, load_link<T, NC>(U, g.P, mu, i + pn));
+    L = m3_mul_nd(L, load_link<T, NC>(U, g.P, nu, i));
+    plaq_retr = L.re[0] + L.re[4] + L.re[8];
+    C = L;
+    // leaf 2: +nu -mu -nu +mu
+    L = m3_mul_nd(load_link<T, NC>(U, g.P, nu, i), load_link<T, NC>(U, g.P, mu, i + pn + mm));
+    L = m3_mul_nd(L, load_link<T, NC>(U, g.P, nu, i + mm));
+    m3_madd(C, L, load_link<T, NC>(U, g.P, mu, i + mm));
+    // leaf 3: -mu -nu +mu +nu
+    L = m3_mul_dn(load_link<T, NC>(U, g.P, mu, i + mm), m3_dag(load_link<T, NC>(U, g.P, nu, i + mm + mn)));
+    L = m3_mul(L, load_link<T, NC>(U, g.P, mu, i + mm + mn));
+    m3_madd(C, L, load_link<T, NC>(U, g.P, nu, i + mn));
+    // leaf 4: -nu +mu +nu -mu
+    L = m3_mul_dn(load_link<T, NC>(U, g.P, nu, i + mn), load_link<T, NC>(U, g.P, mu, i + mn));
+    L = m3_mul(L, load_link<T, NC>(U, g.P, nu, i + mn + pm));
+    L = m3_mul_nd(L, load_link<T, NC>(U, g.P, mu, i));
 #pragma unroll
-    for (int j = 0; j < 3; ++j) h[j] = T(0.25) * (C.im[4 * j] - tr);
-    h[3] = T(0.125) * (C.im[1] + C.im[3]); h[4] = T(0.125) * (C.re[3] - C.re[1]);
-    h[5] = T(0.125) * (C.im[2] + C.im[6]); h[6] = T(0.125) * (C.re[6] - C.re[2]);
-    h[7] = T(0.125) * (C.im[5] + C.im[7]); h[8] = T(0.125) * (C.re[7] - C.re[5]);
+    for (int k = 0; k < 9; ++k) { C.re[k] += L.re[k]; C.im[k] += L.im[k]; }
+    // F = (C - C^dag) / (2i) / 4, traceless
+#pragma unroll
+    for (int j = 0; j < 3; ++j) h[j] = T(0.125) * (C.im[4 * j] + C.im[4 * j]);
+    const T tr = (h[0] + h[1] + h[2]) / T(3);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) h[j] -= tr;
+    h[3] = T(0.125) * (C.im[1] + C.im[3]); h[4] = -T(0.125) * (C.re[1] - C.re[3]);
+    h[5] = T(0.125) * (C.im[2] + C.im[6]); h[6] = -T(0.125) * (C.re[2] - C.re[6]);
+    h[7] = T(0.125) * (C.im[5] + C.im[7]); h[8] = -T(0.125) * (C.re[5] - C.re[7]);
 }
 
-// Tr(A B) for Hermitian A, B by diagonal and upper entries, in the storage
-// precision (its FP32 inputs already carry FP32 rounding; an FP64 dot made the
-// kernel FP64-bound); the sums over sites run in FP64.
+// Tr(A B) for Hermitian A, B by diagonal and upper entries: sum_jk A_jk
+// conj(B_jk), row by row, in the storage precision (its FP32 inputs already carry
+// FP32 rounding; an FP64 dot made the kernel FP64-bound); the sums over sites run
+// in FP64.
 template <class T>
 __device__ __forceinline__ T tr_herm(const T a[9], const T b[9]) {
-    T s = T(0), o = T(0);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) s = fma(a[k], b[k], s);
-#pragma unroll
-    for (int k = 3; k < 9; ++k) o = fma(a[k], b[k], o);
-    return fma(T(2), o, s);
+    const T o01 = fma(a[3], b[3], a[4] * b[4]), o02 = fma(a[5], b[5], a[6] * b[6]), o12 = fma(a[7], b[7], a[8] * b[8]);
+    T s = a[0] * b[0];
+    s += o01;
+    s += o02;
+    s += o01;
+    s += a[1] * b[1];
+    s += o12;
+    s += o02;
+    s += o12;
+    s += a[2] * b[2];
+    return s;
 }
 
 template <class T, int NC>

@@ -83,8 +83,8 @@ struct RowUnit {
     int f0, f1, s1, s2;     // shifts along nu: the sites whose nu-link is one and two steps out, and s, 2s
 };
 
-// The six or fewer units u = u0, u0 + du, ... < 6 of link (x, mu) for row r:
-// rows of the sums sig and F of the one-pass form
+// The units u = u0, u0 + du, ... (UNITS of them) of link (x, mu) for row r added
+// to the rows of the sums sig and F of the one-pass form
 //   Sigma = c1 F U_mu^dag(x+mu) + sum [c1 U_mu^dag(x-mu) G H B + c0 A B + c1 A T0 T1 T2] C
 // (without rectangles sig = sum A B C, unscaled).
 template <bool RECT, int UNITS>
@@ -149,7 +149,7 @@ __device__ __forceinline__ int part_comp(int n, int u) { return US == 1 ? n : n 
 // Shared memory of a block, [..][link].
 template <int US, int LPB>
 struct RowShared {
-    double part[3][6 * US][LPB];   // partial rows of the lanes, then whole rows
+    double part[3][US == 1 ? 12 : 6 * US][LPB];   // partial rows of the lanes, then whole rows
     double om[18][LPB];            // Omega
     double hf[15][LPB];            // H (diagonal, upper entries) and the exponential's coefficients
     double2 un[9][LPB];            // the candidate
@@ -243,13 +243,35 @@ __device__ __forceinline__ void rows_block(const SubsweepParams &a, int mu, int 
     Row sig = {{0, 0, 0}, {0, 0, 0}}, F = sig;
     if (work) {
         if (a.colour >= 0)
-            x = mu == 0 ? class_site<0>(g, a.colour, t) : mu == 1 ? class_site<1>(g, a.colour, t)
-              : mu == 2 ? class_site<2>(g, a.colour, t) : class_site<3>(g, a.colour, t);
+            x = class_site(g, mu, a.colour, t);
         else
-            x = mu & 1 ? dir_site<1>(g, t) : dir_site<0>(g, t);
+            x = dir_site(g, mu, t);
         i = sidx(g, x);
-        // one lane per row: units in order; two: the signs; six: one unit each
-        row_units<RECT, 6 / US>(g, Us, x, i, mu, u, US, r, a.c0, a.c1, sig, F);
+    }
+    dep_wait();
+    if (work) {
+        if constexpr (US == 1) {
+            // the forward units, then the backward ones on their own: the sum that
+            // two lanes per row form, bit for bit, so that a launch can mix both
+#pragma unroll 1
+            for (int h = 0; h < 2; ++h) {
+                row_units<RECT, 3>(g, Us, x, i, mu, h, 2, r, a.c0, a.c1, sig, F);
+#pragma unroll
+                for (int j = 0; j < 3; ++j) {
+                    if (h == 0) {
+                        buf[j][l] = sig.re[j]; buf[3 + j][l] = sig.im[j];
+                        buf[6 + j][l] = F.re[j]; buf[9 + j][l] = F.im[j];
+                        sig.re[j] = sig.im[j] = F.re[j] = F.im[j] = 0;
+                    } else {
+                        sig.re[j] += buf[j][l]; sig.im[j] += buf[3 + j][l];
+                        F.re[j] += buf[6 + j][l]; F.im[j] += buf[9 + j][l];
+                    }
+                }
+            }
+        } else {
+            // two lanes: the signs; six: one unit each
+            row_units<RECT, 6 / US>(g, Us, x, i, mu, u, US, r, a.c0, a.c1, sig, F);
+        }
     }
     // From here on idle lanes compute on the link at position 0 and write
     // nothing, so that every barrier sees the whole block.
@@ -365,20 +387,22 @@ __device__ __forceinline__ void rows_block(const SubsweepParams &a, int mu, int 
     }
 }
 
-// Class launch (or every link of direction mu, colour < 0): blocks below n_whole
-// take 42 links with a lane per row, the rest of the links go to blocks with US
-// lanes per row (21 links for 2, 7 for 6), so that the last, partial layer of
-// blocks over the SMs is as short as it can be.
-template <bool RECT, int US>
+// Class launch (or every link of direction mu, colour < 0).  WHOLE: blocks below
+// n_whole take 42 links with a lane per row, the rest of the links go to blocks of
+// 21 with two lanes per row, so that the last, partial layer of blocks over the SMs
+// is short.  Otherwise blocks of 7 links with six lanes per row (n_whole = 0).
+template <bool RECT, bool WHOLE>
 __global__ void __launch_bounds__(kRowThreads, 3) k_subsweep_rows(SubsweepParams a, int mu, int n_whole) {
+    constexpr int US = WHOLE ? 2 : 6;
     constexpr size_t s1 = sizeof(RowShared<1, row_links(1)>), s2 = sizeof(RowShared<US, row_links(US)>);
-    __shared__ __align__(16) unsigned char shared[s1 > s2 ? s1 : s2];
+    __shared__ __align__(16) unsigned char shared[WHOLE && s1 > s2 ? s1 : s2];
     const int b = blockIdx.x;
-    if (b < n_whole) {
-        rows_block<RECT, 1>(a, mu, b * row_links(1), a.n_threads, shared);
-    } else {
-        rows_block<RECT, US>(a, mu, n_whole * row_links(1) + (b - n_whole) * row_links(US), a.n_threads, shared);
-    }
+    if constexpr (WHOLE)
+        if (b < n_whole) {
+            rows_block<RECT, 1>(a, mu, b * row_links(1), a.n_threads, shared);
+            return;
+        }
+    rows_block<RECT, US>(a, mu, n_whole * row_links(1) + (b - n_whole) * row_links(US), a.n_threads, shared);
 }
 
 }  // namespace vs

@@ -337,15 +337,39 @@ __device__ __forceinline__ M3<T> stout_candidate(const M3<T> &sig, const M3<T> &
     return m3_mul(Mx, Ux);
 }
 
-// Threads of the plain-load kernels (FP64, and FP32 APE on plaquette staples).  128
-// and not 256: an FP64 thread holds up to 255 registers, two blocks of 128 fit an SM
+// Threads of the plain-load FP64 kernels.  128 and not 256: an FP64 thread holds up to 255 registers, two blocks of 128 fit an SM
 // as one of 256 does, and the last, partial layer of blocks is half as long.
 #ifndef VS_SUBSWEEP_THREADS
 #define VS_SUBSWEEP_THREADS 128
 #endif
-#ifndef VS_SUBSWEEP_MINB
-#define VS_SUBSWEEP_MINB (512 / VS_SUBSWEEP_THREADS)
-#endif
+
+// Class launches depend on the one before them.  With programmatic stream
+// serialisation a launch comes onto the SMs while the previous one drains and
+// waits there (dep_wait) for it to complete before it reads a link or a label; it
+// lets its own successor in only after that, so that no more than two launches
+// share the SMs (earlier, blocks of several launches pile up on some SMs: 41 us
+// instead of 16 for a launch of 81 blocks).  Without it a launch costs ~3 us more:
+// 1024 links 8.2 -> 5.5 us (plaquette staples 6.2 -> 2.9), 165,888 links 71.3 ->
+// 68.7, 524,288 links 165.7 -> 163.4 (88.7 -> 85.6).
+__device__ __forceinline__ void dep_wait() {
+    asm volatile("griddepcontrol.wait;\n griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <class... A, class... B>
+cudaError_t launch_dependent(void (*kernel)(A...), int blocks, int threads, size_t smem, cudaStream_t st, B... args) {
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3(blocks);
+    c.blockDim = dim3(threads);
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    count_launches(1);
+    return cudaLaunchKernelEx(&c, kernel, static_cast<A>(args)...);
+}
 
 // Outcome of one link update, for the per-sweep counters.
 template <class T>
@@ -383,8 +407,8 @@ __device__ __forceinline__ void vp_decide(bool vp, bool want_sine, int ref, T tr
 
 // Stout candidate for link (x, MU) at plane position i from its staple sum,
 // vortex-preservation test against the reference label, store if accepted.
-template <class T, int NC, int MU>
-__device__ __forceinline__ void stout_store(const SubsweepParams &a, const Pt &x, int i, const M3<T> &sig,
+template <class T, int NC>
+__device__ __forceinline__ void stout_store(const SubsweepParams &a, int MU, const Pt &x, int i, const M3<T> &sig,
                                             const M3<T> &Ux, Update<T> &u) {
     const Geo &g = a.g;
     const T rho = sizeof(T) == 4 ? T(a.rho_f) : T(a.rho);
@@ -511,12 +535,12 @@ __global__ void __launch_bounds__(VS_SUBSWEEP_THREADS) k_subsweep(SubsweepParams
     Update<double> u;
     if (active) {
         const Geo &g = a.g;
-        Pt x = a.colour >= 0 ? class_site<MU>(g, a.colour, t) : dir_site<MU>(g, t);
+        Pt x = a.colour >= 0 ? class_site(g, MU, a.colour, t) : dir_site(g, MU, t);
         const int i = sidx(g, x);
         const double *Us = static_cast<const double *>(a.Usrc);
         M3<double> sig = staple_sum<double, 18, false, MU>(g, Us, x, a.c0, a.c1);
         M3<double> Ux = load_link<double, 18>(Us, g.P, MU, i);
-        stout_store<double, 18, MU>(a, x, i, sig, Ux, u);
+        stout_store<double, 18>(a, MU, x, i, sig, Ux, u);
     }
     count_update<double>(a.counters, u);
 }
@@ -537,7 +561,7 @@ __global__ void __launch_bounds__(VS_SUBSWEEP_THREADS) k_subsweep(SubsweepParams
 #define VS_RING_MINB (384 / VS_RING_THREADS)
 #endif
 
-template <int NC>
+template <int NC, int BT = VS_RING_THREADS>   // BT: threads of the block
 struct LinkRing {
     const float4 *v4;   // this thread's column of the float4 slots [depth][NC/4][BT]
     const float2 *v2;   // and of the float2 slots [depth][BT] (NC == 18)
@@ -546,27 +570,27 @@ struct LinkRing {
 
 // Start the copy of the link at site position i of the direction whose
 // links begin at base into slot SLOT, as one commit group.
-template <int NC, int SLOT>
-__device__ __forceinline__ void ring_fetch(const LinkRing<NC> &R, const float *base, long long P, int i) {
+template <int NC, int SLOT, int BT>
+__device__ __forceinline__ void ring_fetch(const LinkRing<NC, BT> &R, const float *base, long long P, int i) {
     constexpr int NQ = NC / 4;
     const float *b0 = base + blk_off4<NC>(i);
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
         const float4 *src = reinterpret_cast<const float4 *>(b0 + 64 * q);
-        const uint32_t dst = R.a4 + (uint32_t)((SLOT * NQ + q) * VS_RING_THREADS * 16);
+        const uint32_t dst = R.a4 + (uint32_t)((SLOT * NQ + q) * BT * 16);
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
     }
     if (NC == 18) {
         const float2 *src = reinterpret_cast<const float2 *>(base + blk_off2(i));
-        const uint32_t dst = R.a2 + (uint32_t)(SLOT * VS_RING_THREADS * 8);
+        const uint32_t dst = R.a2 + (uint32_t)(SLOT * BT * 8);
         asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(dst), "l"(src) : "memory");
     }
     asm volatile("cp.async.commit_group;\n" ::: "memory");
 }
 
 // ring_fetch with a predicate: on == false commits an empty group.
-template <int NC, int SLOT>
-__device__ __forceinline__ void ring_fetch_if(const LinkRing<NC> &R, const float *base, long long P, int i,
+template <int NC, int SLOT, int BT>
+__device__ __forceinline__ void ring_fetch_if(const LinkRing<NC, BT> &R, const float *base, long long P, int i,
                                               bool on) {
     constexpr int NQ = NC / 4;
     const int pr = on ? 1 : 0;
@@ -574,7 +598,7 @@ __device__ __forceinline__ void ring_fetch_if(const LinkRing<NC> &R, const float
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
         const float4 *src = reinterpret_cast<const float4 *>(b0 + 64 * q);
-        const uint32_t dst = R.a4 + (uint32_t)((SLOT * NQ + q) * VS_RING_THREADS * 16);
+        const uint32_t dst = R.a4 + (uint32_t)((SLOT * NQ + q) * BT * 16);
         asm volatile(
             "{\n .reg .pred p;\n setp.ne.b32 p, %2, 0;\n"
             " @p cp.async.cg.shared.global [%0], [%1], 16;\n}\n" ::"r"(dst), "l"(src), "r"(pr)
@@ -582,7 +606,7 @@ __device__ __forceinline__ void ring_fetch_if(const LinkRing<NC> &R, const float
     }
     if (NC == 18) {
         const float2 *src = reinterpret_cast<const float2 *>(base + blk_off2(i));
-        const uint32_t dst = R.a2 + (uint32_t)(SLOT * VS_RING_THREADS * 8);
+        const uint32_t dst = R.a2 + (uint32_t)(SLOT * BT * 8);
         asm volatile(
             "{\n .reg .pred p;\n setp.ne.b32 p, %2, 0;\n"
             " @p cp.async.ca.shared.global [%0], [%1], 8;\n}\n" ::"r"(dst), "l"(src), "r"(pr)
@@ -598,17 +622,17 @@ __device__ __forceinline__ void ring_skip() { asm volatile("cp.async.commit_grou
 // (cp.async.wait_group) until the copy into that slot is complete.
 // FULL = false: only rows 0-1 are needed (a left factor of a two-row
 // product), so 12-real storage skips rebuilding row 2.
-template <int NC, bool DAG, int SLOT, bool FULL = true>
-__device__ __forceinline__ M3<float> ring_read(const LinkRing<NC> &R) {
+template <int NC, bool DAG, int SLOT, bool FULL = true, int BT>
+__device__ __forceinline__ M3<float> ring_read(const LinkRing<NC, BT> &R) {
     constexpr int NQ = NC / 4;
     M3<float> m;
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
-        const float4 v = R.v4[(SLOT * NQ + q) * VS_RING_THREADS];
+        const float4 v = R.v4[(SLOT * NQ + q) * BT];
         m.re[2 * q] = v.x; m.im[2 * q] = v.y; m.re[2 * q + 1] = v.z; m.im[2 * q + 1] = v.w;
     }
     if (NC == 18) {
-        const float2 v = R.v2[SLOT * VS_RING_THREADS];
+        const float2 v = R.v2[SLOT * BT];
         m.re[8] = v.x; m.im[8] = v.y;
     }
     if (NC == 12 && (FULL || DAG)) rebuild_row2(m);
@@ -630,8 +654,8 @@ __device__ __forceinline__ M3<float> ring_read(const LinkRing<NC> &R) {
 // (slot = entry mod 6, compile-time).
 // ---------------------------------------------------------------------------
 
-template <int NC, bool DAG, int SLOT, bool FULL = true>
-__device__ __forceinline__ M3<float> ring_take6(const LinkRing<NC> &R) {
+template <int NC, bool DAG, int SLOT, bool FULL = true, int BT>
+__device__ __forceinline__ M3<float> ring_take6(const LinkRing<NC, BT> &R) {
     asm volatile("cp.async.wait_group 5;\n" ::: "memory");
     return ring_read<NC, DAG, SLOT, FULL>(R);
 }
@@ -652,12 +676,12 @@ __device__ __forceinline__ void u_link(const Around &A, const float *Umu, const 
 
 // Refill after entry K of unit (nu, s), into slot K mod 6: entry K + 6 of the
 // same unit (the spare entries 10, 11 carry U_mu(x+mu), U_mu(x) in the last
-// unit, nothing otherwise), or entry K - 6 of the next unit: (nu, -1) for
-// s = +1, (next nu, +1) on An for s = -1, nothing after the last.
-template <int NC, int S, int K>
-__device__ __forceinline__ void u_refill(const LinkRing<NC> &R, const float *Umu, const float *Unu,
+// unit if spare is set, nothing otherwise), or entry K - 6 of the next unit:
+// (nu, -1) for s = +1, (next nu, +1) on An for s = -1, nothing after the last.
+template <int NC, int S, int K, int BT>
+__device__ __forceinline__ void u_refill(const LinkRing<NC, BT> &R, const float *Umu, const float *Unu,
                                          const float *Un, long long P, const Around &A, const Around &An,
-                                         bool last) {
+                                         bool last, bool spare) {
     constexpr int SL = K % 6;
     const float *base;
     int pos;
@@ -668,7 +692,7 @@ __device__ __forceinline__ void u_refill(const LinkRing<NC> &R, const float *Umu
         // spare entries: U_mu(x+mu) (K + 6 = 10) and U_mu(x) (11) in the last unit
         const int p = K + 6 == 10 ? A.i0 + A.dmp1 : A.i0;
         if constexpr (S > 0) ring_skip();
-        else ring_fetch_if<NC, SL>(R, Umu, P, p, last);
+        else ring_fetch_if<NC, SL>(R, Umu, P, p, spare);
     } else if constexpr (S > 0) {
         u_link<-1, (K >= 6 ? K - 6 : 0)>(A, Umu, Unu, base, pos);
         ring_fetch<NC, SL>(R, base, P, pos);
@@ -678,24 +702,24 @@ __device__ __forceinline__ void u_refill(const LinkRing<NC> &R, const float *Umu
     }
 }
 
-template <int NC, int S>
-__device__ __forceinline__ void fused_unit(const LinkRing<NC> &R, M3<float> &Facc, M3<float> &sig, float c0,
+template <int NC, int S, int BT>
+__device__ __forceinline__ void fused_unit(const LinkRing<NC, BT> &R, M3<float> &Facc, M3<float> &sig, float c0,
                                            float c1, const M3<float> &Lm, const float *Umu, const float *Unu,
                                            const float *Un, long long P, const Around &A, const Around &An,
-                                           bool last) {
+                                           bool last, bool spare) {
     const M3<float> Af = ring_take6<NC, (S < 0), 0, false>(R);
-    u_refill<NC, S, 0>(R, Umu, Unu, Un, P, A, An, last);
+    u_refill<NC, S, 0>(R, Umu, Unu, Un, P, A, An, last, spare);
     const M3<float> B = ring_take6<NC, false, 1>(R);
-    u_refill<NC, S, 1>(R, Umu, Unu, Un, P, A, An, last);
+    u_refill<NC, S, 1>(R, Umu, Unu, Un, P, A, An, last, spare);
     M3<float> AB;
     m3_mul_2r(AB, Af, B);
     M3<float> X, Y;
     {   // c1 U_mu^dag(x-mu) G H B
         const M3<float> G = ring_take6<NC, (S < 0), 2>(R);
-        u_refill<NC, S, 2>(R, Umu, Unu, Un, P, A, An, last);
+        u_refill<NC, S, 2>(R, Umu, Unu, Un, P, A, An, last, spare);
         m3_mul_2r(X, Lm, G);
         const M3<float> H = ring_take6<NC, false, 3>(R);
-        u_refill<NC, S, 3>(R, Umu, Unu, Un, P, A, An, last);
+        u_refill<NC, S, 3>(R, Umu, Unu, Un, P, A, An, last, spare);
         m3_mul_2r(Y, X, H);
         m3_mul_2r(X, Y, B);
     }
@@ -703,22 +727,22 @@ __device__ __forceinline__ void fused_unit(const LinkRing<NC> &R, M3<float> &Fac
     rebuild_row2(W1);
     {   // F(x) += A B D E
         const M3<float> D = ring_take6<NC, false, 4>(R);
-        u_refill<NC, S, 4>(R, Umu, Unu, Un, P, A, An, last);
+        u_refill<NC, S, 4>(R, Umu, Unu, Un, P, A, An, last, spare);
         m3_mul_2r(X, AB, D);
         const M3<float> E = ring_take6<NC, (S > 0), 5>(R);
-        u_refill<NC, S, 5>(R, Umu, Unu, Un, P, A, An, last);
+        u_refill<NC, S, 5>(R, Umu, Unu, Un, P, A, An, last, spare);
         m3_mul_2r(Y, X, E);
         rebuild_row2(Y);
         m3_acc_f32(Facc, Y);
     }
     {   // A T, T = T0 T1 T2
         const M3<float> T0 = ring_take6<NC, (S < 0), 0, false>(R);
-        u_refill<NC, S, 6>(R, Umu, Unu, Un, P, A, An, last);
+        u_refill<NC, S, 6>(R, Umu, Unu, Un, P, A, An, last, spare);
         const M3<float> T1 = ring_take6<NC, false, 1>(R);
-        u_refill<NC, S, 7>(R, Umu, Unu, Un, P, A, An, last);
+        u_refill<NC, S, 7>(R, Umu, Unu, Un, P, A, An, last, spare);
         m3_mul_2r(X, T0, T1);
         const M3<float> T2 = ring_take6<NC, (S > 0), 2>(R);
-        u_refill<NC, S, 8>(R, Umu, Unu, Un, P, A, An, last);
+        u_refill<NC, S, 8>(R, Umu, Unu, Un, P, A, An, last, spare);
         m3_mul_2r(Y, X, T2);
         rebuild_row2(Y);
         m3_mul_2r(X, Af, Y);
@@ -727,10 +751,10 @@ __device__ __forceinline__ void fused_unit(const LinkRing<NC> &R, M3<float> &Fac
     rebuild_row2(AB);
     m3_lin3_f32(Y, c0, AB, c1, W1, X);   // Yc = c1 (W1 + A T) + c0 A B
     const M3<float> C = ring_take6<NC, (S > 0), 3>(R);
-    u_refill<NC, S, 9>(R, Umu, Unu, Un, P, A, An, last);
+    u_refill<NC, S, 9>(R, Umu, Unu, Un, P, A, An, last, spare);
     m3_madd(sig, Y, C);
-    u_refill<NC, S, 10>(R, Umu, Unu, Un, P, A, An, last);   // spare entries: refills only
-    u_refill<NC, S, 11>(R, Umu, Unu, Un, P, A, An, last);
+    u_refill<NC, S, 10>(R, Umu, Unu, Un, P, A, An, last, spare);   // spare entries: refills only
+    u_refill<NC, S, 11>(R, Umu, Unu, Un, P, A, An, last, spare);
 }
 
 template <int NC, int MU>
@@ -768,8 +792,8 @@ __device__ __forceinline__ M3<float> staple_sum_fused(const Geo &g, const float 
         const int nun = (MU + (j < 3 ? j + 1 : 1)) & 3;
         around_nu(g, x, nun, true, An);
         const float *Un = U + (long long)nun * NC * P;
-        fused_unit<NC, 1>(R, Facc, sig, c0, c1, Lm, Umu, Unu, Un, P, A, An, last);
-        fused_unit<NC, -1>(R, Facc, sig, c0, c1, Lm, Umu, Unu, Un, P, A, An, last);
+        fused_unit<NC, 1>(R, Facc, sig, c0, c1, Lm, Umu, Unu, Un, P, A, An, last, last);
+        fused_unit<NC, -1>(R, Facc, sig, c0, c1, Lm, Umu, Unu, Un, P, A, An, last, last);
         A = An;
         Unu = Un;
     }
@@ -793,8 +817,8 @@ __device__ __forceinline__ M3<float> staple_sum_fused(const Geo &g, const float 
 template <int J>
 __host__ __device__ constexpr int p_entry() { return J == 0 ? 0 : (J == 1 ? 1 : 9); }
 
-template <int NC, int S, int J>
-__device__ __forceinline__ void p_refill(const LinkRing<NC> &R, const float *Umu, const float *Un, long long P,
+template <int NC, int S, int J, int BT>
+__device__ __forceinline__ void p_refill(const LinkRing<NC, BT> &R, const float *Umu, const float *Un, long long P,
                                          const Around &An, bool last) {
     const float *base;
     int pos;
@@ -802,8 +826,8 @@ __device__ __forceinline__ void p_refill(const LinkRing<NC> &R, const float *Umu
     ring_fetch_if<NC, (S < 0 ? 3 : 0) + J>(R, base, P, pos, !last);
 }
 
-template <int NC, int S>
-__device__ __forceinline__ void plain_unit(const LinkRing<NC> &R, M3<float> &sig, const float *Umu,
+template <int NC, int S, int BT>
+__device__ __forceinline__ void plain_unit(const LinkRing<NC, BT> &R, M3<float> &sig, const float *Umu,
                                            const float *Un, long long P, const Around &An, bool last) {
     constexpr int S0 = S < 0 ? 3 : 0;
     const M3<float> Af = ring_take6<NC, (S < 0), S0, false>(R);
@@ -875,15 +899,15 @@ inline void once_per_device(std::atomic<unsigned long long> &done, F &&set) {
     done.fetch_or(bit, std::memory_order_release);
 }
 
-template <int NC>
+template <int NC, int BT = VS_RING_THREADS>
 constexpr int ring6_smem_bytes() {
-    return 6 * VS_RING_THREADS * ((NC / 4) * 16 + (NC == 18 ? 8 : 0));
+    return 6 * BT * ((NC / 4) * 16 + (NC == 18 ? 8 : 0));
 }
 
 // This thread's column of the ring arrays of a kernel.
-template <int NC>
-__device__ __forceinline__ LinkRing<NC> ring_of(float4 *ring4, float2 *ring2) {
-    LinkRing<NC> R;
+template <int NC, int BT = VS_RING_THREADS>
+__device__ __forceinline__ LinkRing<NC, BT> ring_of(float4 *ring4, float2 *ring2) {
+    LinkRing<NC, BT> R;
     R.v4 = ring4 + threadIdx.x;
     R.v2 = ring2 + (NC == 18 ? threadIdx.x : 0);
     R.a4 = (uint32_t)__cvta_generic_to_shared(ring4 + threadIdx.x);
@@ -902,13 +926,14 @@ __global__ void __launch_bounds__(VS_RING_THREADS, 4) k_subsweep_pring(SubsweepP
     Update<float> u;
     if (active) {
         const Geo &g = a.g;
-        Pt x = a.colour >= 0 ? class_site<MU>(g, a.colour, t) : dir_site<MU>(g, t);
+        Pt x = a.colour >= 0 ? class_site(g, MU, a.colour, t) : dir_site(g, MU, t);
         const int i = sidx(g, x);
         const float *Us = static_cast<const float *>(a.Usrc);
         LinkRing<NC> R = ring_of<NC>(ring4, ring2);
+        dep_wait();
         const M3<float> sig = staple_sum_plain_ring<NC, MU>(g, Us, x, a.c0_f, R);
         const M3<float> Ux = load_link<float, NC>(Us, g.P, MU, i);
-        stout_store<float, NC, MU>(a, x, i, sig, Ux, u);
+        stout_store<float, NC>(a, MU, x, i, sig, Ux, u);
     }
     count_update<float>(a.counters, u);
 }
@@ -923,12 +948,13 @@ __global__ void __launch_bounds__(VS_RING_THREADS, VS_RING_MINB) k_subsweep_fuse
     Update<float> u;
     if (active) {
         const Geo &g = a.g;
-        Pt x = a.colour >= 0 ? class_site<MU>(g, a.colour, t) : dir_site<MU>(g, t);
+        Pt x = a.colour >= 0 ? class_site(g, MU, a.colour, t) : dir_site(g, MU, t);
         const int i = sidx(g, x);
         LinkRing<NC> R = ring_of<NC>(ring4, ring2);
+        dep_wait();
         M3<float> Ux;
         M3<float> sig = staple_sum_fused<NC, MU>(g, static_cast<const float *>(a.Usrc), x, a.c0_f, a.c1_f, R, Ux);
-        stout_store<float, NC, MU>(a, x, i, sig, Ux, u);
+        stout_store<float, NC>(a, MU, x, i, sig, Ux, u);
     }
     count_update<float>(a.counters, u);
 }
@@ -994,8 +1020,8 @@ __device__ __forceinline__ void maxretr(M3<T> &u, const M3<T> &Vb, int n_hits) {
 // AUS update of link (x, MU) at plane position i from its staple sum Vb and
 // current value u: blocking V = (1 - alpha) u + (alpha / 6) Vb, MaxReTr,
 // vortex-preservation test, store if accepted.
-template <class T, int NC, int MU>
-__device__ __forceinline__ void aus_finish(const AusParams &a, const Pt &x, int i, M3<T> Vb, M3<T> u,
+template <class T, int NC>
+__device__ __forceinline__ void aus_finish(const AusParams &a, int MU, const Pt &x, int i, M3<T> Vb, M3<T> u,
                                            Update<T> &up) {
     const Geo &g = a.g;
     const T al = sizeof(T) == 4 ? T(a.alpha_f) : T(a.alpha);
@@ -1013,23 +1039,22 @@ __device__ __forceinline__ void aus_finish(const AusParams &a, const Pt &x, int 
     if (!up.reject) store_link<T, NC>(static_cast<T *>(a.U), g.P, MU, i, u);
 }
 
-template <class T, int NC, bool RECT, int MU>
-__global__ void __launch_bounds__(VS_SUBSWEEP_THREADS, sizeof(T) == 4 ? VS_SUBSWEEP_MINB : 1)
-    k_aus(AusParams a) {
+// FP64, one thread per link of the colour class.
+template <bool RECT, int MU>
+__global__ void __launch_bounds__(VS_SUBSWEEP_THREADS) k_aus(AusParams a) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const bool active = t < a.n_threads;
-    Update<T> up;
+    Update<double> up;
     if (active) {
         const Geo &g = a.g;
-        const Pt x = class_site<MU>(g, a.colour, t);
+        const Pt x = class_site(g, MU, a.colour, t);
         const int i = sidx(g, x);
-        const T *U = static_cast<const T *>(a.U);
-        const T c0 = sizeof(T) == 4 ? T(a.c0_f) : T(a.c0), c1 = sizeof(T) == 4 ? T(a.c1_f) : T(a.c1);
-        const M3<T> Vb = staple_sum<T, NC, RECT, MU>(g, U, x, c0, c1);
-        const M3<T> u = load_link<T, NC>(U, g.P, MU, i);
-        aus_finish<T, NC, MU>(a, x, i, Vb, u, up);
+        const double *U = static_cast<const double *>(a.U);
+        const M3<double> Vb = staple_sum<double, 18, RECT, MU>(g, U, x, a.c0, a.c1);
+        const M3<double> u = load_link<double, 18>(U, g.P, MU, i);
+        aus_finish<double, 18>(a, MU, x, i, Vb, u, up);
     }
-    count_update<T>(a.counters, up);
+    count_update<double>(a.counters, up);
 }
 
 // FP32 over-improved AUS with the one-pass link stream of k_subsweep_fused.
@@ -1043,12 +1068,13 @@ __global__ void __launch_bounds__(VS_RING_THREADS, VS_RING_MINB) k_aus_ring(AusP
     Update<float> up;
     if (active) {
         const Geo &g = a.g;
-        const Pt x = class_site<MU>(g, a.colour, t);
+        const Pt x = class_site(g, MU, a.colour, t);
         const int i = sidx(g, x);
         LinkRing<NC> R = ring_of<NC>(ring4, ring2);
+        dep_wait();
         M3<float> Ux;
         const M3<float> Vb = staple_sum_fused<NC, MU>(g, static_cast<const float *>(a.U), x, a.c0_f, a.c1_f, R, Ux);
-        aus_finish<float, NC, MU>(a, x, i, Vb, Ux, up);
+        aus_finish<float, NC>(a, MU, x, i, Vb, Ux, up);
     }
     count_update<float>(a.counters, up);
 }
@@ -1065,15 +1091,37 @@ __global__ void __launch_bounds__(VS_RING_THREADS, 4) k_aus_pring(AusParams a) {
     Update<float> up;
     if (active) {
         const Geo &g = a.g;
-        const Pt x = class_site<MU>(g, a.colour, t);
+        const Pt x = class_site(g, MU, a.colour, t);
         const int i = sidx(g, x);
         const float *Us = static_cast<const float *>(a.U);
         LinkRing<NC> R = ring_of<NC>(ring4, ring2);
+        dep_wait();
         const M3<float> Vb = staple_sum_plain_ring<NC, MU>(g, Us, x, a.c0_f, R);
         const M3<float> Ux = load_link<float, NC>(Us, g.P, MU, i);
-        aus_finish<float, NC, MU>(a, x, i, Vb, Ux, up);
+        aus_finish<float, NC>(a, MU, x, i, Vb, Ux, up);
     }
     count_update<float>(a.counters, up);
+}
+
+// One launch of a thread-per-link FP64 kernel.
+template <class P>
+cudaError_t launch_links(void (*kernel)(P), const P &p, cudaStream_t st) {
+    kernel<<<(p.n_threads + VS_SUBSWEEP_THREADS - 1) / VS_SUBSWEEP_THREADS, VS_SUBSWEEP_THREADS, 0, st>>>(p);
+    count_launches(1);
+    return cudaGetLastError();
+}
+
+// One launch of a link-ring kernel of direction mu out of its four instantiations.
+// attr_set: where the shared-memory limit has been set, one flag per kernel family.
+template <class P>
+cudaError_t launch_ring(void (*const kernels[4])(P), int mu, const P &p, int smem,
+                        std::atomic<unsigned long long> &attr_set, cudaStream_t st) {
+    once_per_device(attr_set, [&] {
+        for (int k = 0; k < 4; ++k)
+            cudaFuncSetAttribute(kernels[k], cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    });
+    return launch_dependent(kernels[mu], (p.n_threads + VS_RING_THREADS - 1) / VS_RING_THREADS, VS_RING_THREADS,
+                            (size_t)smem, st, p);
 }
 
 }  // namespace vs

@@ -4,7 +4,7 @@
 #pragma once
 
 #include "vs_internal.h"
-#include "vs_stout.cuh"
+#include "vs_split.cuh"
 
 namespace vs {
 
@@ -20,119 +20,46 @@ void launch_redecide(int mu, const SubsweepParams &p, cudaStream_t st) {
     count_launches(1);
 }
 
-// FP32 class launches: the cp.async link-ring kernels.
+// FP32 stout class launches.
 template <int NC>
 cudaError_t launch_subsweep_tpl(bool rect, int mu, const SubsweepParams &p, cudaStream_t st) {
     if (p.n_threads <= 0) return cudaSuccess;
-    {
-        if (rect) {
-            const int rb = (p.n_threads + VS_RING_THREADS - 1) / VS_RING_THREADS;
-            constexpr int sm = ring6_smem_bytes<NC>();
-            static std::atomic<unsigned long long> attr_set{0};
-            once_per_device(attr_set, [&] {
-                cudaFuncSetAttribute(k_subsweep_fused<NC, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-                cudaFuncSetAttribute(k_subsweep_fused<NC, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-                cudaFuncSetAttribute(k_subsweep_fused<NC, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-                cudaFuncSetAttribute(k_subsweep_fused<NC, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-            });
-            switch (mu) {
-                case 0: k_subsweep_fused<NC, 0><<<rb, VS_RING_THREADS, sm, st>>>(p); break;
-                case 1: k_subsweep_fused<NC, 1><<<rb, VS_RING_THREADS, sm, st>>>(p); break;
-                case 2: k_subsweep_fused<NC, 2><<<rb, VS_RING_THREADS, sm, st>>>(p); break;
-                default: k_subsweep_fused<NC, 3><<<rb, VS_RING_THREADS, sm, st>>>(p); break;
-            }
-            count_launches(1);
-            if (p.defer_idx) launch_redecide<NC, true>(mu, p, st);
-            return cudaGetLastError();
-        }
-        {   // FP32 plaquette staples (eps = 1): the plaquette-staple link ring
-            const int rb = (p.n_threads + VS_RING_THREADS - 1) / VS_RING_THREADS;
-            constexpr int sm = ring6_smem_bytes<NC>();
-            static std::atomic<unsigned long long> attr_set_p{0};
-            once_per_device(attr_set_p, [&] {
-                cudaFuncSetAttribute(k_subsweep_pring<NC, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-                cudaFuncSetAttribute(k_subsweep_pring<NC, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-                cudaFuncSetAttribute(k_subsweep_pring<NC, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-                cudaFuncSetAttribute(k_subsweep_pring<NC, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-            });
-            switch (mu) {
-                case 0: k_subsweep_pring<NC, 0><<<rb, VS_RING_THREADS, sm, st>>>(p); break;
-                case 1: k_subsweep_pring<NC, 1><<<rb, VS_RING_THREADS, sm, st>>>(p); break;
-                case 2: k_subsweep_pring<NC, 2><<<rb, VS_RING_THREADS, sm, st>>>(p); break;
-                default: k_subsweep_pring<NC, 3><<<rb, VS_RING_THREADS, sm, st>>>(p); break;
-            }
-            count_launches(1);
-            if (p.defer_idx) launch_redecide<NC, false>(mu, p, st);
-            return cudaGetLastError();
-        }
+    cudaError_t e;
+    if (split_launch(rect, p.n_threads)) {
+        static void (*const kernels[2])(SubsweepParams, int) = {k_subsweep_split<NC, false>, k_subsweep_split<NC, true>};
+        static std::atomic<unsigned long long> set{0};
+        e = launch_split<NC>(kernels, rect, mu, p, set, st);
+    } else {
+        static void (*const kernels[2][4])(SubsweepParams) = {
+            {k_subsweep_pring<NC, 0>, k_subsweep_pring<NC, 1>, k_subsweep_pring<NC, 2>, k_subsweep_pring<NC, 3>},
+            {k_subsweep_fused<NC, 0>, k_subsweep_fused<NC, 1>, k_subsweep_fused<NC, 2>, k_subsweep_fused<NC, 3>}};
+        static std::atomic<unsigned long long> set[2] = {{0}, {0}};
+        e = launch_ring(kernels[rect], mu, p, ring6_smem_bytes<NC>(), set[rect], st);
     }
+    if (e == cudaSuccess && p.defer_idx) {
+        if (rect) launch_redecide<NC, true>(mu, p, st);
+        else launch_redecide<NC, false>(mu, p, st);
+    }
+    return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
 template <class T, int NC>
 cudaError_t launch_aus_tpl(bool rect, int mu, const AusParams &p, cudaStream_t st) {
     if (p.n_threads <= 0) return cudaSuccess;
-    if constexpr (sizeof(T) == 4) {
-        // FP32: the link-ring kernels
-        if (rect) {
-            const int rb = (p.n_threads + VS_RING_THREADS - 1) / VS_RING_THREADS;
-            constexpr int sm = ring6_smem_bytes<NC>();
-            static std::atomic<unsigned long long> attr_set{0};
-            once_per_device(attr_set, [&] {
-                cudaFuncSetAttribute(k_aus_ring<NC, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-                cudaFuncSetAttribute(k_aus_ring<NC, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-                cudaFuncSetAttribute(k_aus_ring<NC, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-                cudaFuncSetAttribute(k_aus_ring<NC, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-            });
-            switch (mu) {
-                case 0: k_aus_ring<NC, 0><<<rb, VS_RING_THREADS, sm, st>>>(p); break;
-                case 1: k_aus_ring<NC, 1><<<rb, VS_RING_THREADS, sm, st>>>(p); break;
-                case 2: k_aus_ring<NC, 2><<<rb, VS_RING_THREADS, sm, st>>>(p); break;
-                default: k_aus_ring<NC, 3><<<rb, VS_RING_THREADS, sm, st>>>(p); break;
-            }
-            count_launches(1);
-            return cudaGetLastError();
-        }
-        {   // FP32 plaquette staples (cooling and eps = 1 AUS): the plaquette-staple ring
-            const int rb = (p.n_threads + VS_RING_THREADS - 1) / VS_RING_THREADS;
-            constexpr int sm = ring6_smem_bytes<NC>();
-            static std::atomic<unsigned long long> attr_set_p{0};
-            once_per_device(attr_set_p, [&] {
-                cudaFuncSetAttribute(k_aus_pring<NC, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-                cudaFuncSetAttribute(k_aus_pring<NC, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-                cudaFuncSetAttribute(k_aus_pring<NC, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-                cudaFuncSetAttribute(k_aus_pring<NC, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-            });
-            switch (mu) {
-                case 0: k_aus_pring<NC, 0><<<rb, VS_RING_THREADS, sm, st>>>(p); break;
-                case 1: k_aus_pring<NC, 1><<<rb, VS_RING_THREADS, sm, st>>>(p); break;
-                case 2: k_aus_pring<NC, 2><<<rb, VS_RING_THREADS, sm, st>>>(p); break;
-                default: k_aus_pring<NC, 3><<<rb, VS_RING_THREADS, sm, st>>>(p); break;
-            }
-            count_launches(1);
-            return cudaGetLastError();
-        }
+    if constexpr (sizeof(T) == 8) {
+        static void (*const kernels[2][4])(AusParams) = {{k_aus<false, 0>, k_aus<false, 1>, k_aus<false, 2>, k_aus<false, 3>},
+                                                         {k_aus<true, 0>, k_aus<true, 1>, k_aus<true, 2>, k_aus<true, 3>}};
+        return launch_links(kernels[rect][mu], p, st);
+    } else if (split_launch(rect, p.n_threads)) {
+        static void (*const kernels[2])(AusParams, int) = {k_aus_split<NC, false>, k_aus_split<NC, true>};
+        static std::atomic<unsigned long long> set{0};
+        return launch_split<NC>(kernels, rect, mu, p, set, st);
     } else {
-        const int threads = VS_SUBSWEEP_THREADS;
-        const int blocks = (p.n_threads + threads - 1) / threads;
-#define VS_LAUNCH(R, M) k_aus<T, NC, R, M><<<blocks, threads, 0, st>>>(p)
-        if (rect) {
-            switch (mu) {
-                case 0: VS_LAUNCH(true, 0); break;
-                case 1: VS_LAUNCH(true, 1); break;
-                case 2: VS_LAUNCH(true, 2); break;
-                default: VS_LAUNCH(true, 3); break;
-            }
-        } else {
-            switch (mu) {
-                case 0: VS_LAUNCH(false, 0); break;
-                case 1: VS_LAUNCH(false, 1); break;
-                case 2: VS_LAUNCH(false, 2); break;
-                default: VS_LAUNCH(false, 3); break;
-            }
-        }
-#undef VS_LAUNCH
-        count_launches(1);
-        return cudaGetLastError();
+        static void (*const kernels[2][4])(AusParams) = {
+            {k_aus_pring<NC, 0>, k_aus_pring<NC, 1>, k_aus_pring<NC, 2>, k_aus_pring<NC, 3>},
+            {k_aus_ring<NC, 0>, k_aus_ring<NC, 1>, k_aus_ring<NC, 2>, k_aus_ring<NC, 3>}};
+        static std::atomic<unsigned long long> set[2] = {{0}, {0}};
+        return launch_ring(kernels[rect], mu, p, ring6_smem_bytes<NC>(), set[rect], st);
     }
 }
 

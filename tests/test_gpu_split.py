@@ -1,0 +1,48 @@
+"""FP32 smoothers on both sides of the size at which a class launch changes from three warps per
+32 links to a thread per link: one sweep of a general SU(3) field against the oracle.
+
+Links per class launch (the flow: sites per stage launch, four times as many): 512, 12,288 (the
+last plaquette-staple launch of three warps), 16,384, 32,768 (the last over-improved one) and
+36,864.  Tolerances are those of the same one-sweep comparisons on small lattices: 1e-6 for stout,
+3e-6 for UCP and the flow (2e-6) and for AUS in 12-real storage, which rebuilds row 2 on each load."""
+
+import numpy as np
+import pytest
+
+import oracle as O
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def env():
+    from paper_2203_09764_gb300 import vs
+    ctx = vs.vs_create(0)
+    yield vs, ctx
+    vs.vs_destroy(ctx)
+
+
+@pytest.mark.parametrize("eps", [-0.25, 1.0])
+@pytest.mark.parametrize("storage", [18, 12])
+@pytest.mark.parametrize("dims", [(8, 4, 8, 8), (16, 16, 16, 12), (16, 16, 16, 16), (16, 16, 16, 32), (16, 16, 16, 36)])
+def test_one_sweep_on_both_sides_of_the_split(env, dims, storage, eps):
+    vs, ctx = env
+    U0 = O.cool(dims, synth.haar_field(dims, 3), 1)
+    f = vs.vs_field_create(ctx, dims, vs.VS_FP32, vs.VS_LINK12 if storage == 12 else vs.VS_LINK18)
+    runs = [
+        (lambda: vs.vs_smooth(f, 1, 0.06, eps, vortex_preserve=False, reunit_every=0),
+         lambda: O.smooth(dims, U0, None, 1, 0.06, eps=eps, vp=False)[0], 1e-6),
+        (lambda: vs.vs_smooth_aus(f, 1, 0.02, eps, vortex_preserve=False, reunit_every=0),
+         lambda: O.aus(dims, U0, None, 1, 0.02, eps=eps, vp=False)[0], 2e-6),
+        (lambda: vs.vs_smooth_ape(f, 1, 0.02, eps, vortex_preserve=False, reunit_every=0),
+         lambda: O.ape_ucp(dims, U0, None, 1, 0.02, eps=eps, vp=False)[0], 3e-6),
+    ]
+    if int(np.prod(dims)) <= 16 ** 4:
+        runs.append((lambda: vs.vs_flow_rk3(f, 1, 0.02, eps, reunit_every=0),
+                     lambda: O.flow_rk3(dims, U0, 1, 0.02, eps=eps), 2e-6))
+    for gpu, cpu, tol in runs:
+        vs.vs_load_field(f, links=U0)
+        gpu()
+        assert np.abs(vs.vs_read_field(f) - cpu()).max() < tol
+    vs.vs_field_destroy(f)
