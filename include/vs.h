@@ -73,7 +73,9 @@ typedef struct {
     vs_alloc_fn alloc;          /* NULL: cudaMalloc */
     vs_free_fn free_fn;         /* NULL: cudaFree */
     void *alloc_user;
-    uint64_t hbm_budget_bytes;  /* serving admission cap on device bytes; 0 = no cap */
+    uint64_t hbm_budget_bytes;  /* serving admission cap on device bytes; 0 = no cap.  Without allocator
+                                   hooks the blocks of finished jobs are kept, within the cap, for the next
+                                   jobs, and freed when the loop has been idle for 100 ms */
     int32_t max_slots;          /* serving: jobs on the device at once; 0 -> 8 */
     int32_t max_queue;          /* serving: waiting jobs before VS_EBUSY; 0 -> 1024 */
 } vs_options;

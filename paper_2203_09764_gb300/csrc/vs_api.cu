@@ -52,7 +52,11 @@ void *vs::dev_alloc(vs_ctx *c, size_t bytes) {
     void *p = nullptr;
     if (cudaMalloc(&p, bytes) != cudaSuccess) {
         cudaGetLastError();
-        return nullptr;
+        c->pool.trim();     // idle blocks of the serving loop
+        if (cudaMalloc(&p, bytes) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
     }
     return p;
 }
@@ -61,6 +65,76 @@ void vs::dev_free(vs_ctx *c, void *p) {
     if (!p) return;
     if (c->opt.free_fn) c->opt.free_fn(p, c->opt.alloc_user);
     else cudaFree(p);
+}
+
+bool DevicePool::empty() {
+    std::lock_guard<std::mutex> g(mu);
+    return idle.empty();
+}
+
+void *DevicePool::take(size_t bytes) {
+    std::lock_guard<std::mutex> g(mu);
+    auto it = idle.find(bytes);
+    if (it != idle.end()) {
+        void *p = it->second;
+        idle.erase(it);
+        idle_bytes -= bytes;
+        return p;
+    }
+    void *p = nullptr;
+    if (cudaMalloc(&p, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        for (auto &b : idle) {
+            size.erase(b.second);
+            cudaFree(b.second);
+        }
+        idle.clear();
+        idle_bytes = 0;
+        if (cudaMalloc(&p, bytes) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+    }
+    size[p] = bytes;
+    return p;
+}
+
+void DevicePool::give(void *p) {
+    if (!p) return;
+    std::lock_guard<std::mutex> g(mu);
+    const size_t n = size[p];
+    idle.emplace(n, p);
+    idle_bytes += n;
+}
+
+void DevicePool::trim() {
+    std::lock_guard<std::mutex> g(mu);
+    for (auto &b : idle) {
+        size.erase(b.second);
+        cudaFree(b.second);
+    }
+    idle.clear();
+    idle_bytes = 0;
+}
+
+void DevicePool::make_room(const size_t *sizes, int n, uint64_t others, uint64_t budget) {
+    std::lock_guard<std::mutex> g(mu);
+    std::map<size_t, size_t> keep;     // of each size, how many idle blocks the field takes
+    size_t kept = 0;
+    for (int k = 0; k < n; ++k)
+        if (keep[sizes[k]] < idle.count(sizes[k])) {
+            ++keep[sizes[k]];
+            kept += sizes[k];
+        }
+    for (auto it = idle.end(); it != idle.begin() && others + (idle_bytes - kept) > budget;) {
+        --it;
+        const size_t bytes = it->first;
+        if (idle.count(bytes) <= keep[bytes]) continue;
+        size.erase(it->second);
+        cudaFree(it->second);
+        idle_bytes -= bytes;
+        it = idle.erase(it);
+    }
 }
 
 extern "C" vs_status vs_create(const vs_options *opt, vs_ctx **out) {
@@ -121,15 +195,40 @@ bool vs::valid_dims(const int32_t d[4]) {
     return true;
 }
 
+int vs::field_block_sizes(const int32_t dims[4], int32_t precision, int32_t storage, size_t sizes[kFieldBlocks]) {
+    const size_t P = (size_t)make_geo(dims).P;   // plane stride, with the layout's unused positions
+    const int nc = storage == VS_LINK12 ? 12 : 18;
+    sizes[0] = 4 * nc * P * (precision == VS_FP64 ? 8 : 4);
+    sizes[1] = sizes[2] = 4 * P;
+    sizes[3] = kPartials * sizeof(double) + 256;
+    sizes[4] = kDeferCap * sizeof(int);
+    return precision == VS_FP32 ? 5 : 4;
+}
+
 uint64_t vs::field_footprint(const int32_t dims[4], int32_t precision, int32_t storage) {
-    const long long P = make_geo(dims).P;   // plane stride, with the layout's unused positions
-    int nc = storage == VS_LINK12 ? 12 : 18;
-    uint64_t links = (uint64_t)4 * nc * P * (precision == VS_FP64 ? 8 : 4);
-    return links + 8ull * P + kPartials * 8 + 256 + (precision == VS_FP32 ? kDeferCap * sizeof(int) : 0);
+    size_t sizes[kFieldBlocks];
+    const int n = field_block_sizes(dims, precision, storage, sizes);
+    uint64_t sum = 0;
+    for (int k = 0; k < n; ++k) sum += sizes[k];
+    return sum;
+}
+
+static void *field_alloc(vs_field *f, size_t bytes) {
+    return f->pool ? f->pool->take(bytes) : dev_alloc(f->ctx, bytes);
+}
+
+static void field_free(vs_field *f, void *p) {
+    if (f->pool) f->pool->give(p);
+    else dev_free(f->ctx, p);
 }
 
 extern "C" vs_status vs_field_create(vs_ctx *c, const int32_t dims[4], int32_t precision, int32_t storage,
                                      void *stream, vs_field **out) {
+    return field_create(c, dims, precision, storage, stream, nullptr, out);
+}
+
+vs_status vs::field_create(vs_ctx *c, const int32_t dims[4], int32_t precision, int32_t storage, void *stream,
+                           DevicePool *pool, vs_field **out) {
     if (!c || !dims || !out) return fail(VS_EINVAL, "vs_field_create: NULL argument");
     *out = nullptr;
     if (!valid_dims(dims))
@@ -144,6 +243,7 @@ extern "C" vs_status vs_field_create(vs_ctx *c, const int32_t dims[4], int32_t p
     vs_field *f = new (std::nothrow) vs_field();
     if (!f) return fail(VS_ENOMEM, "vs_field_create: out of host memory");
     f->ctx = c;
+    f->pool = pool;
     f->prec = precision;
     f->nc = storage == VS_LINK12 ? 12 : 18;
     f->g = make_geo(dims);
@@ -154,11 +254,13 @@ extern "C" vs_status vs_field_create(vs_ctx *c, const int32_t dims[4], int32_t p
         if (e != cudaSuccess) { delete f; return cuda_fail(e, "cudaStreamCreate"); }
         f->own_stream = true;
     }
-    f->U = dev_alloc(c, field_bytes(f));
-    f->ref = (int8_t *)dev_alloc(c, 4 * (size_t)f->g.P);
-    f->cur = (int8_t *)dev_alloc(c, 4 * (size_t)f->g.P);
-    f->partials = (double *)dev_alloc(c, kPartials * sizeof(double) + 256);
-    if (precision == VS_FP32) f->defer_idx = (int *)dev_alloc(c, kDeferCap * sizeof(int));
+    size_t sizes[kFieldBlocks];
+    field_block_sizes(dims, precision, storage, sizes);
+    f->U = field_alloc(f, sizes[0]);
+    f->ref = (int8_t *)field_alloc(f, sizes[1]);
+    f->cur = (int8_t *)field_alloc(f, sizes[2]);
+    f->partials = (double *)field_alloc(f, sizes[3]);
+    if (precision == VS_FP32) f->defer_idx = (int *)field_alloc(f, sizes[4]);
     if (!f->U || !f->ref || !f->cur || !f->partials || (precision == VS_FP32 && !f->defer_idx)) {
         vs_field_destroy(f);
         return fail(VS_ENOMEM, "vs_field_create: device allocation of %zu bytes failed", field_bytes(f));
@@ -181,16 +283,16 @@ extern "C" void vs_field_destroy(vs_field *f) {
     if (!f) return;
     cudaSetDevice(f->ctx->opt.device);
     if (f->stream) cudaStreamSynchronize(f->stream);
-    dev_free(f->ctx, f->U);
-    dev_free(f->ctx, f->ref);
-    dev_free(f->ctx, f->cur);
-    dev_free(f->ctx, f->G);
-    dev_free(f->ctx, f->partials);
-    dev_free(f->ctx, f->defer_idx);
-    dev_free(f->ctx, f->scratch);
-    dev_free(f->ctx, f->flowS);
-    dev_free(f->ctx, f->sweep_counts);
-    dev_free(f->ctx, f->sweep_actions);
+    field_free(f, f->U);
+    field_free(f, f->ref);
+    field_free(f, f->cur);
+    field_free(f, f->G);
+    field_free(f, f->partials);
+    field_free(f, f->defer_idx);
+    field_free(f, f->scratch);
+    field_free(f, f->flowS);
+    field_free(f, f->sweep_counts);
+    field_free(f, f->sweep_actions);
     for (auto &e : f->events) cudaEventDestroy(e);
     if (f->own_stream && f->stream) cudaStreamDestroy(f->stream);
     delete f;
@@ -199,8 +301,8 @@ extern "C" void vs_field_destroy(vs_field *f) {
 static vs_status ensure_scratch(vs_field *f, size_t bytes) {
     if (f->scratch_bytes >= bytes) return VS_OK;
     CK(cudaStreamSynchronize(f->stream));
-    dev_free(f->ctx, f->scratch);
-    f->scratch = dev_alloc(f->ctx, bytes);
+    field_free(f, f->scratch);
+    f->scratch = field_alloc(f, bytes);
     f->scratch_bytes = f->scratch ? bytes : 0;
     if (!f->scratch) return fail(VS_ENOMEM, "scratch allocation of %zu bytes failed", bytes);
     return VS_OK;
@@ -454,7 +556,7 @@ extern "C" vs_status vs_gauge_transform(vs_field *f, const double *G, int32_t wh
     CK(cudaSetDevice(f->ctx->opt.device));
     const size_t V = f->g.V;
     if (!f->G) {
-        f->G = dev_alloc(f->ctx, (size_t)f->g.P * 18 * (f->prec == VS_FP64 ? 8 : 4));
+        f->G = field_alloc(f, (size_t)f->g.P * 18 * (f->prec == VS_FP64 ? 8 : 4));
         if (!f->G) return fail(VS_ENOMEM, "vs_gauge_transform: allocation failed");
     }
     const double *src = G;
@@ -606,10 +708,10 @@ vs_status vs::smooth_enqueue(vs_field *f, int32_t n_sweeps, double rho, double e
     // per-sweep device counters and actions
     if (want_stats && f->sweep_cap < n_sweeps) {
         CK(cudaStreamSynchronize(f->stream));
-        dev_free(f->ctx, f->sweep_counts);
-        dev_free(f->ctx, f->sweep_actions);
-        f->sweep_counts = (unsigned long long *)dev_alloc(f->ctx, kSweepSlots * sizeof(unsigned long long) * n_sweeps);
-        f->sweep_actions = (double *)dev_alloc(f->ctx, sizeof(double) * n_sweeps);
+        field_free(f, f->sweep_counts);
+        field_free(f, f->sweep_actions);
+        f->sweep_counts = (unsigned long long *)field_alloc(f, kSweepSlots * sizeof(unsigned long long) * n_sweeps);
+        f->sweep_actions = (double *)field_alloc(f, sizeof(double) * n_sweeps);
         if (!f->sweep_counts || !f->sweep_actions) {
             f->sweep_cap = 0;
             return fail(VS_ENOMEM, "vs_smooth: stats allocation failed");
@@ -722,10 +824,10 @@ extern "C" vs_status vs_smooth_aus(vs_field *f, int32_t n_sweeps, double alpha, 
     const int p = f->prec == VS_FP32;
     if (stats && f->sweep_cap < n_sweeps) {
         CK(cudaStreamSynchronize(f->stream));
-        dev_free(f->ctx, f->sweep_counts);
-        dev_free(f->ctx, f->sweep_actions);
-        f->sweep_counts = (unsigned long long *)dev_alloc(f->ctx, kSweepSlots * sizeof(unsigned long long) * n_sweeps);
-        f->sweep_actions = (double *)dev_alloc(f->ctx, sizeof(double) * n_sweeps);
+        field_free(f, f->sweep_counts);
+        field_free(f, f->sweep_actions);
+        f->sweep_counts = (unsigned long long *)field_alloc(f, kSweepSlots * sizeof(unsigned long long) * n_sweeps);
+        f->sweep_actions = (double *)field_alloc(f, sizeof(double) * n_sweeps);
         if (!f->sweep_counts || !f->sweep_actions) {
             f->sweep_cap = 0;
             return fail(VS_ENOMEM, "vs_smooth_aus: stats allocation failed");
@@ -782,10 +884,10 @@ static cudaError_t flow_launch(vs_field *f, bool rect, int mu, const FlowParams 
 static vs_status ensure_sweep_counts(vs_field *f, int32_t n, const char *who) {
     if (f->sweep_cap >= n) return VS_OK;
     CK(cudaStreamSynchronize(f->stream));
-    dev_free(f->ctx, f->sweep_counts);
-    dev_free(f->ctx, f->sweep_actions);
-    f->sweep_counts = (unsigned long long *)dev_alloc(f->ctx, kSweepSlots * sizeof(unsigned long long) * n);
-    f->sweep_actions = (double *)dev_alloc(f->ctx, sizeof(double) * n);
+    field_free(f, f->sweep_counts);
+    field_free(f, f->sweep_actions);
+    f->sweep_counts = (unsigned long long *)field_alloc(f, kSweepSlots * sizeof(unsigned long long) * n);
+    f->sweep_actions = (double *)field_alloc(f, sizeof(double) * n);
     if (!f->sweep_counts || !f->sweep_actions) {
         f->sweep_cap = 0;
         return fail(VS_ENOMEM, "%s: stats allocation failed", who);
@@ -881,8 +983,8 @@ extern "C" vs_status vs_flow_rk3(vs_field *f, int32_t n_steps, double step, doub
     const size_t sbytes = 4ull * 9 * f->g.P * (f->prec == VS_FP32 ? sizeof(float) : sizeof(double));
     if (f->flowS_bytes < sbytes) {
         CK(cudaStreamSynchronize(f->stream));
-        dev_free(f->ctx, f->flowS);
-        f->flowS = dev_alloc(f->ctx, sbytes);
+        field_free(f, f->flowS);
+        f->flowS = field_alloc(f, sbytes);
         f->flowS_bytes = f->flowS ? sbytes : 0;
         if (!f->flowS) return fail(VS_ENOMEM, "vs_flow_rk3: exponent buffer of %zu bytes failed", sbytes);
     }

@@ -19,18 +19,45 @@
 #include "vs_internal.h"
 
 namespace vs {
+
 struct Serve;
-}
+
+// Device blocks of the served jobs' fields.  A finished job's blocks are kept for
+// the next job: cudaFree waits for the whole device, so freeing them while other
+// jobs run stopped the scheduler until the longest running chunk was done (a mix of
+// 12 short jobs of four shapes: 27.4 ms, 12 of them in one such wait).  The idle
+// blocks count against the admission budget, and the scheduler gives them back
+// once it has been idle for kPoolLingerMs.  A block is given after the stream that
+// used it has been synchronised, so the next owner may use any stream.
+struct DevicePool {
+    std::mutex mu;
+    std::multimap<size_t, void *> idle;
+    std::map<void *, size_t> size;     // of every block taken or idle
+    size_t idle_bytes = 0;
+
+    bool empty();                      // no idle block
+    void *take(size_t bytes);          // an idle block of this size, or a new one (nullptr: no memory)
+    void give(void *p);
+    void trim();                       // free every idle block
+    // Free idle blocks, except one for each of the n sizes that a field is about to
+    // take, until the others and `others` more bytes are within `budget`.
+    void make_room(const size_t *sizes, int n, uint64_t others, uint64_t budget);
+};
+constexpr int kPoolLingerMs = 100;
+
+}  // namespace vs
 
 struct vs_ctx {
     vs_options opt;
     std::chrono::steady_clock::time_point t0;
     vs::Serve *serve = nullptr;      // owned; released by serve_shutdown
+    vs::DevicePool pool;             // blocks of served jobs (not used with the caller's allocator hooks)
     std::mutex serve_init_mu;
 };
 
 struct vs_field {
     vs_ctx *ctx = nullptr;
+    vs::DevicePool *pool = nullptr; // served job: its device blocks come from here and go back
     vs::Geo g{};
     int prec = VS_FP64;
     int nc = 18;
@@ -79,6 +106,11 @@ vs_status cuda_fail(cudaError_t e, const char *what);
 void *dev_alloc(vs_ctx *c, size_t bytes);
 void dev_free(vs_ctx *c, void *p);
 uint64_t field_footprint(const int32_t dims[4], int32_t precision, int32_t storage);
+// Sizes of the device blocks of a field (links, two label planes, scalars, FP32: the re-decision list).
+constexpr int kFieldBlocks = 5;
+int field_block_sizes(const int32_t dims[4], int32_t precision, int32_t storage, size_t sizes[kFieldBlocks]);
+vs_status field_create(vs_ctx *c, const int32_t dims[4], int32_t precision, int32_t storage, void *stream,
+                       DevicePool *pool, vs_field **out);
 bool valid_dims(const int32_t dims[4]);
 
 // Enqueue n_sweeps on the field's stream.  want_stats: per-sweep counters and

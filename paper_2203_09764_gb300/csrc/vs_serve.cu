@@ -144,9 +144,19 @@ bool Serve::admit_one(std::unique_lock<std::mutex> &lk) {
         bytes_in_use += jp->footprint;
         peak_bytes = std::max(peak_bytes, bytes_in_use);
         running.push_back(t);
+        // without a budget the idle blocks may take as much as jobs ever did, or 1 GB
+        const uint64_t used = budget ? bytes_in_use : 0, most = budget ? budget : std::max<uint64_t>(peak_bytes, 1u << 30);
         lk.unlock();
-        vs_status st = vs_field_create(ctx, jp->spec.dims, jp->spec.precision, jp->spec.storage,
-                                       (void *)jp->stream, &jp->f);
+        DevicePool *const from = ctx->opt.alloc ? nullptr : &ctx->pool;
+        if (from && !from->empty()) {
+            // idle blocks count against the budget, those this job takes only once
+            size_t sizes[kFieldBlocks + 1];
+            int n = field_block_sizes(jp->spec.dims, jp->spec.precision, jp->spec.storage, sizes);
+            sizes[n++] = jp->footprint - field_footprint(jp->spec.dims, jp->spec.precision, jp->spec.storage);  // staging
+            from->make_room(sizes, n, used, most);
+        }
+        vs_status st = field_create(ctx, jp->spec.dims, jp->spec.precision, jp->spec.storage, (void *)jp->stream, from,
+                                    &jp->f);
         if (st == VS_OK) {
             if (!jp->labels.empty()) st = vs_load_field(jp->f, nullptr, jp->labels.data(), VS_HOST);
             else st = vs_load_cooled(jp->f, jp->spec.seed, jp->spec.n_cool);
@@ -336,7 +346,12 @@ void Serve::loop() {
         step_running(lk, progressed);
         if (stop) break;
         if (running.empty() && waiting.empty()) {
-            cv_work.wait(lk);
+            if (ctx->pool.empty()) {
+                cv_work.wait(lk);
+            } else if (cv_work.wait_for(lk, std::chrono::milliseconds(kPoolLingerMs)) == std::cv_status::timeout &&
+                       running.empty() && waiting.empty()) {
+                ctx->pool.trim();   // nothing runs: give the memory back
+            }
         } else if (!progressed) {
             cv_work.wait_for(lk, std::chrono::microseconds(50));
         }
@@ -390,6 +405,7 @@ void serve_shutdown(vs_ctx *c) {
     for (auto &kv : s->graph_pool)
         for (auto g : kv.second) cudaGraphExecDestroy(g);
     for (auto st : s->streams) cudaStreamDestroy(st);
+    c->pool.trim();
     delete s;
     c->serve = nullptr;
 }
