@@ -143,8 +143,9 @@ __global__ void __launch_bounds__(VS_SUBSWEEP_THREADS) k_ape(ApeParams a) {
     count_update<double>(a.counters, up);
 }
 
-// FP32: the staple links through the per-thread ring, the one-pass stream of
-// k_subsweep_fused for over-improved staples, the plaquette-staple ring for eps = 1.
+// FP32 colour class, or every link of direction MU (colour < 0): the staple links
+// through the per-thread ring, the one-pass stream of k_subsweep_fused for
+// over-improved staples, the plaquette-staple ring for eps = 1.
 template <int NC, bool RECT, int MU>
 __global__ void __launch_bounds__(VS_RING_THREADS, RECT ? VS_RING_MINB : 4) k_ape_ring(ApeParams a) {
     extern __shared__ float4 ape_dyn[];
@@ -162,12 +163,40 @@ __global__ void __launch_bounds__(VS_RING_THREADS, RECT ? VS_RING_MINB : 4) k_ap
         dep_wait();
         M3<float> Vb, Ux;
         if constexpr (RECT) {
-            Vb = staple_sum_fused<NC, MU>(g, Us, x, a.c0_f, a.c1_f, R, Ux);
+            Vb = staple_sum_fused<NC>(g, Us, MU, x, a.c0_f, a.c1_f, R, Ux);
         } else {
-            Vb = staple_sum_plain_ring<NC, MU>(g, Us, x, a.c0_f, R);
+            Vb = staple_sum_plain_ring<NC>(g, Us, MU, x, a.c0_f, R);
             Ux = load_link<float, NC>(Us, g.P, MU, i);
         }
         ape_finish<float, NC>(a, MU, x, i, Vb, Ux, up);
+    }
+    count_update<float>(a.counters, up);
+}
+
+// The same for every link, from Usrc (simultaneous sweeps).
+template <int NC, bool RECT>
+__global__ void __launch_bounds__(VS_RING_THREADS, RECT ? VS_RING_MINB : 4) k_ape_all(ApeParams a) {
+    extern __shared__ float4 ape_dyn[];
+    float4 *ring4 = ape_dyn;
+    float2 *ring2 = reinterpret_cast<float2 *>(ape_dyn + 6 * (NC / 4) * VS_RING_THREADS);
+    int t;
+    const int mu = all_directions(VS_RING_THREADS, t);
+    Update<float> up;
+    if (t < a.n_threads) {
+        const Geo &g = a.g;
+        const Pt x = site_of_index(g, t);
+        const int i = sidx(g, x);
+        const float *Us = static_cast<const float *>(a.Usrc);
+        LinkRing<NC> R = ring_of<NC>(ring4, ring2);
+        dep_wait();
+        M3<float> Vb, Ux;
+        if constexpr (RECT) {
+            Vb = staple_sum_fused<NC>(g, Us, mu, x, a.c0_f, a.c1_f, R, Ux);
+        } else {
+            Vb = staple_sum_plain_ring<NC>(g, Us, mu, x, a.c0_f, R);
+            Ux = load_link<float, NC>(Us, g.P, mu, i);
+        }
+        ape_finish<float, NC>(a, mu, x, i, Vb, Ux, up);
     }
     count_update<float>(a.counters, up);
 }
@@ -223,19 +252,20 @@ __global__ void __launch_bounds__(VS_SUBSWEEP_THREADS) k_flow_stage(FlowParams a
     flow_count(a, used64);
 }
 
-// The same stage in FP32 with the staple links streamed through the per-thread
-// cp.async ring: the one-pass stream of the class kernel for over-improved
-// staples, the plaquette-staple ring for eps = 1.
+// The same stage in FP32 with the staple links streamed through the per-thread cp.async ring: the one-pass stream of the class
+// kernel for over-improved staples, the plaquette-staple ring for eps = 1.
+// MU: every direction in one launch (-1), or this one.
 template <int NC, bool RECT, int MU>
 __global__ void __launch_bounds__(VS_RING_THREADS, RECT ? VS_RING_MINB : 4) k_flow_stage_ring(FlowParams a) {
     extern __shared__ float4 flow_dyn[];
     float4 *ring4 = flow_dyn;
     float2 *ring2 = reinterpret_cast<float2 *>(flow_dyn + 6 * (NC / 4) * VS_RING_THREADS);
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    int t = blockIdx.x * VS_RING_THREADS + threadIdx.x, mu = MU;
+    if constexpr (MU < 0) mu = all_directions(VS_RING_THREADS, t);
     bool used64 = false;
     if (t < a.n_threads) {
         const Geo &g = a.g;
-        const Pt x = dir_site(g, MU, t);
+        const Pt x = MU < 0 ? site_of_index(g, t) : dir_site(g, MU, t);
         const int i = sidx(g, x);
         const float *Us = static_cast<const float *>(a.Usrc);
         LinkRing<NC> R = ring_of<NC>(ring4, ring2);
@@ -244,16 +274,16 @@ __global__ void __launch_bounds__(VS_RING_THREADS, RECT ? VS_RING_MINB : 4) k_fl
         // the exponent H_S of this link, read before the staple stream so that
         // its latency hides behind it (stage 1 of a step does not read it)
         float s_old[9];
-        const float *Sp = static_cast<const float *>(a.S) + (long long)MU * 9 * g.P + i;
+        const float *Sp = static_cast<const float *>(a.S) + (long long)mu * 9 * g.P + i;
 #pragma unroll
         for (int k = 0; k < 9; ++k) s_old[k] = a.b_f != 0.0f ? __ldg(Sp + (long long)k * g.P) : 0.0f;
         if constexpr (RECT) {
-            sig = staple_sum_fused<NC, MU>(g, Us, x, a.c0_f, a.c1_f, R, u);
+            sig = staple_sum_fused<NC>(g, Us, mu, x, a.c0_f, a.c1_f, R, u);
         } else {
-            sig = staple_sum_plain_ring<NC, MU>(g, Us, x, a.c0_f, R);
-            u = load_link<float, NC>(Us, g.P, MU, i);
+            sig = staple_sum_plain_ring<NC>(g, Us, mu, x, a.c0_f, R);
+            u = load_link<float, NC>(Us, g.P, mu, i);
         }
-        flow_finish<float, NC>(a, MU, i, sig, u, used64, s_old);
+        flow_finish<float, NC>(a, mu, i, sig, u, used64, s_old);
     }
     flow_count(a, used64);
 }

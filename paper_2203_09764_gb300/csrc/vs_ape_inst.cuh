@@ -7,18 +7,29 @@
 
 namespace vs {
 
-// annealed classes and simultaneous sweeps alike
+// A colour class of direction mu, or every link (mu < 0: simultaneous sweeps).
 template <class T, int NC>
 cudaError_t launch_ape_tpl(bool rect, int mu, const ApeParams &p, cudaStream_t st) {
     if (p.n_threads <= 0) return cudaSuccess;
     if constexpr (sizeof(T) == 8) {
         static void (*const kernels[2][4])(ApeParams) = {{k_ape<false, 0>, k_ape<false, 1>, k_ape<false, 2>, k_ape<false, 3>},
                                                          {k_ape<true, 0>, k_ape<true, 1>, k_ape<true, 2>, k_ape<true, 3>}};
-        return launch_links(kernels[rect][mu], p, st);
-    } else if (split_launch(rect, p.n_threads)) {
+        cudaError_t e = cudaSuccess;
+        for (int d = mu < 0 ? 0 : mu; e == cudaSuccess && d <= (mu < 0 ? 3 : mu); ++d)
+            e = launch_links(kernels[rect][d], p, st);
+        return e;
+    } else if (mu < 0 && !all_launch(rect, p.n_threads)) {
+        cudaError_t e = cudaSuccess;
+        for (int d = 0; e == cudaSuccess && d < 4; ++d) e = launch_ape_tpl<T, NC>(rect, d, p, st);
+        return e;
+    } else if ((mu < 0 || p.colour >= 0) && split_launch(rect, mu < 0 ? 4ll * p.n_threads : p.n_threads)) {
         static void (*const kernels[2])(ApeParams, int) = {k_ape_split<NC, false>, k_ape_split<NC, true>};
         static std::atomic<unsigned long long> set{0};
         return launch_split<NC>(kernels, rect, mu, p, set, st);
+    } else if (mu < 0) {
+        static void (*const kernels[2])(ApeParams) = {k_ape_all<NC, false>, k_ape_all<NC, true>};
+        static std::atomic<unsigned long long> set{0};
+        return launch_all<NC>(kernels, rect, p, set, st);
     } else {
         static void (*const kernels[2][4])(ApeParams) = {
             {k_ape_ring<NC, false, 0>, k_ape_ring<NC, false, 1>, k_ape_ring<NC, false, 2>, k_ape_ring<NC, false, 3>},
@@ -28,26 +39,32 @@ cudaError_t launch_ape_tpl(bool rect, int mu, const ApeParams &p, cudaStream_t s
     }
 }
 
+// One stage, every direction.
 template <class T, int NC>
-cudaError_t launch_flow_tpl(bool rect, int mu, const FlowParams &p, cudaStream_t st) {
+cudaError_t launch_flow_tpl(bool rect, const FlowParams &p, cudaStream_t st) {
     if (p.n_threads <= 0) return cudaSuccess;
     if constexpr (sizeof(T) == 8) {
         static void (*const kernels[2][4])(FlowParams) = {
             {k_flow_stage<false, 0>, k_flow_stage<false, 1>, k_flow_stage<false, 2>, k_flow_stage<false, 3>},
             {k_flow_stage<true, 0>, k_flow_stage<true, 1>, k_flow_stage<true, 2>, k_flow_stage<true, 3>}};
-        return launch_links(kernels[rect][mu], p, st);
-    } else if (split_launch(rect, p.n_threads)) {
+        for (int mu = 0; mu < 4; ++mu) {
+            const cudaError_t e = launch_links(kernels[rect][mu], p, st);
+            if (e != cudaSuccess) return e;
+        }
+        return cudaSuccess;
+    } else if (split_launch(rect, 4ll * p.n_threads)) {
         static void (*const kernels[2])(FlowParams, int) = {k_flow_split<NC, false>, k_flow_split<NC, true>};
         static std::atomic<unsigned long long> set{0};
-        return launch_split<NC>(kernels, rect, mu, p, set, st);
+        return launch_split<NC>(kernels, rect, -1, p, set, st);
     } else {
-        static void (*const kernels[2][4])(FlowParams) = {
-            {k_flow_stage_ring<NC, false, 0>, k_flow_stage_ring<NC, false, 1>, k_flow_stage_ring<NC, false, 2>,
-             k_flow_stage_ring<NC, false, 3>},
-            {k_flow_stage_ring<NC, true, 0>, k_flow_stage_ring<NC, true, 1>, k_flow_stage_ring<NC, true, 2>,
-             k_flow_stage_ring<NC, true, 3>}};
+        static void (*const all[2])(FlowParams) = {k_flow_stage_ring<NC, false, -1>, k_flow_stage_ring<NC, true, -1>};
+        static void (*const each[4])(FlowParams) = {k_flow_stage_ring<NC, true, 0>, k_flow_stage_ring<NC, true, 1>,
+                                                    k_flow_stage_ring<NC, true, 2>, k_flow_stage_ring<NC, true, 3>};
         static std::atomic<unsigned long long> set[2] = {{0}, {0}};
-        return launch_ring(kernels[rect], mu, p, ring6_smem_bytes<NC>(), set[rect], st);
+        if (all_launch(rect, p.n_threads)) return launch_all<NC>(all, rect, p, set[0], st);
+        cudaError_t e = cudaSuccess;
+        for (int d = 0; e == cudaSuccess && d < 4; ++d) e = launch_ring(each, d, p, ring6_smem_bytes<NC>(), set[1], st);
+        return e;
     }
 }
 

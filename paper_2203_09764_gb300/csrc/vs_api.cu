@@ -754,7 +754,7 @@ vs_status vs::smooth_enqueue(vs_field *f, int32_t n_sweeps, double rho, double e
             p.U = nxt;
             p.colour = -1;
             p.n_threads = f->g.V;
-            for (int mu = 0; mu < 4; ++mu) CK(subsweep_launch(f, rect, mu, p));
+            CK(subsweep_launch(f, rect, -1, p));   // every direction
             std::swap(cur, nxt);
         }
         if (f->profiling) CK(cudaEventRecord(f->events[2 * s + 1], f->stream));
@@ -771,7 +771,9 @@ vs_status vs::smooth_enqueue(vs_field *f, int32_t n_sweeps, double rho, double e
             float ms = 0;
             CK(cudaEventElapsedTime(&ms, f->events[2 * s], f->events[2 * s + 1]));
             f->prof_ms += ms;
-            f->prof_launches += a.kind == VS_ANNEALED ? 16 : 4;
+            // a simultaneous FP32 sweep is one launch, except with the re-decision list and on large lattices
+            const bool per_direction = f->prec == VS_FP64 || (a.fp64_redecide && vp) || (rect && f->g.V > kAllMostRect);
+            f->prof_launches += a.kind == VS_ANNEALED ? 16 : per_direction ? 4 : 1;
         }
     }
     f->last_action_every = a.action_every;
@@ -874,10 +876,10 @@ static cudaError_t ape_launch(vs_field *f, bool rect, int mu, const ApeParams &p
     return launch_ape_f18(rect, mu, p, f->stream);
 }
 
-static cudaError_t flow_launch(vs_field *f, bool rect, int mu, const FlowParams &p) {
-    if (f->prec == VS_FP64) return launch_flow_d18(rect, mu, p, f->stream);
-    if (f->nc == 12) return launch_flow_f12(rect, mu, p, f->stream);
-    return launch_flow_f18(rect, mu, p, f->stream);
+static cudaError_t flow_launch(vs_field *f, bool rect, const FlowParams &p) {
+    if (f->prec == VS_FP64) return launch_flow_d18(rect, p, f->stream);
+    if (f->nc == 12) return launch_flow_f12(rect, p, f->stream);
+    return launch_flow_f18(rect, p, f->stream);
 }
 
 // per-sweep counter blocks (kSweepSlots each) in the field's stats buffer
@@ -944,7 +946,7 @@ extern "C" vs_status vs_smooth_ape(vs_field *f, int32_t n_sweeps, double alpha, 
             a.U = nxt;
             a.colour = -1;
             a.n_threads = f->g.V;
-            for (int mu = 0; mu < 4; ++mu) CK(ape_launch(f, rect, mu, a));
+            CK(ape_launch(f, rect, -1, a));   // every direction
             std::swap(cur, nxt);
         }
         if (f->prec == VS_FP32 && reunit_every > 0 && (f->sweeps_done + s + 1) % reunit_every == 0)
@@ -1026,7 +1028,7 @@ extern "C" vs_status vs_flow_rk3(vs_field *f, int32_t n_steps, double step, doub
             p.c_f = (float)p.c;
             p.Usrc = cur;
             p.U = nxt;
-            for (int mu = 0; mu < 4; ++mu) CK(flow_launch(f, rect, mu, p));
+            CK(flow_launch(f, rect, p));
             std::swap(cur, nxt);
         }
         if (f->prec == VS_FP32 && reunit_every > 0 && (f->sweeps_done + s + 1) % reunit_every == 0)

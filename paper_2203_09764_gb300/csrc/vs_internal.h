@@ -50,6 +50,10 @@ constexpr unsigned long long kMarginInit = 0x7f7f7f7f7f7f7f7full;   // a double 
 // undecidable).
 constexpr int kDeferCap = 16384;
 
+// FP32 updates that read one field and write another: the most sites for which one
+// over-improved launch takes every direction (vs_stout.cuh, all_launch).
+constexpr int kAllMostRect = 786432;
+
 // process-wide count of direct kernel launches
 void count_launches(int n);
 long long launches();
@@ -89,14 +93,14 @@ struct ApeParams {
 };
 
 // One stage of the third-order Runge-Kutta Wilson flow for every link of
-// direction mu: with H_Z the Hermitian form of h Q[W_i] (Eq. generator),
+// every direction: with H_Z the Hermitian form of h Q[W_i] (Eq. generator),
 // H_S <- a H_Z + b H_S (b = 0: H_S not read), W_{i+1} = exp(i c H_S) W_i.
 struct FlowParams {
     Geo g;
     void *U;             // W_{i+1}
     const void *Usrc;    // W_i
     void *S;             // H_S, 9 reals per link [mu][9][P] in the field precision
-    int n_threads;
+    int n_threads;       // sites
     double h, a, b, c, c0, c1;
     float h_f, a_f, b_f, c_f, c0_f, c1_f;
     unsigned long long *counters;  // kCntSecond: FP64 exponentials of the step (may be null)
@@ -105,9 +109,9 @@ struct FlowParams {
 cudaError_t launch_ape_f18(bool rect, int mu, const ApeParams &p, cudaStream_t st);
 cudaError_t launch_ape_f12(bool rect, int mu, const ApeParams &p, cudaStream_t st);
 cudaError_t launch_ape_d18(bool rect, int mu, const ApeParams &p, cudaStream_t st);
-cudaError_t launch_flow_f18(bool rect, int mu, const FlowParams &p, cudaStream_t st);
-cudaError_t launch_flow_f12(bool rect, int mu, const FlowParams &p, cudaStream_t st);
-cudaError_t launch_flow_d18(bool rect, int mu, const FlowParams &p, cudaStream_t st);
+cudaError_t launch_flow_f18(bool rect, const FlowParams &p, cudaStream_t st);
+cudaError_t launch_flow_f12(bool rect, const FlowParams &p, cudaStream_t st);
+cudaError_t launch_flow_d18(bool rect, const FlowParams &p, cudaStream_t st);
 
 cudaError_t launch_aus_f18(bool rect, int mu, const AusParams &p, cudaStream_t st);
 cudaError_t launch_aus_f12(bool rect, int mu, const AusParams &p, cudaStream_t st);

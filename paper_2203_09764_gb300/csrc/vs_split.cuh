@@ -103,13 +103,25 @@ __device__ __forceinline__ bool staple_sum_split(const Geo &g, const float *__re
     return true;
 }
 
-// Links per launch are a multiple of 64 (a quarter of V), so every warp is full.
+// Site and direction of this lane: colour class (direction `arg`), or with colour < 0
+// every link, `arg` blocks per direction.  Links per launch are a multiple of 64 (a
+// quarter of V), so every warp is full.
+__device__ __forceinline__ Pt split_site(const Geo &g, int colour, int arg, int &mu) {
+    const int lane = threadIdx.x & 31, b = blockIdx.x;
+    if (colour >= 0) {
+        mu = arg;
+        return class_site(g, mu, colour, b * 32 + lane);
+    }
+    mu = b / arg;
+    return site_of_index(g, (b - mu * arg) * 32 + lane);
+}
+
 template <int NC, bool RECT>
-__global__ void __launch_bounds__(kSplitThreads, 4) k_subsweep_split(SubsweepParams a, int mu) {
+__global__ void __launch_bounds__(kSplitThreads, 4) k_subsweep_split(SubsweepParams a, int arg) {
     extern __shared__ float4 split_dyn[];
     const Geo &g = a.g;
-    const int t = blockIdx.x * 32 + (threadIdx.x & 31);
-    const Pt x = a.colour >= 0 ? class_site(g, mu, a.colour, t) : dir_site(g, mu, t);
+    int mu;
+    const Pt x = split_site(g, a.colour, arg, mu);
     M3<float> sig, Ux;
     if (!staple_sum_split<NC, RECT>(g, static_cast<const float *>(a.Usrc), mu, x, a.c0_f, a.c1_f, split_dyn, sig, Ux))
         return;
@@ -132,11 +144,11 @@ __global__ void __launch_bounds__(kSplitThreads, 4) k_aus_split(AusParams a, int
 }
 
 template <int NC, bool RECT>
-__global__ void __launch_bounds__(kSplitThreads, 4) k_ape_split(ApeParams a, int mu) {
+__global__ void __launch_bounds__(kSplitThreads, 4) k_ape_split(ApeParams a, int arg) {
     extern __shared__ float4 split_dyn[];
     const Geo &g = a.g;
-    const int t = blockIdx.x * 32 + (threadIdx.x & 31);
-    const Pt x = a.colour >= 0 ? class_site(g, mu, a.colour, t) : dir_site(g, mu, t);
+    int mu;
+    const Pt x = split_site(g, a.colour, arg, mu);
     M3<float> sig, Ux;
     if (!staple_sum_split<NC, RECT>(g, static_cast<const float *>(a.Usrc), mu, x, a.c0_f, a.c1_f, split_dyn, sig, Ux))
         return;
@@ -146,10 +158,11 @@ __global__ void __launch_bounds__(kSplitThreads, 4) k_ape_split(ApeParams a, int
 }
 
 template <int NC, bool RECT>
-__global__ void __launch_bounds__(kSplitThreads, 4) k_flow_split(FlowParams a, int mu) {
+__global__ void __launch_bounds__(kSplitThreads, 4) k_flow_split(FlowParams a, int arg) {
     extern __shared__ float4 split_dyn[];
     const Geo &g = a.g;
-    const Pt x = dir_site(g, mu, blockIdx.x * 32 + (threadIdx.x & 31));
+    int mu;
+    const Pt x = split_site(g, -1, arg, mu);
     M3<float> sig, u;
     if (!staple_sum_split<NC, RECT>(g, static_cast<const float *>(a.Usrc), mu, x, a.c0_f, a.c1_f, split_dyn, sig, u))
         return;
@@ -166,9 +179,10 @@ __global__ void __launch_bounds__(kSplitThreads, 4) k_flow_split(FlowParams a, i
 // 5.5, 16,384 4.4 / 4.6.
 constexpr int kSplitMost = 32768, kSplitMostPlain = 12288;
 
-inline bool split_launch(bool rect, int links) { return links <= (rect ? kSplitMost : kSplitMostPlain); }
+inline bool split_launch(bool rect, long long links) { return links <= (rect ? kSplitMost : kSplitMostPlain); }
 
-// The launch of a smoother's over-improved or plaquette-staple kernel.
+// The launch of a smoother's plaquette-staple (0) or over-improved (1) kernel for a
+// colour class of direction mu, or for every link of p.n_threads sites (mu < 0).
 template <int NC, class P>
 cudaError_t launch_split(void (*const kernels[2])(P, int), bool rect, int mu, const P &p,
                          std::atomic<unsigned long long> &attr_set, cudaStream_t st) {
@@ -177,7 +191,8 @@ cudaError_t launch_split(void (*const kernels[2])(P, int), bool rect, int mu, co
         for (int k = 0; k < 2; ++k)
             cudaFuncSetAttribute(kernels[k], cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
     });
-    return launch_dependent(kernels[rect], p.n_threads / 32, kSplitThreads, (size_t)sm, st, p, mu);
+    const int b = p.n_threads / 32;
+    return launch_dependent(kernels[rect], mu < 0 ? 4 * b : b, kSplitThreads, (size_t)sm, st, p, mu < 0 ? b : mu);
 }
 
 }  // namespace vs

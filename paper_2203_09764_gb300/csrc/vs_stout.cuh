@@ -757,8 +757,8 @@ __device__ __forceinline__ void fused_unit(const LinkRing<NC, BT> &R, M3<float> 
     u_refill<NC, S, 11>(R, Umu, Unu, Un, P, A, An, last, spare);
 }
 
-template <int NC, int MU>
-__device__ __forceinline__ M3<float> staple_sum_fused(const Geo &g, const float *__restrict__ U, Pt x, float c0,
+template <int NC>
+__device__ __forceinline__ M3<float> staple_sum_fused(const Geo &g, const float *__restrict__ U, int MU, Pt x, float c0,
                                                       float c1, const LinkRing<NC> &R, M3<float> &Ux) {
     const long long P = g.P;
     Around A, An;
@@ -844,8 +844,8 @@ __device__ __forceinline__ void plain_unit(const LinkRing<NC, BT> &R, M3<float> 
     for (int k = 0; k < 9; ++k) { sig.re[k] += Y.re[k]; sig.im[k] += Y.im[k]; }
 }
 
-template <int NC, int MU>
-__device__ __forceinline__ M3<float> staple_sum_plain_ring(const Geo &g, const float *__restrict__ U, Pt x,
+template <int NC>
+__device__ __forceinline__ M3<float> staple_sum_plain_ring(const Geo &g, const float *__restrict__ U, int MU, Pt x,
                                                            float c0, const LinkRing<NC> &R) {
     const long long P = g.P;
     Around A, An;
@@ -931,7 +931,7 @@ __global__ void __launch_bounds__(VS_RING_THREADS, 4) k_subsweep_pring(SubsweepP
         const float *Us = static_cast<const float *>(a.Usrc);
         LinkRing<NC> R = ring_of<NC>(ring4, ring2);
         dep_wait();
-        const M3<float> sig = staple_sum_plain_ring<NC, MU>(g, Us, x, a.c0_f, R);
+        const M3<float> sig = staple_sum_plain_ring<NC>(g, Us, MU, x, a.c0_f, R);
         const M3<float> Ux = load_link<float, NC>(Us, g.P, MU, i);
         stout_store<float, NC>(a, MU, x, i, sig, Ux, u);
     }
@@ -953,7 +953,7 @@ __global__ void __launch_bounds__(VS_RING_THREADS, VS_RING_MINB) k_subsweep_fuse
         LinkRing<NC> R = ring_of<NC>(ring4, ring2);
         dep_wait();
         M3<float> Ux;
-        M3<float> sig = staple_sum_fused<NC, MU>(g, static_cast<const float *>(a.Usrc), x, a.c0_f, a.c1_f, R, Ux);
+        M3<float> sig = staple_sum_fused<NC>(g, static_cast<const float *>(a.Usrc), MU, x, a.c0_f, a.c1_f, R, Ux);
         stout_store<float, NC>(a, MU, x, i, sig, Ux, u);
     }
     count_update<float>(a.counters, u);
@@ -1073,7 +1073,7 @@ __global__ void __launch_bounds__(VS_RING_THREADS, VS_RING_MINB) k_aus_ring(AusP
         LinkRing<NC> R = ring_of<NC>(ring4, ring2);
         dep_wait();
         M3<float> Ux;
-        const M3<float> Vb = staple_sum_fused<NC, MU>(g, static_cast<const float *>(a.U), x, a.c0_f, a.c1_f, R, Ux);
+        const M3<float> Vb = staple_sum_fused<NC>(g, static_cast<const float *>(a.U), MU, x, a.c0_f, a.c1_f, R, Ux);
         aus_finish<float, NC>(a, MU, x, i, Vb, Ux, up);
     }
     count_update<float>(a.counters, up);
@@ -1096,11 +1096,77 @@ __global__ void __launch_bounds__(VS_RING_THREADS, 4) k_aus_pring(AusParams a) {
         const float *Us = static_cast<const float *>(a.U);
         LinkRing<NC> R = ring_of<NC>(ring4, ring2);
         dep_wait();
-        const M3<float> Vb = staple_sum_plain_ring<NC, MU>(g, Us, x, a.c0_f, R);
+        const M3<float> Vb = staple_sum_plain_ring<NC>(g, Us, MU, x, a.c0_f, R);
         const M3<float> Ux = load_link<float, NC>(Us, g.P, MU, i);
         aus_finish<float, NC>(a, MU, x, i, Vb, Ux, up);
     }
     count_update<float>(a.counters, up);
+}
+
+// FP32 updates that read one field and write another (simultaneous sweeps, the
+// Runge-Kutta stages) take every direction in one launch.  Its blocks come in groups
+// of kAllGroup per direction, direction after direction, so that the directions of the
+// same sites run at the same time and share their links in L2.  Against a launch per
+// direction: small lattices save three launches of four and fill the chip (flow stage
+// with eps = 1, per direction: 1024 sites 4.6 -> 1.1 us, 16,384 sites 9.1 -> 6.5);
+// from 262,144 sites on, the links' way from L2 into the SMs (1.4 KB per link, 17 TB/s)
+// is the bound and the order changes little (177.7 -> 177.3 us at 32^3x64).
+// Over-improved staples need every register, and a direction known at compile time
+// saves a few: above kAllMostRect sites they keep a launch per direction (1,048,576
+// sites, APE 362 us per direction against 356; 663,552 sites 245 against 249).
+constexpr int kAllGroup = 114;   // a quarter of the resident blocks
+inline bool all_launch(bool rect, int sites) { return !rect || sites <= kAllMostRect; }
+
+// Direction and first-to-last site number of this thread in such a launch; the blocks
+// hold `threads` sites each, four times as many blocks as sites / threads.
+__device__ __forceinline__ int all_directions(int threads, int &t) {
+    const int per = (int)(gridDim.x >> 2);
+    const int first = (int)(blockIdx.x / (4 * kAllGroup)) * kAllGroup;
+    const int size = min(kAllGroup, per - first), r = (int)blockIdx.x - 4 * first;
+    const int mu = r / size;
+    t = (first + r - mu * size) * threads + (int)threadIdx.x;
+    return mu;
+}
+
+// The same for every link, from Usrc.
+template <int NC, bool RECT>
+__global__ void __launch_bounds__(VS_RING_THREADS, RECT ? VS_RING_MINB : 4) k_subsweep_all(SubsweepParams a) {
+    extern __shared__ float4 all_dyn[];
+    float4 *ring4 = all_dyn;
+    float2 *ring2 = reinterpret_cast<float2 *>(all_dyn + 6 * (NC / 4) * VS_RING_THREADS);
+    int t;
+    const int mu = all_directions(VS_RING_THREADS, t);
+    Update<float> u;
+    if (t < a.n_threads) {
+        const Geo &g = a.g;
+        const Pt x = site_of_index(g, t);
+        const int i = sidx(g, x);
+        const float *Us = static_cast<const float *>(a.Usrc);
+        LinkRing<NC> R = ring_of<NC>(ring4, ring2);
+        dep_wait();
+        M3<float> sig, Ux;
+        if constexpr (RECT) {
+            sig = staple_sum_fused<NC>(g, Us, mu, x, a.c0_f, a.c1_f, R, Ux);
+        } else {
+            sig = staple_sum_plain_ring<NC>(g, Us, mu, x, a.c0_f, R);
+            Ux = load_link<float, NC>(Us, g.P, mu, i);
+        }
+        stout_store<float, NC>(a, mu, x, i, sig, Ux, u);
+    }
+    count_update<float>(a.counters, u);
+}
+
+// One launch over every direction of a plaquette-staple (0) or over-improved (1) kernel.
+template <int NC, class P>
+cudaError_t launch_all(void (*const kernels[2])(P), bool rect, const P &p, std::atomic<unsigned long long> &attr_set,
+                       cudaStream_t st) {
+    constexpr int sm = ring6_smem_bytes<NC>();
+    once_per_device(attr_set, [&] {
+        for (int k = 0; k < 2; ++k)
+            cudaFuncSetAttribute(kernels[k], cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    });
+    const int per = (p.n_threads + VS_RING_THREADS - 1) / VS_RING_THREADS;
+    return launch_dependent(kernels[rect], 4 * per, VS_RING_THREADS, (size_t)sm, st, p);
 }
 
 // One launch of a thread-per-link FP64 kernel.

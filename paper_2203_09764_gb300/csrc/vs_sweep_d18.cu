@@ -53,6 +53,11 @@ static void launch_rows(int mu, const SubsweepParams &p, cudaStream_t st) {
 
 cudaError_t launch_subsweep_d18(bool rect, int mu, const SubsweepParams &p, cudaStream_t st) {
     if (p.n_threads <= 0) return cudaSuccess;
+    if (mu < 0) {   // simultaneous sweep
+        cudaError_t e = cudaSuccess;
+        for (int d = 0; e == cudaSuccess && d < 4; ++d) e = launch_subsweep_d18(rect, d, p, st);
+        return e;
+    }
     if (rect) {
         launch_rows<true>(mu, p, st);
     } else if (p.n_threads < kRowsMost) {

@@ -20,15 +20,26 @@ void launch_redecide(int mu, const SubsweepParams &p, cudaStream_t st) {
     count_launches(1);
 }
 
-// FP32 stout class launches.
+// FP32 stout: a colour class of direction mu, or every link (mu < 0: simultaneous
+// sweeps; the re-decision list holds links of one direction, so with it each direction
+// is a launch of its own, as it is on large lattices).
 template <int NC>
 cudaError_t launch_subsweep_tpl(bool rect, int mu, const SubsweepParams &p, cudaStream_t st) {
     if (p.n_threads <= 0) return cudaSuccess;
+    if (mu < 0 && (p.defer_idx || !all_launch(rect, p.n_threads))) {
+        cudaError_t e = cudaSuccess;
+        for (int d = 0; e == cudaSuccess && d < 4; ++d) e = launch_subsweep_tpl<NC>(rect, d, p, st);
+        return e;
+    }
     cudaError_t e;
-    if (split_launch(rect, p.n_threads)) {
+    if ((mu < 0 || p.colour >= 0) && split_launch(rect, mu < 0 ? 4ll * p.n_threads : p.n_threads)) {
         static void (*const kernels[2])(SubsweepParams, int) = {k_subsweep_split<NC, false>, k_subsweep_split<NC, true>};
         static std::atomic<unsigned long long> set{0};
         e = launch_split<NC>(kernels, rect, mu, p, set, st);
+    } else if (mu < 0) {
+        static void (*const kernels[2])(SubsweepParams) = {k_subsweep_all<NC, false>, k_subsweep_all<NC, true>};
+        static std::atomic<unsigned long long> set{0};
+        e = launch_all<NC>(kernels, rect, p, set, st);
     } else {
         static void (*const kernels[2][4])(SubsweepParams) = {
             {k_subsweep_pring<NC, 0>, k_subsweep_pring<NC, 1>, k_subsweep_pring<NC, 2>, k_subsweep_pring<NC, 3>},
