@@ -220,6 +220,45 @@ __device__ __forceinline__ Part<US> part_mul(const Row &x, const RowLink &L, int
     return y;
 }
 
+// Coefficient f_which of exp(iH) = f0 + f1 H + f2 H^2 by the series of ch_exp_coeffs
+// (H by its diagonal and upper entries): three operations per term where all three
+// coefficients take five.
+__device__ __forceinline__ void exp_coefficient(const double h[9], int which, double &re, double &im) {
+    const double a01 = h[3] * h[3] + h[4] * h[4], a02 = h[5] * h[5] + h[6] * h[6], a12 = h[7] * h[7] + h[8] * h[8];
+    const double tau = 0.5 * (h[0] * h[0] + h[1] * h[1] + h[2] * h[2]) + a01 + a02 + a12;
+    const double pr = h[3] * h[7] - h[4] * h[8], pi = h[3] * h[8] + h[4] * h[7];
+    const double delta = h[0] * h[1] * h[2] + 2.0 * (pr * h[5] + pi * h[6]) - h[0] * a12 - h[1] * a02 - h[2] * a01;
+    const double r4 = 4.0 * tau * tau;
+    double sr = 0, si = 0, cm = 0, c = 0, cp = 1, w = 1, bound = 1;   // c_{n-1}, c_n, c_{n+1} at n = 1; 1 / n!
+    const auto pick = [&] { return which == 0 ? cm : which == 1 ? cp : c; };
+    const auto next = [&] {
+        const double v = fma(tau, c, delta * cm);
+        cm = c;
+        c = cp;
+        cp = v;
+    };
+#pragma unroll
+    for (int g4 = 0; g4 < 12; ++g4) {
+        const int n = 4 * g4 + 1;
+        w *= 1.0 / n;
+        si = fma(w, pick(), si);                              // i^n = i, -1, -i, 1
+        next();
+        w *= 1.0 / (n + 1);
+        sr = fma(-w, pick(), sr);
+        next();
+        w *= 1.0 / (n + 2);
+        si = fma(-w, pick(), si);
+        next();
+        w *= 1.0 / (n + 3);
+        sr = fma(w, pick(), sr);
+        next();
+        bound *= r4 * (1.0 / ((double)n * (n + 1) * (n + 2) * (n + 3)));
+        if (bound < Tol<double>::eps()) break;
+    }
+    re = which == 0 ? fma(delta, sr, 1.0) : sr;
+    im = which == 0 ? delta * si : si;
+}
+
 // Update of LPB links t0 .. t0 + LPB - 1 of a class launch by one block: blocks of
 // four warps (one per SM sub-partition; three warps leave one idle), LPB =
 // 128 / (3 US) links of 3 US lanes each, thread (r US + u) LPB + link.
@@ -293,17 +332,35 @@ __device__ __forceinline__ void rows_block(const SubsweepParams &a, int mu, int 
             for (int n = 0; n < 6 / US; ++n) sh.om[6 * r + part_comp<US>(n, u)][l] = om.v[n];
     }
     __syncthreads();
-    if (r == 0 && own) {
+    const double third = 1.0 / 3.0, hr2 = 0.5 * a.rho;
+    // H as in stout_H: component k of its diagonal (0-2) and upper entries (3-8)
+    const auto h_comp = [&](int k) {
+        if (k < 3) {
+            const double d = sh.om[8 * k + 1][l], d1 = sh.om[k == 0 ? 9 : 1][l], d2 = sh.om[k == 2 ? 9 : 17][l];
+            return a.rho * ((2.0 * d - d1 - d2) * third);
+        }
+        const int q = (k - 3) >> 1;                           // (0,1), (0,2), (1,2): entries 1, 2, 5 and 3, 6, 7
+        const int up = q == 0 ? 1 : q == 1 ? 2 : 5, dn = q == 0 ? 3 : q == 1 ? 6 : 7;
+        return k & 1 ? hr2 * (sh.om[2 * up + 1][l] + sh.om[2 * dn + 1][l])
+                     : -hr2 * (sh.om[2 * up][l] - sh.om[2 * dn][l]);
+    };
+    if constexpr (US == 6) {
+        // one of the 18 lanes per component, then each row sums one coefficient
+        if (work && part < 9) sh.hf[part][l] = h_comp(part);
+        __syncthreads();
+        if (own) {
+            double h[9], re, im;
+#pragma unroll
+            for (int k = 0; k < 9; ++k) h[k] = sh.hf[k][l];
+            exp_coefficient(h, r, re, im);
+            sh.hf[9 + 2 * r][l] = re;
+            sh.hf[10 + 2 * r][l] = im;
+        }
+    } else if (r == 0 && own) {
         // once per link, not once per row
-        const double third = 1.0 / 3.0, hr = 0.5 * a.rho;
-        const double d0 = sh.om[1][l], d1 = sh.om[9][l], d2 = sh.om[17][l];
         double h[9], f[6];
-        h[0] = a.rho * ((2.0 * d0 - d1 - d2) * third);
-        h[1] = a.rho * ((2.0 * d1 - d0 - d2) * third);
-        h[2] = a.rho * ((2.0 * d2 - d0 - d1) * third);
-        h[3] = hr * (sh.om[3][l] + sh.om[7][l]); h[4] = -hr * (sh.om[2][l] - sh.om[6][l]);
-        h[5] = hr * (sh.om[5][l] + sh.om[13][l]); h[6] = -hr * (sh.om[4][l] - sh.om[12][l]);
-        h[7] = hr * (sh.om[11][l] + sh.om[15][l]); h[8] = -hr * (sh.om[10][l] - sh.om[14][l]);
+#pragma unroll
+        for (int k = 0; k < 9; ++k) h[k] = h_comp(k);
         ch_exp_coeffs<double, 12>(h[0], h[1], h[2], h[3], h[4], h[5], h[6], h[7], h[8], 1e300, f);
 #pragma unroll
         for (int k = 0; k < 9; ++k) sh.hf[k][l] = h[k];
@@ -319,14 +376,27 @@ __device__ __forceinline__ void rows_block(const SubsweepParams &a, int mu, int 
         const double Hr[9] = {h0, ar, br, ar, h1, cr, br, cr, h2};
         const double Hi[9] = {0.0, ai, bi, -ai, 0.0, ci, -bi, -ci, 0.0};
         const double f2r = sh.hf[13][l], f2i = sh.hf[14][l];
+        const auto entry = [&](const double m[9], int k) {   // entry (r, k) of a matrix in registers
+            const double c0 = r == 0 ? m[0] : r == 1 ? m[3] : m[6], c1 = r == 0 ? m[1] : r == 1 ? m[4] : m[7],
+                         c2 = r == 0 ? m[2] : r == 1 ? m[5] : m[8];
+            return k == 0 ? c0 : k == 1 ? c1 : c2;
+        };
         Row y;
+        if constexpr (US == 6) {
+            Part<US> yp;
+            const int k = u >> 1;
+            const double xr = entry(Hr, k), xi = entry(Hi, k);
+            yp.v[0] = u & 1 ? f2r * xi + f2i * xr : f2r * xr - f2i * xi;
+            if (k == r) yp.v[0] += sh.hf[11 + (u & 1)][l];
+            y = part_gather<US, LPB>(yp, buf, u, l, work);
+        } else {
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const double xr = r == 0 ? Hr[k] : r == 1 ? Hr[3 + k] : Hr[6 + k];
-            const double xi = r == 0 ? Hi[k] : r == 1 ? Hi[3 + k] : Hi[6 + k];
-            y.re[k] = f2r * xr - f2i * xi;
-            y.im[k] = f2r * xi + f2i * xr;
-            if (k == r) { y.re[k] += sh.hf[11][l]; y.im[k] += sh.hf[12][l]; }
+            for (int k = 0; k < 3; ++k) {
+                const double xr = entry(Hr, k), xi = entry(Hi, k);
+                y.re[k] = f2r * xr - f2i * xi;
+                y.im[k] = f2r * xi + f2i * xr;
+                if (k == r) { y.re[k] += sh.hf[11][l]; y.im[k] += sh.hf[12][l]; }
+            }
         }
         Part<US> m;
 #pragma unroll
