@@ -147,6 +147,21 @@ __device__ __forceinline__ Pt class_site(const Geo &g, int MU, int c, int t) {
     return p;
 }
 
+// Number of the class site that thread k of a class launch of n links takes, n or
+// more for an idle thread: site k, except in rows of 20 sites (Lx/4 = 5).  There a
+// row's class sites are a run of five positions in a line of eight, and a warp that
+// takes 32 sites in order touches parts of 7 or 8 runs with every load; it takes six
+// whole runs and leaves two lanes idle (20^3x40, 18 reals: 51.3 -> 48.2 us per class
+// launch, MaxReTr 52.5 -> 49.6).  Rows of 24, five runs of six to a warp, are slower
+// that way: 68.6 -> 69.6 us at 24^3x48, 61.2 -> 64.0 with 12 reals.
+__device__ __forceinline__ int class_thread(const Geo &g, int k, int n) {
+    if (g.Q != 5) return k;
+    return (k & 31) < 30 ? k - 2 * (k >> 5) : n;
+}
+
+// Threads of a class launch of n links.
+inline int class_threads(const Geo &g, int n) { return g.Q != 5 ? n : (n + 29) / 30 * 32; }
+
 // --------------------------------------------------------------------------
 // 3x3 complex matrices in registers
 // --------------------------------------------------------------------------

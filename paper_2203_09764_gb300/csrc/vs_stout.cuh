@@ -921,7 +921,8 @@ __global__ void __launch_bounds__(VS_RING_THREADS, 4) k_subsweep_pring(SubsweepP
     extern __shared__ float4 pring_dyn[];
     float4 *ring4 = pring_dyn;
     float2 *ring2 = reinterpret_cast<float2 *>(pring_dyn + 6 * (NC / 4) * VS_RING_THREADS);
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (a.colour >= 0) t = class_thread(a.g, t, a.n_threads);
     const bool active = t < a.n_threads;
     Update<float> u;
     if (active) {
@@ -943,7 +944,8 @@ __global__ void __launch_bounds__(VS_RING_THREADS, VS_RING_MINB) k_subsweep_fuse
     extern __shared__ float4 ring6_dyn[];
     float4 *ring4 = ring6_dyn;
     float2 *ring2 = reinterpret_cast<float2 *>(ring6_dyn + 6 * (NC / 4) * VS_RING_THREADS);
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (a.colour >= 0) t = class_thread(a.g, t, a.n_threads);
     const bool active = t < a.n_threads;
     Update<float> u;
     if (active) {
@@ -1063,7 +1065,8 @@ __global__ void __launch_bounds__(VS_RING_THREADS, VS_RING_MINB) k_aus_ring(AusP
     extern __shared__ float4 aus_dyn[];
     float4 *ring4 = aus_dyn;
     float2 *ring2 = reinterpret_cast<float2 *>(aus_dyn + 6 * (NC / 4) * VS_RING_THREADS);
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    int t = blockIdx.x * blockDim.x + threadIdx.x;
+    t = class_thread(a.g, t, a.n_threads);
     const bool active = t < a.n_threads;
     Update<float> up;
     if (active) {
@@ -1086,7 +1089,8 @@ __global__ void __launch_bounds__(VS_RING_THREADS, 4) k_aus_pring(AusParams a) {
     extern __shared__ float4 ausp_dyn[];
     float4 *ring4 = ausp_dyn;
     float2 *ring2 = reinterpret_cast<float2 *>(ausp_dyn + 6 * (NC / 4) * VS_RING_THREADS);
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    int t = blockIdx.x * blockDim.x + threadIdx.x;
+    t = class_thread(a.g, t, a.n_threads);
     const bool active = t < a.n_threads;
     Update<float> up;
     if (active) {
@@ -1180,13 +1184,13 @@ cudaError_t launch_links(void (*kernel)(P), const P &p, cudaStream_t st) {
 // One launch of a link-ring kernel of direction mu out of its four instantiations.
 // attr_set: where the shared-memory limit has been set, one flag per kernel family.
 template <class P>
-cudaError_t launch_ring(void (*const kernels[4])(P), int mu, const P &p, int smem,
+cudaError_t launch_ring(void (*const kernels[4])(P), int mu, const P &p, int threads, int smem,
                         std::atomic<unsigned long long> &attr_set, cudaStream_t st) {
     once_per_device(attr_set, [&] {
         for (int k = 0; k < 4; ++k)
             cudaFuncSetAttribute(kernels[k], cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     });
-    return launch_dependent(kernels[mu], (p.n_threads + VS_RING_THREADS - 1) / VS_RING_THREADS, VS_RING_THREADS,
+    return launch_dependent(kernels[mu], (threads + VS_RING_THREADS - 1) / VS_RING_THREADS, VS_RING_THREADS,
                             (size_t)smem, st, p);
 }
 
