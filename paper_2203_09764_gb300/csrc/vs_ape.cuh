@@ -162,6 +162,7 @@ __global__ void __launch_bounds__(VS_RING_THREADS, RECT ? VS_RING_MINB : 4) k_ap
         const float *Us = static_cast<const float *>(a.Usrc);
         LinkRing<NC> R = ring_of<NC>(ring4, ring2);
         dep_wait();
+        if (!RECT) dep_launch();
         M3<float> Vb, Ux;
         if constexpr (RECT) {
             Vb = staple_sum_fused<NC>(g, Us, MU, x, a.c0_f, a.c1_f, R, Ux);
@@ -169,6 +170,7 @@ __global__ void __launch_bounds__(VS_RING_THREADS, RECT ? VS_RING_MINB : 4) k_ap
             Vb = staple_sum_plain_ring<NC>(g, Us, MU, x, a.c0_f, R);
             Ux = load_link<float, NC>(Us, g.P, MU, i);
         }
+        if (RECT) dep_launch();
         ape_finish<float, NC>(a, MU, x, i, Vb, Ux, up);
     }
     count_update<float>(a.counters, up);
@@ -189,7 +191,7 @@ __global__ void __launch_bounds__(VS_RING_THREADS, RECT ? VS_RING_MINB : 4) k_ap
         const int i = sidx(g, x);
         const float *Us = static_cast<const float *>(a.Usrc);
         LinkRing<NC> R = ring_of<NC>(ring4, ring2);
-        dep_wait();
+        dep_wait_launch();
         M3<float> Vb, Ux;
         if constexpr (RECT) {
             Vb = staple_sum_fused<NC>(g, Us, mu, x, a.c0_f, a.c1_f, R, Ux);
@@ -270,7 +272,7 @@ __global__ void __launch_bounds__(VS_RING_THREADS, RECT ? VS_RING_MINB : 4) k_fl
         const int i = sidx(g, x);
         const float *Us = static_cast<const float *>(a.Usrc);
         LinkRing<NC> R = ring_of<NC>(ring4, ring2);
-        dep_wait();
+        dep_wait_launch();
         M3<float> sig, u;
         // the exponent H_S of this link, read before the staple stream so that
         // its latency hides behind it (stage 1 of a step does not read it)

@@ -287,7 +287,7 @@ __device__ __forceinline__ void rows_block(const SubsweepParams &a, int mu, int 
             x = dir_site(g, mu, t);
         i = sidx(g, x);
     }
-    dep_wait();
+    dep_wait_launch();
     if (work) {
         if constexpr (US == 1) {
             // the forward units, then the backward ones on their own: the sum that

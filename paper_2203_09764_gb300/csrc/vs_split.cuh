@@ -40,7 +40,7 @@ __device__ __forceinline__ bool staple_sum_split(const Geo &g, const float *__re
     M3<float> F, Lp;
     m3_zero(F);
     m3_zero(sig);
-    dep_wait();
+    dep_wait_launch();
     const auto fetch = [&](auto sign, auto entry, auto slot) {
         const float *b;
         int q;
@@ -173,11 +173,11 @@ __global__ void __launch_bounds__(kSplitThreads, 4) k_flow_split(FlowParams a, i
 
 // Up to this many links per launch three warps share 32 links.  us per class launch
 // with one warp / three, 18 reals: over-improved 1024 links 12.3 / 5.5, 3456 15.7 /
-// 6.7, 10,368 16.1 / 16.0, 16,384 11.8 / 9.7, 24,576 15.9 / 14.4, 32,768 22.4 / 17.7,
-// 49,152 24.2 / 25.9 (two warps, one per sign, run two code paths at a time and
-// lose to either: 6.5, 8.1, 13.0, 14.0, 16.3, 22.1, 29.5); plaquette staples 1024 5.0 / 2.9, 6912 6.2 / 4.2, 10,368 6.2 /
-// 5.5, 16,384 4.4 / 4.6.
-constexpr int kSplitMost = 32768, kSplitMostPlain = 12288;
+// 6.7, 10,368 16.3 / 16.0, 16,384 13.0 / 9.8, 24,576 15.9 / 14.3, 32,768 17.1 / 17.7
+// (12 reals 16.2 / 18.4); two warps, one per sign, run two code paths at a time and
+// lose to either (6.5, 8.1, 13.0, 14.0, 16.3, 22.1).  Plaquette staples 1024 5.0 /
+// 2.9, 6912 6.2 / 4.2, 10,368 6.2 / 5.5, 16,384 4.4 / 4.6.
+constexpr int kSplitMost = 28672, kSplitMostPlain = 12288;
 
 inline bool split_launch(bool rect, long long links) { return links <= (rect ? kSplitMost : kSplitMostPlain); }
 

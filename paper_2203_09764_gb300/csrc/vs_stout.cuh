@@ -345,14 +345,22 @@ __device__ __forceinline__ M3<T> stout_candidate(const M3<T> &sig, const M3<T> &
 
 // Class launches depend on the one before them.  With programmatic stream
 // serialisation a launch comes onto the SMs while the previous one drains and
-// waits there (dep_wait) for it to complete before it reads a link or a label; it
-// lets its own successor in only after that, so that no more than two launches
-// share the SMs (earlier, blocks of several launches pile up on some SMs: 41 us
-// instead of 16 for a launch of 81 blocks).  Without it a launch costs ~3 us more:
-// 1024 links 8.2 -> 5.5 us (plaquette staples 6.2 -> 2.9), 165,888 links 71.3 ->
-// 68.7, 524,288 links 165.7 -> 163.4 (88.7 -> 85.6).
-__device__ __forceinline__ void dep_wait() {
-    asm volatile("griddepcontrol.wait;\n griddepcontrol.launch_dependents;" ::: "memory");
+// waits there (dep_wait) for it to complete before it reads a link or a label.
+// Without it a launch costs ~3 us more: 1024 links 8.2 -> 5.5 us (plaquette staples
+// 6.2 -> 2.9), 165,888 links 71.3 -> 68.7, 524,288 links 165.7 -> 163.4 (88.7 -> 85.6).
+// A launch lets its own successor in (dep_launch) never before its wait, so that no
+// more than two launches share the SMs (earlier, blocks of several launches pile up on
+// some SMs: 41 us instead of 16 for a launch of 81 blocks).  The over-improved kernels
+// with a thread per link do it after the staple sum: the successor's blocks, placed on
+// whatever SMs have room, then hold their places for the update only (32,768 links
+// 22.4 -> 17.1 us, 49,152 24.2 -> 23.6, 524,288 163.0 -> 162.4).  The short launches of
+// the other kernels do it at once (with three warps per 32 links 3456 links take 6.6 us
+// that way and 8.1 the other, plaquette staples at 32,768 links 6.1 and 7.3).
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void dep_wait_launch() {
+    dep_wait();
+    dep_launch();
 }
 
 template <class... A, class... B>
@@ -931,7 +939,7 @@ __global__ void __launch_bounds__(VS_RING_THREADS, 4) k_subsweep_pring(SubsweepP
         const int i = sidx(g, x);
         const float *Us = static_cast<const float *>(a.Usrc);
         LinkRing<NC> R = ring_of<NC>(ring4, ring2);
-        dep_wait();
+        dep_wait_launch();
         const M3<float> sig = staple_sum_plain_ring<NC>(g, Us, MU, x, a.c0_f, R);
         const M3<float> Ux = load_link<float, NC>(Us, g.P, MU, i);
         stout_store<float, NC>(a, MU, x, i, sig, Ux, u);
@@ -956,6 +964,7 @@ __global__ void __launch_bounds__(VS_RING_THREADS, VS_RING_MINB) k_subsweep_fuse
         dep_wait();
         M3<float> Ux;
         M3<float> sig = staple_sum_fused<NC>(g, static_cast<const float *>(a.Usrc), MU, x, a.c0_f, a.c1_f, R, Ux);
+        dep_launch();
         stout_store<float, NC>(a, MU, x, i, sig, Ux, u);
     }
     count_update<float>(a.counters, u);
@@ -1077,6 +1086,7 @@ __global__ void __launch_bounds__(VS_RING_THREADS, VS_RING_MINB) k_aus_ring(AusP
         dep_wait();
         M3<float> Ux;
         const M3<float> Vb = staple_sum_fused<NC>(g, static_cast<const float *>(a.U), MU, x, a.c0_f, a.c1_f, R, Ux);
+        dep_launch();
         aus_finish<float, NC>(a, MU, x, i, Vb, Ux, up);
     }
     count_update<float>(a.counters, up);
@@ -1099,7 +1109,7 @@ __global__ void __launch_bounds__(VS_RING_THREADS, 4) k_aus_pring(AusParams a) {
         const int i = sidx(g, x);
         const float *Us = static_cast<const float *>(a.U);
         LinkRing<NC> R = ring_of<NC>(ring4, ring2);
-        dep_wait();
+        dep_wait_launch();
         const M3<float> Vb = staple_sum_plain_ring<NC>(g, Us, MU, x, a.c0_f, R);
         const M3<float> Ux = load_link<float, NC>(Us, g.P, MU, i);
         aus_finish<float, NC>(a, MU, x, i, Vb, Ux, up);
@@ -1147,7 +1157,7 @@ __global__ void __launch_bounds__(VS_RING_THREADS, RECT ? VS_RING_MINB : 4) k_su
         const int i = sidx(g, x);
         const float *Us = static_cast<const float *>(a.Usrc);
         LinkRing<NC> R = ring_of<NC>(ring4, ring2);
-        dep_wait();
+        dep_wait_launch();
         M3<float> sig, Ux;
         if constexpr (RECT) {
             sig = staple_sum_fused<NC>(g, Us, mu, x, a.c0_f, a.c1_f, R, Ux);
