@@ -35,7 +35,7 @@ cudaError_t launch_ape_tpl(bool rect, int mu, const ApeParams &p, cudaStream_t s
             {k_ape_ring<NC, false, 0>, k_ape_ring<NC, false, 1>, k_ape_ring<NC, false, 2>, k_ape_ring<NC, false, 3>},
             {k_ape_ring<NC, true, 0>, k_ape_ring<NC, true, 1>, k_ape_ring<NC, true, 2>, k_ape_ring<NC, true, 3>}};
         static std::atomic<unsigned long long> set[2] = {{0}, {0}};
-        return launch_ring(kernels[rect], mu, p, p.colour >= 0 ? class_threads(p.g, p.n_threads) : p.n_threads,
+        return launch_ring(kernels[rect], mu, p, p.colour >= 0 ? class_threads<NC>(p.g, p.n_threads) : p.n_threads,
                            ring6_smem_bytes<NC>(), set[rect], st);
     }
 }

@@ -148,19 +148,26 @@ __device__ __forceinline__ Pt class_site(const Geo &g, int MU, int c, int t) {
 }
 
 // Number of the class site that thread k of a class launch of n links takes, n or
-// more for an idle thread: site k, except in rows of 20 sites (Lx/4 = 5).  There a
-// row's class sites are a run of five positions in a line of eight, and a warp that
-// takes 32 sites in order touches parts of 7 or 8 runs with every load; it takes six
-// whole runs and leaves two lanes idle (20^3x40, 18 reals: 51.3 -> 48.2 us per class
-// launch, MaxReTr 52.5 -> 49.6).  Rows of 24, five runs of six to a warp, are slower
-// that way: 68.6 -> 69.6 us at 24^3x48, 61.2 -> 64.0 with 12 reals.
+// more for an idle thread: site k, except for 18-real links in rows of 20 sites
+// (Lx/4 = 5).  There a row's class sites are a run of five positions in a line of
+// eight, and a warp that takes 32 sites in order touches parts of 7 or 8 runs with
+// every load; it takes six whole runs and leaves two lanes idle (20^3x40: 51.3 -> 48.2
+// us per class launch, MaxReTr 52.5 -> 49.6).  Rows of 24, five runs of six to a warp,
+// are slower that way: 68.6 -> 69.6 us at 24^3x48, 61.2 -> 64.0 with 12 reals.  With 12
+// reals rows of 20 gain 0.3 us of 40.3, but the mapping costs the kernel registers
+// (spills of 28-44 bytes instead of 0-28) and every other size pays for it: without it
+// 62.0 -> 61.1 us at 165,888 links, 170.1 -> 169.0 at 524,288.
+template <int NC>
 __device__ __forceinline__ int class_thread(const Geo &g, int k, int n) {
-    if (g.Q != 5) return k;
+    if (NC != 18 || g.Q != 5) return k;
     return (k & 31) < 30 ? k - 2 * (k >> 5) : n;
 }
 
 // Threads of a class launch of n links.
-inline int class_threads(const Geo &g, int n) { return g.Q != 5 ? n : (n + 29) / 30 * 32; }
+template <int NC>
+int class_threads(const Geo &g, int n) {
+    return NC != 18 || g.Q != 5 ? n : (n + 29) / 30 * 32;
+}
 
 // --------------------------------------------------------------------------
 // 3x3 complex matrices in registers

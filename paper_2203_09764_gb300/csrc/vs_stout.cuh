@@ -930,7 +930,7 @@ __global__ void __launch_bounds__(VS_RING_THREADS, 4) k_subsweep_pring(SubsweepP
     float4 *ring4 = pring_dyn;
     float2 *ring2 = reinterpret_cast<float2 *>(pring_dyn + 6 * (NC / 4) * VS_RING_THREADS);
     int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (a.colour >= 0) t = class_thread(a.g, t, a.n_threads);
+    if (a.colour >= 0) t = class_thread<NC>(a.g, t, a.n_threads);
     const bool active = t < a.n_threads;
     Update<float> u;
     if (active) {
@@ -953,7 +953,7 @@ __global__ void __launch_bounds__(VS_RING_THREADS, VS_RING_MINB) k_subsweep_fuse
     float4 *ring4 = ring6_dyn;
     float2 *ring2 = reinterpret_cast<float2 *>(ring6_dyn + 6 * (NC / 4) * VS_RING_THREADS);
     int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (a.colour >= 0) t = class_thread(a.g, t, a.n_threads);
+    if (a.colour >= 0) t = class_thread<NC>(a.g, t, a.n_threads);
     const bool active = t < a.n_threads;
     Update<float> u;
     if (active) {
@@ -1075,7 +1075,7 @@ __global__ void __launch_bounds__(VS_RING_THREADS, VS_RING_MINB) k_aus_ring(AusP
     float4 *ring4 = aus_dyn;
     float2 *ring2 = reinterpret_cast<float2 *>(aus_dyn + 6 * (NC / 4) * VS_RING_THREADS);
     int t = blockIdx.x * blockDim.x + threadIdx.x;
-    t = class_thread(a.g, t, a.n_threads);
+    t = class_thread<NC>(a.g, t, a.n_threads);
     const bool active = t < a.n_threads;
     Update<float> up;
     if (active) {
@@ -1100,7 +1100,7 @@ __global__ void __launch_bounds__(VS_RING_THREADS, 4) k_aus_pring(AusParams a) {
     float4 *ring4 = ausp_dyn;
     float2 *ring2 = reinterpret_cast<float2 *>(ausp_dyn + 6 * (NC / 4) * VS_RING_THREADS);
     int t = blockIdx.x * blockDim.x + threadIdx.x;
-    t = class_thread(a.g, t, a.n_threads);
+    t = class_thread<NC>(a.g, t, a.n_threads);
     const bool active = t < a.n_threads;
     Update<float> up;
     if (active) {
