@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(VS_RING_THREADS, RECT ? VS_RING_MINB : 4) k_ap
             Vb = staple_sum_fused<NC>(g, Us, MU, x, a.c0_f, a.c1_f, R, Ux);
         } else {
             Vb = staple_sum_plain_ring<NC>(g, Us, MU, x, a.c0_f, R);
-            Ux = load_link<float, NC>(Us, g.P, MU, i);
+            Ux = load_link<float, NC, kLive>(Us, g.P, MU, i);
         }
         if (RECT) dep_launch();
         ape_finish<float, NC>(a, MU, x, i, Vb, Ux, up);
@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(VS_RING_THREADS, RECT ? VS_RING_MINB : 4) k_ap
             Vb = staple_sum_fused<NC>(g, Us, mu, x, a.c0_f, a.c1_f, R, Ux);
         } else {
             Vb = staple_sum_plain_ring<NC>(g, Us, mu, x, a.c0_f, R);
-            Ux = load_link<float, NC>(Us, g.P, mu, i);
+            Ux = load_link<float, NC, kLive>(Us, g.P, mu, i);
         }
         ape_finish<float, NC>(a, mu, x, i, Vb, Ux, up);
     }
@@ -279,12 +279,12 @@ __global__ void __launch_bounds__(VS_RING_THREADS, RECT ? VS_RING_MINB : 4) k_fl
         float s_old[9];
         const float *Sp = static_cast<const float *>(a.S) + (long long)mu * 9 * g.P + i;
 #pragma unroll
-        for (int k = 0; k < 9; ++k) s_old[k] = a.b_f != 0.0f ? __ldg(Sp + (long long)k * g.P) : 0.0f;
+        for (int k = 0; k < 9; ++k) s_old[k] = a.b_f != 0.0f ? Sp[(long long)k * g.P] : 0.0f;
         if constexpr (RECT) {
             sig = staple_sum_fused<NC>(g, Us, mu, x, a.c0_f, a.c1_f, R, u);
         } else {
             sig = staple_sum_plain_ring<NC>(g, Us, mu, x, a.c0_f, R);
-            u = load_link<float, NC>(Us, g.P, mu, i);
+            u = load_link<float, NC, kLive>(Us, g.P, mu, i);
         }
         flow_finish<float, NC>(a, mu, i, sig, u, used64, s_old);
     }

@@ -467,36 +467,47 @@ __device__ __forceinline__ void rebuild_row2(M3<T> &m) {
     }
 }
 
+// A vector of a link.  The read-only path (__ldg) is for data that no one writes while
+// the reading kernel runs.  A dependent launch (dep_wait in vs_stout.cuh) is on the SMs
+// while the launch before it still writes links: it reads them with ordinary loads
+// (LIVE), which the compiler keeps behind its wait.
+constexpr bool kLive = true;
+template <bool LIVE, class V>
+__device__ __forceinline__ V load_vec(const V *p) {
+    if constexpr (LIVE) return *p;
+    else return __ldg(p);
+}
+
 // The stored reals of a link (row 2 of 12-real links not yet rebuilt).
-template <class T, int NC>
-__device__ __forceinline__ M3<T> load_link_raw(const T *__restrict__ U, long long P, int mu, int i) {
+template <class T, int NC, bool LIVE = false>
+__device__ __forceinline__ M3<T> load_link_raw(const T *U, long long P, int mu, int i) {
     const T *base = U + (long long)mu * NC * P;
     M3<T> m;
     if constexpr (sizeof(T) == 4) {
         const float *b0 = base + blk_off4<NC>(i);
 #pragma unroll
         for (int q = 0; q < NC / 4; ++q) {
-            float4 v = __ldg(reinterpret_cast<const float4 *>(b0 + 64 * q));
+            float4 v = load_vec<LIVE>(reinterpret_cast<const float4 *>(b0 + 64 * q));
             m.re[2 * q] = v.x; m.im[2 * q] = v.y; m.re[2 * q + 1] = v.z; m.im[2 * q + 1] = v.w;
         }
         if (NC == 18) {
-            float2 v = __ldg(reinterpret_cast<const float2 *>(base + blk_off2(i)));
+            float2 v = load_vec<LIVE>(reinterpret_cast<const float2 *>(base + blk_off2(i)));
             m.re[8] = v.x; m.im[8] = v.y;
         }
     } else {
         const T *b0 = base + blk_offd(i);
 #pragma unroll
         for (int e = 0; e < NC / 2; ++e) {
-            double2 v = __ldg(reinterpret_cast<const double2 *>(b0 + 32 * e));
+            double2 v = load_vec<LIVE>(reinterpret_cast<const double2 *>(b0 + 32 * e));
             m.re[e] = v.x; m.im[e] = v.y;
         }
     }
     return m;
 }
 
-template <class T, int NC>
-__device__ __forceinline__ M3<T> load_link(const T *__restrict__ U, long long P, int mu, int i) {
-    M3<T> m = load_link_raw<T, NC>(U, P, mu, i);
+template <class T, int NC, bool LIVE = false>
+__device__ __forceinline__ M3<T> load_link(const T *U, long long P, int mu, int i) {
+    M3<T> m = load_link_raw<T, NC, LIVE>(U, P, mu, i);
     if (NC == 12) rebuild_row2(m);
     return m;
 }

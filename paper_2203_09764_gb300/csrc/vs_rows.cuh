@@ -31,7 +31,7 @@ struct RowLink {
     unsigned m;
 };
 
-__device__ __forceinline__ RowLink row_link(const double *__restrict__ base, int i, bool dag) {
+__device__ __forceinline__ RowLink row_link(const double *base, int i, bool dag) {
     RowLink L;
     L.p = base + blk_offd(i);
     L.rs = dag ? 32 : 96;
@@ -41,7 +41,7 @@ __device__ __forceinline__ RowLink row_link(const double *__restrict__ base, int
 }
 
 __device__ __forceinline__ double2 row_entry(const RowLink &L, int k, int j) {
-    double2 v = __ldg(reinterpret_cast<const double2 *>(L.p + k * L.rs + j * L.cs));
+    double2 v = load_vec<kLive>(reinterpret_cast<const double2 *>(L.p + k * L.rs + j * L.cs));
     v.y = __hiloint2double(__double2hiint(v.y) ^ (int)L.m, __double2loint(v.y));
     return v;
 }
@@ -88,7 +88,7 @@ struct RowUnit {
 //   Sigma = c1 F U_mu^dag(x+mu) + sum [c1 U_mu^dag(x-mu) G H B + c0 A B + c1 A T0 T1 T2] C
 // (without rectangles sig = sum A B C, unscaled).
 template <bool RECT, int UNITS>
-__device__ __forceinline__ void row_units(const Geo &g, const double *__restrict__ U, const Pt &x, int i0, int mu,
+__device__ __forceinline__ void row_units(const Geo &g, const double *U, const Pt &x, int i0, int mu,
                                           int u0, int du, int r, double c0, double c1, Row &sig, Row &F) {
     RowUnit S;
     S.i0 = i0;
@@ -452,7 +452,7 @@ __device__ __forceinline__ void rows_block(const SubsweepParams &a, int mu, int 
             if (sh.keep[l]) *reinterpret_cast<double2 *>(dst + 32 * e) = sh.un[e][l];
             else if (a.U != a.Usrc)
                 *reinterpret_cast<double2 *>(dst + 32 * e) =
-                    __ldg(reinterpret_cast<const double2 *>(Umu + blk_offd(i) + 32 * e));
+                    load_vec<kLive>(reinterpret_cast<const double2 *>(Umu + blk_offd(i) + 32 * e));
         }
     }
 }

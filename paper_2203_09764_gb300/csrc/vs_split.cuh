@@ -22,7 +22,7 @@ constexpr int kSplit = 3, kSplitThreads = 32 * kSplit;   // warps per 32 links
 // Staple sum of link (x, mu) and the link, complete in the first warp (returns
 // true there).  Every thread of the block calls it.
 template <int NC, bool RECT>
-__device__ __forceinline__ bool staple_sum_split(const Geo &g, const float *__restrict__ U, int mu, const Pt &x,
+__device__ __forceinline__ bool staple_sum_split(const Geo &g, const float *U, int mu, const Pt &x,
                                                  float c0, float c1, float4 *shared, M3<float> &sig, M3<float> &Ux) {
     constexpr int BT = kSplitThreads;
     const LinkRing<NC, BT> R = ring_of<NC, BT>(shared, reinterpret_cast<float2 *>(shared + 6 * (NC / 4) * BT));
@@ -51,7 +51,7 @@ __device__ __forceinline__ bool staple_sum_split(const Geo &g, const float *__re
         // entries 0-5 of the first unit
         fetch(Int<1>(), Int<0>(), Int<0>()); fetch(Int<1>(), Int<1>(), Int<1>()); fetch(Int<1>(), Int<2>(), Int<2>());
         fetch(Int<1>(), Int<3>(), Int<3>()); fetch(Int<1>(), Int<4>(), Int<4>()); fetch(Int<1>(), Int<5>(), Int<5>());
-        const M3<float> Lm = m3_dag(load_link<float, NC>(U, P, mu, A.i0 + A.dmm1));
+        const M3<float> Lm = m3_dag(load_link<float, NC, kLive>(U, P, mu, A.i0 + A.dmm1));
         fused_unit<NC, 1>(R, F, sig, c0, c1, Lm, Umu, Unu, Unu, P, A, A, true, first);
         fused_unit<NC, -1>(R, F, sig, c0, c1, Lm, Umu, Unu, Unu, P, A, A, true, first);
         asm volatile("cp.async.wait_group 0;\n" ::: "memory");
@@ -62,7 +62,7 @@ __device__ __forceinline__ bool staple_sum_split(const Geo &g, const float *__re
     } else {
         fetch(Int<1>(), Int<0>(), Int<0>()); fetch(Int<1>(), Int<1>(), Int<1>()); fetch(Int<1>(), Int<9>(), Int<2>());
         fetch(Int<-1>(), Int<0>(), Int<3>()); fetch(Int<-1>(), Int<1>(), Int<4>()); fetch(Int<-1>(), Int<9>(), Int<5>());
-        if (first) Ux = load_link<float, NC>(U, P, mu, A.i0);
+        if (first) Ux = load_link<float, NC, kLive>(U, P, mu, A.i0);
         plain_unit<NC, 1>(R, sig, Umu, Unu, P, A, true);
         plain_unit<NC, -1>(R, sig, Umu, Unu, P, A, true);
         asm volatile("cp.async.wait_group 0;\n" ::: "memory");

@@ -345,7 +345,9 @@ __device__ __forceinline__ M3<T> stout_candidate(const M3<T> &sig, const M3<T> &
 
 // Class launches depend on the one before them.  With programmatic stream
 // serialisation a launch comes onto the SMs while the previous one drains and
-// waits there (dep_wait) for it to complete before it reads a link or a label.
+// waits there (dep_wait) for it to complete before it reads a link or a label; links
+// and flow exponents are then read with ordinary loads (kLive), never through the
+// read-only path, which needs them constant for as long as the kernel is resident.
 // Without it a launch costs ~3 us more: 1024 links 8.2 -> 5.5 us (plaquette staples
 // 6.2 -> 2.9), 165,888 links 71.3 -> 68.7, 524,288 links 165.7 -> 163.4 (88.7 -> 85.6).
 // A launch lets its own successor in (dep_launch) never before its wait, so that no
@@ -766,7 +768,7 @@ __device__ __forceinline__ void fused_unit(const LinkRing<NC, BT> &R, M3<float> 
 }
 
 template <int NC>
-__device__ __forceinline__ M3<float> staple_sum_fused(const Geo &g, const float *__restrict__ U, int MU, Pt x, float c0,
+__device__ __forceinline__ M3<float> staple_sum_fused(const Geo &g, const float *U, int MU, Pt x, float c0,
                                                       float c1, const LinkRing<NC> &R, M3<float> &Ux) {
     const long long P = g.P;
     Around A, An;
@@ -790,7 +792,7 @@ __device__ __forceinline__ M3<float> staple_sum_fused(const Geo &g, const float 
         u_link<1, 5>(A, Umu, Unu, b, q); ring_fetch<NC, 5>(R, b, P, q);
     }
     // U_mu^dag(x - mu): rows 0-1 only are used (left factor of two-row products)
-    const M3<float> Lm = m3_dag(load_link<float, NC>(U, P, MU, A.i0 + A.dmm1));
+    const M3<float> Lm = m3_dag(load_link<float, NC, kLive>(U, P, MU, A.i0 + A.dmm1));
     M3<float> Facc, sig;
     m3_zero(Facc);
     m3_zero(sig);
@@ -853,7 +855,7 @@ __device__ __forceinline__ void plain_unit(const LinkRing<NC, BT> &R, M3<float> 
 }
 
 template <int NC>
-__device__ __forceinline__ M3<float> staple_sum_plain_ring(const Geo &g, const float *__restrict__ U, int MU, Pt x,
+__device__ __forceinline__ M3<float> staple_sum_plain_ring(const Geo &g, const float *U, int MU, Pt x,
                                                            float c0, const LinkRing<NC> &R) {
     const long long P = g.P;
     Around A, An;
@@ -941,7 +943,7 @@ __global__ void __launch_bounds__(VS_RING_THREADS, 4) k_subsweep_pring(SubsweepP
         LinkRing<NC> R = ring_of<NC>(ring4, ring2);
         dep_wait_launch();
         const M3<float> sig = staple_sum_plain_ring<NC>(g, Us, MU, x, a.c0_f, R);
-        const M3<float> Ux = load_link<float, NC>(Us, g.P, MU, i);
+        const M3<float> Ux = load_link<float, NC, kLive>(Us, g.P, MU, i);
         stout_store<float, NC>(a, MU, x, i, sig, Ux, u);
     }
     count_update<float>(a.counters, u);
@@ -1111,7 +1113,7 @@ __global__ void __launch_bounds__(VS_RING_THREADS, 4) k_aus_pring(AusParams a) {
         LinkRing<NC> R = ring_of<NC>(ring4, ring2);
         dep_wait_launch();
         const M3<float> Vb = staple_sum_plain_ring<NC>(g, Us, MU, x, a.c0_f, R);
-        const M3<float> Ux = load_link<float, NC>(Us, g.P, MU, i);
+        const M3<float> Ux = load_link<float, NC, kLive>(Us, g.P, MU, i);
         aus_finish<float, NC>(a, MU, x, i, Vb, Ux, up);
     }
     count_update<float>(a.counters, up);
@@ -1163,7 +1165,7 @@ __global__ void __launch_bounds__(VS_RING_THREADS, RECT ? VS_RING_MINB : 4) k_su
             sig = staple_sum_fused<NC>(g, Us, mu, x, a.c0_f, a.c1_f, R, Ux);
         } else {
             sig = staple_sum_plain_ring<NC>(g, Us, mu, x, a.c0_f, R);
-            Ux = load_link<float, NC>(Us, g.P, mu, i);
+            Ux = load_link<float, NC, kLive>(Us, g.P, mu, i);
         }
         stout_store<float, NC>(a, mu, x, i, sig, Ux, u);
     }
