@@ -94,7 +94,8 @@ void vs_destroy(vs_ctx *ctx);
  * stream.  EINVAL: an extent not a positive multiple of 4, more than 2^30
  * plane positions (sites, plus the layout's unused positions when Lx/4 is 5,
  * 6 or 7; see vs_field_describe), or an unknown precision/storage;
- * EUNSUPPORTED: FP64 with 12-real storage. */
+ * ENOMEM: out of memory, or more than 256 GiB of links; EUNSUPPORTED: FP64
+ * with 12-real storage. */
 vs_status vs_field_create(vs_ctx *ctx, const int32_t dims[4], int32_t precision,
                           int32_t storage, void *stream, vs_field **out);
 /* Device memory of a field: the links (4 V x 18 or 12 reals), two label planes

@@ -240,6 +240,9 @@ vs_status vs::field_create(vs_ctx *c, const int32_t dims[4], int32_t precision, 
     if (precision == VS_FP64 && storage == VS_LINK12)
         return fail(VS_EUNSUPPORTED, "vs_field_create: 12-real storage is built for FP32 only");
     CK(cudaSetDevice(c->opt.device));
+    const int link_bytes = (storage == VS_LINK12 ? 12 : 18) * (precision == VS_FP64 ? 8 : 4);
+    if (!links_fit(make_geo(dims).P, link_bytes))
+        return fail(VS_ENOMEM, "vs_field_create: more than 256 GiB of links");
     vs_field *f = new (std::nothrow) vs_field();
     if (!f) return fail(VS_ENOMEM, "vs_field_create: out of host memory");
     f->ctx = c;
@@ -555,6 +558,8 @@ extern "C" vs_status vs_gauge_transform(vs_field *f, const double *G, int32_t wh
     if (f->gauge_on) return fail(VS_EINVAL, "vs_gauge_transform: field already transformed (reload first)");
     CK(cudaSetDevice(f->ctx->opt.device));
     const size_t V = f->g.V;
+    if (!links_fit(f->g.P, 18 * (f->prec == VS_FP64 ? 8 : 4)))   // G, laid out as one direction of 18-real links
+        return fail(VS_ENOMEM, "vs_gauge_transform: more than 64 GiB of gauge matrices");
     if (!f->G) {
         f->G = field_alloc(f, (size_t)f->g.P * 18 * (f->prec == VS_FP64 ? 8 : 4));
         if (!f->G) return fail(VS_ENOMEM, "vs_gauge_transform: allocation failed");

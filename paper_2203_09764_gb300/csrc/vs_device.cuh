@@ -447,10 +447,27 @@ __device__ __forceinline__ void m3_scale(M3<T> &r, T s) {
 // (chunk bytes x 16 before c) + (i mod 16) x (chunk bytes): the chunks of a link
 // sit at compile-time offsets from its first one (a single address per link),
 // and every float4 chunk run of a block starts on a 128-byte line.
+// Offsets are counted in 16-byte vectors, unsigned, and widened to 64 bits on the
+// pointer: a direction of 64 GiB, which the four of a field may not pass (links_fit).
+// (Counted in reals in an int, 18 i passes 2^31 at 119,304,648 positions.)  The
+// widening costs nothing: against the int offsets a class launch takes 0.97-1.01 of
+// the time (524,288 links 162.6 -> 160.3 us, 12 reals 169.3 -> 167.8); with 64-bit
+// products of i all through it took up to 1.02 (stout), 1.03 (Runge-Kutta stages).
+__host__ __device__ constexpr bool links_fit(long long P, int link_bytes) { return P * link_bytes <= 1ll << 36; }
+__host__ __device__ __forceinline__ const char *blk_ptr(const void *plane, int i, int block) {
+    const unsigned u = (unsigned)i;
+    return static_cast<const char *>(plane) + (unsigned long long)(u + (u >> 4) * (unsigned)(block / 16 - 16)) * 16u;
+}
 template <int NC>
-__device__ __forceinline__ int blk_off4(int i) { return 4 * i + (i >> 4) * (16 * NC - 64); }  // float4 chunk 0
-__device__ __forceinline__ int blk_off2(int i) { return 2 * i + (i >> 4) * (16 * 18 - 32) + 256; }  // float2 chunk
-__device__ __forceinline__ int blk_offd(int i) { return 2 * i + (i >> 4) * (16 * 18 - 32); }  // double2 chunk 0
+__host__ __device__ __forceinline__ const float4 *blk_float4(const float *plane, int i) {   // chunk 0
+    return reinterpret_cast<const float4 *>(blk_ptr(plane, i, 64 * NC));
+}
+__host__ __device__ __forceinline__ const float2 *blk_float2(const float *plane, int i) {   // entry 8 of 18-real links
+    return reinterpret_cast<const float2 *>(blk_ptr(plane, i, 1152) + 1024) - (i & 15);
+}
+__host__ __device__ __forceinline__ const double2 *blk_double2(const double *plane, int i) {   // chunk 0
+    return reinterpret_cast<const double2 *>(blk_ptr(plane, i, 2304));
+}
 // row 2 = conj(row 0 x row 1): the third row of an SU(3) matrix from the first two,
 // each component one chain of fused multiply-adds (four operations)
 template <class T>
@@ -484,21 +501,21 @@ __device__ __forceinline__ M3<T> load_link_raw(const T *U, long long P, int mu, 
     const T *base = U + (long long)mu * NC * P;
     M3<T> m;
     if constexpr (sizeof(T) == 4) {
-        const float *b0 = base + blk_off4<NC>(i);
+        const float4 *b0 = blk_float4<NC>(base, i);
 #pragma unroll
         for (int q = 0; q < NC / 4; ++q) {
-            float4 v = load_vec<LIVE>(reinterpret_cast<const float4 *>(b0 + 64 * q));
+            float4 v = load_vec<LIVE>(b0 + 16 * q);
             m.re[2 * q] = v.x; m.im[2 * q] = v.y; m.re[2 * q + 1] = v.z; m.im[2 * q + 1] = v.w;
         }
         if (NC == 18) {
-            float2 v = load_vec<LIVE>(reinterpret_cast<const float2 *>(base + blk_off2(i)));
+            float2 v = load_vec<LIVE>(blk_float2(base, i));
             m.re[8] = v.x; m.im[8] = v.y;
         }
     } else {
-        const T *b0 = base + blk_offd(i);
+        const double2 *b0 = blk_double2(base, i);
 #pragma unroll
         for (int e = 0; e < NC / 2; ++e) {
-            double2 v = load_vec<LIVE>(reinterpret_cast<const double2 *>(b0 + 32 * e));
+            double2 v = load_vec<LIVE>(b0 + 16 * e);
             m.re[e] = v.x; m.im[e] = v.y;
         }
     }
@@ -537,17 +554,15 @@ template <class T, int NC>
 __device__ __forceinline__ void store_link(T *__restrict__ U, long long P, int mu, int i, const M3<T> &m) {
     T *base = U + (long long)mu * NC * P;
     if constexpr (sizeof(T) == 4) {
-        float *b0 = base + blk_off4<NC>(i);
+        float4 *b0 = const_cast<float4 *>(blk_float4<NC>(base, i));
 #pragma unroll
         for (int q = 0; q < NC / 4; ++q)
-            *reinterpret_cast<float4 *>(b0 + 64 * q) =
-                make_float4(m.re[2 * q], m.im[2 * q], m.re[2 * q + 1], m.im[2 * q + 1]);
-        if (NC == 18) *reinterpret_cast<float2 *>(base + blk_off2(i)) = make_float2(m.re[8], m.im[8]);
+            b0[16 * q] = make_float4(m.re[2 * q], m.im[2 * q], m.re[2 * q + 1], m.im[2 * q + 1]);
+        if (NC == 18) *const_cast<float2 *>(blk_float2(base, i)) = make_float2(m.re[8], m.im[8]);
     } else {
-        T *b0 = base + blk_offd(i);
+        double2 *b0 = const_cast<double2 *>(blk_double2(base, i));
 #pragma unroll
-        for (int e = 0; e < NC / 2; ++e)
-            *reinterpret_cast<double2 *>(b0 + 32 * e) = make_double2(m.re[e], m.im[e]);
+        for (int e = 0; e < NC / 2; ++e) b0[16 * e] = make_double2(m.re[e], m.im[e]);
     }
 }
 

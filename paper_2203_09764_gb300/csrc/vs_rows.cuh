@@ -23,25 +23,25 @@ struct Row {      // a row of a 3x3 matrix
 };
 
 // A link as the right factor of a row product: entry (k, j) of it, or of its
-// adjoint, is at p + k rs + j cs, the imaginary part with the sign bit flipped
+// adjoint, is at p[k rs + j cs], the imaginary part with the sign bit flipped
 // by m.  Both orientations are the same code, so lanes may differ in s.
 struct RowLink {
-    const double *p;
+    const double2 *p;
     int rs, cs;
     unsigned m;
 };
 
 __device__ __forceinline__ RowLink row_link(const double *base, int i, bool dag) {
     RowLink L;
-    L.p = base + blk_offd(i);
-    L.rs = dag ? 32 : 96;
-    L.cs = dag ? 96 : 32;
+    L.p = blk_double2(base, i);
+    L.rs = dag ? 16 : 48;
+    L.cs = dag ? 48 : 16;
     L.m = dag ? 0x80000000u : 0u;
     return L;
 }
 
 __device__ __forceinline__ double2 row_entry(const RowLink &L, int k, int j) {
-    double2 v = load_vec<kLive>(reinterpret_cast<const double2 *>(L.p + k * L.rs + j * L.cs));
+    double2 v = load_vec<kLive>(L.p + k * L.rs + j * L.cs);
     v.y = __hiloint2double(__double2hiint(v.y) ^ (int)L.m, __double2loint(v.y));
     return v;
 }
@@ -446,13 +446,11 @@ __device__ __forceinline__ void rows_block(const SubsweepParams &a, int mu, int 
     if (own) {
         // a rejected link keeps its value: nothing to write in place (annealed),
         // the old link into the destination when that is another buffer
-        double *dst = static_cast<double *>(a.U) + (long long)mu * 18 * g.P + blk_offd(i);
+        double2 *dst = const_cast<double2 *>(blk_double2(static_cast<double *>(a.U) + (long long)mu * 18 * g.P, i));
 #pragma unroll
         for (int e = 3 * r; e < 3 * r + 3; ++e) {
-            if (sh.keep[l]) *reinterpret_cast<double2 *>(dst + 32 * e) = sh.un[e][l];
-            else if (a.U != a.Usrc)
-                *reinterpret_cast<double2 *>(dst + 32 * e) =
-                    load_vec<kLive>(reinterpret_cast<const double2 *>(Umu + blk_offd(i) + 32 * e));
+            if (sh.keep[l]) dst[16 * e] = sh.un[e][l];
+            else if (a.U != a.Usrc) dst[16 * e] = load_vec<kLive>(blk_double2(Umu, i) + 16 * e);
         }
     }
 }

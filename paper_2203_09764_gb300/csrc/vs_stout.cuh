@@ -583,15 +583,15 @@ struct LinkRing {
 template <int NC, int SLOT, int BT>
 __device__ __forceinline__ void ring_fetch(const LinkRing<NC, BT> &R, const float *base, long long P, int i) {
     constexpr int NQ = NC / 4;
-    const float *b0 = base + blk_off4<NC>(i);
+    const float4 *b0 = blk_float4<NC>(base, i);
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
-        const float4 *src = reinterpret_cast<const float4 *>(b0 + 64 * q);
+        const float4 *src = b0 + 16 * q;
         const uint32_t dst = R.a4 + (uint32_t)((SLOT * NQ + q) * BT * 16);
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
     }
     if (NC == 18) {
-        const float2 *src = reinterpret_cast<const float2 *>(base + blk_off2(i));
+        const float2 *src = blk_float2(base, i);
         const uint32_t dst = R.a2 + (uint32_t)(SLOT * BT * 8);
         asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(dst), "l"(src) : "memory");
     }
@@ -604,10 +604,10 @@ __device__ __forceinline__ void ring_fetch_if(const LinkRing<NC, BT> &R, const f
                                               bool on) {
     constexpr int NQ = NC / 4;
     const int pr = on ? 1 : 0;
-    const float *b0 = base + blk_off4<NC>(i);
+    const float4 *b0 = blk_float4<NC>(base, i);
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
-        const float4 *src = reinterpret_cast<const float4 *>(b0 + 64 * q);
+        const float4 *src = b0 + 16 * q;
         const uint32_t dst = R.a4 + (uint32_t)((SLOT * NQ + q) * BT * 16);
         asm volatile(
             "{\n .reg .pred p;\n setp.ne.b32 p, %2, 0;\n"
@@ -615,7 +615,7 @@ __device__ __forceinline__ void ring_fetch_if(const LinkRing<NC, BT> &R, const f
             : "memory");
     }
     if (NC == 18) {
-        const float2 *src = reinterpret_cast<const float2 *>(base + blk_off2(i));
+        const float2 *src = blk_float2(base, i);
         const uint32_t dst = R.a2 + (uint32_t)(SLOT * BT * 8);
         asm volatile(
             "{\n .reg .pred p;\n setp.ne.b32 p, %2, 0;\n"
