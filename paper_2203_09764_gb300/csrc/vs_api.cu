@@ -301,7 +301,7 @@ extern "C" void vs_field_destroy(vs_field *f) {
     delete f;
 }
 
-static vs_status ensure_scratch(vs_field *f, size_t bytes) {
+vs_status vs::ensure_scratch(vs_field *f, size_t bytes) {
     if (f->scratch_bytes >= bytes) return VS_OK;
     CK(cudaStreamSynchronize(f->stream));
     field_free(f, f->scratch);

@@ -39,8 +39,8 @@ struct DevicePool {
     void *take(size_t bytes);          // an idle block of this size, or a new one (nullptr: no memory)
     void give(void *p);
     void trim();                       // free every idle block
-    // Free idle blocks, except one for each of the n sizes that a field is about to
-    // take, until the others and `others` more bytes are within `budget`.
+    // Free idle blocks, except one for each of the n sizes that a job is about to
+    // take, until the rest and `others` more bytes are within `budget`.
     void make_room(const size_t *sizes, int n, uint64_t others, uint64_t budget);
 };
 constexpr int kPoolLingerMs = 100;
@@ -111,6 +111,7 @@ constexpr int kFieldBlocks = 5;
 int field_block_sizes(const int32_t dims[4], int32_t precision, int32_t storage, size_t sizes[kFieldBlocks]);
 vs_status field_create(vs_ctx *c, const int32_t dims[4], int32_t precision, int32_t storage, void *stream,
                        DevicePool *pool, vs_field **out);
+vs_status ensure_scratch(vs_field *f, size_t bytes);   // the field's staging block, at least `bytes`
 bool valid_dims(const int32_t dims[4]);
 
 // Enqueue n_sweeps on the field's stream.  want_stats: per-sweep counters and

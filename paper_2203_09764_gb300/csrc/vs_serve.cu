@@ -99,12 +99,14 @@ cudaEvent_t Serve::get_event() {
     return e;
 }
 
+// Staging of a job, one block for the labels on the way in and the links on the way out.
+static uint64_t job_staging(const vs_job &s) {
+    const uint64_t V = (uint64_t)s.dims[0] * s.dims[1] * s.dims[2] * s.dims[3];
+    return s.links_out ? 4 * V * 18 * sizeof(double) : 4 * V;
+}
+
 static uint64_t job_footprint(const vs_job &s) {
-    uint64_t b = field_footprint(s.dims, s.precision, s.storage);
-    uint64_t V = (uint64_t)s.dims[0] * s.dims[1] * s.dims[2] * s.dims[3];
-    if (s.links_out) b += 4 * V * 18 * sizeof(double);   // read-back staging
-    else b += 4 * V;                                      // label staging
-    return b;
+    return field_footprint(s.dims, s.precision, s.storage) + job_staging(s);
 }
 
 // Priority level of a job from its work, 4 V (n_sweeps + n_cool) link
@@ -152,11 +154,14 @@ bool Serve::admit_one(std::unique_lock<std::mutex> &lk) {
             // idle blocks count against the budget, those this job takes only once
             size_t sizes[kFieldBlocks + 1];
             int n = field_block_sizes(jp->spec.dims, jp->spec.precision, jp->spec.storage, sizes);
-            sizes[n++] = jp->footprint - field_footprint(jp->spec.dims, jp->spec.precision, jp->spec.storage);  // staging
+            sizes[n++] = job_staging(jp->spec);
             from->make_room(sizes, n, used, most);
         }
         vs_status st = field_create(ctx, jp->spec.dims, jp->spec.precision, jp->spec.storage, (void *)jp->stream, from,
                                     &jp->f);
+        // at its final size at once: a block outgrown later would stay in the pool beside
+        // its successor, on top of the job's footprint
+        if (st == VS_OK && (!jp->labels.empty() || jp->spec.links_out)) st = ensure_scratch(jp->f, job_staging(jp->spec));
         if (st == VS_OK) {
             if (!jp->labels.empty()) st = vs_load_field(jp->f, nullptr, jp->labels.data(), VS_HOST);
             else st = vs_load_cooled(jp->f, jp->spec.seed, jp->spec.n_cool);
