@@ -74,8 +74,10 @@ typedef struct {
     vs_free_fn free_fn;         /* NULL: cudaFree */
     void *alloc_user;
     uint64_t hbm_budget_bytes;  /* serving admission cap on device bytes; 0 = no cap.  Without allocator
-                                   hooks the blocks of finished jobs are kept, within the cap, for the next
-                                   jobs, and freed when the loop has been idle for 100 ms */
+                                   hooks the blocks of finished jobs are kept for the next jobs, and freed
+                                   when the loop has been idle for 100 ms: together with the running jobs
+                                   they stay within the cap, or without one within the most that jobs have
+                                   taken at a time (at least 1 GiB) */
     int32_t max_slots;          /* serving: jobs on the device at once; 0 -> 8 */
     int32_t max_queue;          /* serving: waiting jobs before VS_EBUSY; 0 -> 1024 */
 } vs_options;

@@ -146,8 +146,8 @@ bool Serve::admit_one(std::unique_lock<std::mutex> &lk) {
         bytes_in_use += jp->footprint;
         peak_bytes = std::max(peak_bytes, bytes_in_use);
         running.push_back(t);
-        // without a budget the idle blocks may take as much as jobs ever did, or 1 GB
-        const uint64_t used = budget ? bytes_in_use : 0, most = budget ? budget : std::max<uint64_t>(peak_bytes, 1u << 30);
+        // without a budget running jobs and idle blocks together may take what jobs ever did, or 1 GB
+        const uint64_t used = bytes_in_use, most = budget ? budget : std::max<uint64_t>(peak_bytes, 1u << 30);
         lk.unlock();
         DevicePool *const from = ctx->opt.alloc ? nullptr : &ctx->pool;
         if (from && !from->empty()) {

@@ -1,6 +1,7 @@
 """Device memory that the serving loop holds, running jobs and kept blocks together, as the driver
 counts it right after a job (kept blocks are freed 100 ms later): within a job's footprint after a job
-that came with labels and took its links out."""
+that came with labels and took its links out, and within the cap, or without one within what jobs have
+taken at a time and at least 1 GiB, when jobs of another shape follow."""
 
 import time
 
@@ -39,3 +40,29 @@ def test_staging_is_within_the_footprint():
     vs.vs_destroy(ctx)
     assert max(held) > footprint - ROUNDING         # seen before the blocks were freed
     assert max(held) <= footprint + ROUNDING
+
+
+@pytest.mark.parametrize("budget", [0, 900 * MIB])
+def test_jobs_of_another_shape_replace_kept_blocks(budget):
+    from paper_2203_09764_gb300 import vs
+    ctx = vs.vs_create(0, hbm_budget_bytes=budget, max_slots=2)
+    small = vs.make_job((32, 32, 32, 32), 0.06, 60, seed=1, n_cool=0)     # 300 MiB
+    large = vs.make_job((32, 32, 32, 64), 0.06, 1, seed=2, n_cool=0)      # 600 MiB
+
+    def both():
+        tickets = [vs.vs_submit(ctx, small), vs.vs_submit(ctx, small)]
+        assert all(vs.vs_poll(ctx, t)["status"] == vs.VS_OK for t in tickets)
+
+    both()
+    vs.vs_poll(ctx, vs.vs_submit(ctx, large))
+    held = []
+    for _ in range(3):
+        time.sleep(0.6)
+        before = _free()
+        both()
+        vs.vs_poll(ctx, vs.vs_submit(ctx, large))
+        held.append(before - _free())
+    peak = vs.vs_serve_stats_get(ctx)["peak_bytes_in_use"]
+    vs.vs_destroy(ctx)
+    assert max(held) > 600 * MIB                     # seen before the blocks were freed
+    assert max(held) <= (budget or max(peak, 1 << 30)) + 2 * ROUNDING
