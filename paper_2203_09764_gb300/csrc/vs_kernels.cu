@@ -286,6 +286,21 @@ template <> struct ShortSum<float> {
     __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
 };
 
+// Sum of 3 - Re Tr P over a site's six plaquettes.  FP64 adds the differences, which
+// are exact near 3: a smooth field's small action keeps its digits, where 18 less the
+// sum of the traces would round at the size of 18.  The FP32 sum of the traces is exact.
+template <class T> struct PlaqSum;
+template <> struct PlaqSum<double> {
+    double v = 0;
+    __device__ __forceinline__ void add(double retr) { v += 3.0 - retr; }
+    __device__ __forceinline__ double value() const { return v; }
+};
+template <> struct PlaqSum<float> {
+    ShortSum<float> tr;
+    __device__ __forceinline__ void add(float retr) { tr.add(retr); }
+    __device__ __forceinline__ double value() const { return 18.0 - tr.value(); }
+};
+
 // Blocks of the measurement kernels: kMeasThreads threads, one wave of resident
 // blocks, grid-stride over the sites.  Both are bound by the latency and the
 // L1/L2 rate of their link loads (1.5 and 6 KB per site), so what counts is warps
@@ -301,7 +316,7 @@ __global__ void __launch_bounds__(kMeasThreads, sizeof(T) == 4 ? kActionPerSM : 
     for (int d = blockIdx.x * blockDim.x + threadIdx.x; d < g.V; d += gridDim.x * blockDim.x) {
         const Pt x = site_of_index(g, d);
         const int i = sidx(g, x);
-        ShortSum<T> tr;
+        PlaqSum<T> s;
 #pragma unroll 1
         for (int mu = 0; mu < 3; ++mu) {
             const M3<T> Umu = load_link<T, NC>(U, g.P, mu, i);
@@ -318,10 +333,10 @@ __global__ void __launch_bounds__(kMeasThreads, sizeof(T) == 4 ? kActionPerSM : 
                 T re = T(0);
 #pragma unroll
                 for (int k = 0; k < 9; ++k) re = fma(X.re[k], Y.re[k], fma(X.im[k], Y.im[k], re));
-                tr.add(re);
+                s.add(re);
             }
         }
-        acc += 18.0 - tr.value();
+        acc += s.value();
     }
     double b = block_sum(acc);
     if (threadIdx.x == 0) partials[blockIdx.x] = b;
@@ -401,7 +416,8 @@ __global__ void __launch_bounds__(kMeasThreads, sizeof(T) == 4 ? kObsPerSM : 2)
     for (int d = blockIdx.x * blockDim.x + threadIdx.x; d < g.V; d += gridDim.x * blockDim.x) {
         const Pt x = site_of_index(g, d);
         const int i = sidx(g, x);
-        ShortSum<T> ss, ssr, sq;
+        PlaqSum<T> ss;
+        ShortSum<T> ssr, sq;
         // the pairings (01, 23), (02, 13), (03, 12) with signs +, -, +, one plane
         // at a time so that the clover code exists once
         T fa[9];
@@ -420,7 +436,7 @@ __global__ void __launch_bounds__(kMeasThreads, sizeof(T) == 4 ? kObsPerSM : 2)
 #pragma unroll
             for (int k = 0; k < 9; ++k) fa[k] = f[k];
         }
-        const double s = (18.0 - ss.value()) * (2.0 / 72.0), sr = ssr.value() / 72.0,
+        const double s = ss.value() * (2.0 / 72.0), sr = ssr.value() / 72.0,
                      q = sq.value() / (4.0 * 9.869604401089358);
         const int lx = lexidx(g, x);
         if (S_site) S_site[lx] = s;
