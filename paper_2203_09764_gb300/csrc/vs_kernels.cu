@@ -283,7 +283,8 @@ template <> struct ShortSum<float> {
         lo += (hi - (s - b)) + (x - b);
         hi = s;
     }
-    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+    // an infinite sum leaves NaN in lo
+    __device__ __forceinline__ double value() const { return lo == lo ? (double)hi + (double)lo : (double)hi; }
 };
 
 // Sum of 3 - Re Tr P over a site's six plaquettes.  FP64 adds the differences, which
