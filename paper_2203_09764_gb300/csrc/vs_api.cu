@@ -520,6 +520,7 @@ static AusParams make_aus_params(vs_field *f, double alpha, double eps, double u
     a.ref = f->ref;
     a.G = f->gauge_on ? f->G : nullptr;
     a.n_threads = f->g.V / 4;
+    a.crowded = f->served;
     a.alpha = alpha;
     a.c0 = (5.0 - 2.0 * eps) / 3.0;
     a.c1 = (eps - 1.0) / (12.0 * u0 * u0);
@@ -641,6 +642,7 @@ static SubsweepParams make_params(vs_field *f, double rho, double eps, double u0
     p.Usrc = f->U;
     p.ref = f->ref;
     p.G = f->gauge_on ? f->G : nullptr;
+    p.crowded = f->served;
     p.rho = rho;
     p.c0 = (5.0 - 2.0 * eps) / 3.0;
     p.c1 = (eps - 1.0) / (12.0 * u0 * u0);

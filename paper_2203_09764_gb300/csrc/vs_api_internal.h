@@ -58,6 +58,7 @@ struct vs_ctx {
 struct vs_field {
     vs_ctx *ctx = nullptr;
     vs::DevicePool *pool = nullptr; // served job: its device blocks come from here and go back
+    bool served = false;            // a job of the serving loop
     vs::Geo g{};
     int prec = VS_FP64;
     int nc = 18;

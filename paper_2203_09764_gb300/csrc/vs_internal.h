@@ -16,6 +16,7 @@ struct SubsweepParams {
     const void *G;       // random gauge transformation (18 reals per site) or null
     int colour;          // 0..3, or -1: every site of direction mu
     int n_threads;
+    int crowded;         // a served job: launches of other jobs share the SMs (read on the host)
     double rho, c0, c1;
     float rho_f, c0_f, c1_f;   // the same, rounded once on the host for the FP32 kernels
     int vp;
@@ -68,6 +69,7 @@ struct AusParams {
     const void *G;       // random gauge transformation or null
     int colour;
     int n_threads;
+    int crowded;         // as in SubsweepParams
     double alpha, c0, c1;
     float alpha_f, c0_f, c1_f;
     int n_hits;

@@ -159,6 +159,7 @@ bool Serve::admit_one(std::unique_lock<std::mutex> &lk) {
         }
         vs_status st = field_create(ctx, jp->spec.dims, jp->spec.precision, jp->spec.storage, (void *)jp->stream, from,
                                     &jp->f);
+        if (st == VS_OK) jp->f->served = true;
         // at its final size at once: a block outgrown later would stay in the pool beside
         // its successor, on top of the job's footprint
         if (st == VS_OK && (!jp->labels.empty() || jp->spec.links_out)) st = ensure_scratch(jp->f, job_staging(jp->spec));

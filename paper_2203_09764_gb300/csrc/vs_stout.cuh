@@ -27,6 +27,7 @@
 // |H| <= 1 and needs no eigenvalues, so it has no degeneracy problem.
 #pragma once
 
+#include <algorithm>
 #include <atomic>
 #include <mutex>
 
@@ -570,6 +571,7 @@ __global__ void __launch_bounds__(VS_SUBSWEEP_THREADS) k_subsweep(SubsweepParams
 #ifndef VS_RING_MINB
 #define VS_RING_MINB (384 / VS_RING_THREADS)
 #endif
+constexpr int kRingPerSM[2] = {4, VS_RING_MINB};   // blocks per SM: plaquette staples, over-improved
 
 template <int NC, int BT = VS_RING_THREADS>   // BT: threads of the block
 struct LinkRing {
@@ -1193,17 +1195,41 @@ cudaError_t launch_links(void (*kernel)(P), const P &p, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-// One launch of a link-ring kernel of direction mu out of its four instantiations.
-// attr_set: where the shared-memory limit has been set, one flag per kernel family.
+// Dynamic shared memory of a launch of `blocks` blocks that need smem bytes each and of
+// which per_sm fit an SM.  Blocks of a dependent launch come in while the launch before it
+// drains, on whatever SMs have room; a launch that fills the chip less than once would then
+// lie per_sm deep on some SMs and thinly on others, and last as long as the deepest.  It
+// takes so much shared memory that no SM holds more of its blocks than an even spread gives.
+// us per class launch, 18 reals, without dependent launches / with them / evenly spread:
+// over-improved 12x16x28x28 (37,632 links) 32.0 / 35.5 / 29.4, 16x12x28x28 (37,632) 18.6 /
+// 19.4 / 16.4; plaquette staples 12x20x20x40 (48,000 links) 17.7 / 18.6 / 14.6.  Not in the
+// serving loop: there the room on an SM is other jobs' (a mix of 12 jobs 24.4 -> 24.65 ms).
+// n_sm, all, reserved, most: the device's SMs, shared memory of an SM, what a block takes on
+// top of its own, and the most that a block may have.
+inline int even_smem(int blocks, int smem, int per_sm, int n_sm, int all, int reserved, int most) {
+    const int need = (blocks + n_sm - 1) / n_sm;
+    return need >= per_sm ? smem : std::max(smem, std::min(most, (all / need - reserved) & ~127));
+}
+
+// One launch of a link-ring kernel of direction mu out of its four instantiations, evenly
+// spread if it has less than per_sm blocks per SM (0: as they come).  attr_set: where the
+// shared-memory limit has been set, one flag per kernel family.
 template <class P>
-cudaError_t launch_ring(void (*const kernels[4])(P), int mu, const P &p, int threads, int smem,
+cudaError_t launch_ring(void (*const kernels[4])(P), int mu, const P &p, int threads, int smem, int per_sm,
                         std::atomic<unsigned long long> &attr_set, cudaStream_t st) {
+    int dev = 0, n_sm = 1, all = 0, reserved = 0, most = smem;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    cudaDeviceGetAttribute(&all, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
+    cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     once_per_device(attr_set, [&] {
         for (int k = 0; k < 4; ++k)
-            cudaFuncSetAttribute(kernels[k], cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            cudaFuncSetAttribute(kernels[k], cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     });
-    return launch_dependent(kernels[mu], (threads + VS_RING_THREADS - 1) / VS_RING_THREADS, VS_RING_THREADS,
-                            (size_t)smem, st, p);
+    const int blocks = (threads + VS_RING_THREADS - 1) / VS_RING_THREADS;
+    return launch_dependent(kernels[mu], blocks, VS_RING_THREADS,
+                            (size_t)even_smem(blocks, smem, per_sm, n_sm, all, reserved, most), st, p);
 }
 
 }  // namespace vs
