@@ -27,6 +27,7 @@ struct Geo {
     int Qp;         // positions of that group in the layout (Q, or 8 for Q = 5, 6, 7)
     int Lxp;        // positions of an x-row: 4 Qp
     int V;          // sites
+    int runs;       // of a class launch: warps take whole runs of sites (class_thread)
     long long P;    // site positions per direction (plane stride): Lxp Ly Lz Lt >= V
 };
 
@@ -38,6 +39,7 @@ __host__ __device__ inline Geo make_geo(const int dims[4]) {
     g.Qp = (g.Q == 5 || g.Q == 6 || g.Q == 7) ? 8 : g.Q;
     g.Lxp = 4 * g.Qp;
     g.V = (int)((long long)dims[0] * dims[1] * dims[2] * dims[3]);
+    g.runs = 0;
     g.P = (long long)g.Lxp * dims[1] * dims[2] * dims[3];
     return g;
 }
@@ -147,26 +149,13 @@ __device__ __forceinline__ Pt class_site(const Geo &g, int MU, int c, int t) {
     return p;
 }
 
-// Number of the class site that thread k of a class launch of n links takes, n or
-// more for an idle thread: site k, except for 18-real links in rows of 20 sites
-// (Lx/4 = 5).  There a row's class sites are a run of five positions in a line of
-// eight, and a warp that takes 32 sites in order touches parts of 7 or 8 runs with
-// every load; it takes six whole runs and leaves two lanes idle (20^3x40: 51.3 -> 48.2
-// us per class launch, MaxReTr 52.5 -> 49.6).  Rows of 24, five runs of six to a warp,
-// are slower that way: 68.6 -> 69.6 us at 24^3x48, 61.2 -> 64.0 with 12 reals.  With 12
-// reals rows of 20 gain 0.3 us of 40.3, but the mapping costs the kernel registers
-// (spills of 28-44 bytes instead of 0-28) and every other size pays for it: without it
-// 62.0 -> 61.1 us at 165,888 links, 170.1 -> 169.0 at 524,288.
+// Number of the class site that thread k of a class launch of n links takes, n or more
+// for an idle thread: site k, or with g.runs (set for a launch by class_threads in
+// vs_stout.cuh) six whole runs of five sites per warp and two idle lanes.
 template <int NC>
-__device__ __forceinline__ int class_thread(const Geo &g, int k, int n) {
-    if (NC != 18 || g.Q != 5) return k;
+__host__ __device__ __forceinline__ int class_thread(const Geo &g, int k, int n) {
+    if (NC != 18 || !g.runs) return k;
     return (k & 31) < 30 ? k - 2 * (k >> 5) : n;
-}
-
-// Threads of a class launch of n links.
-template <int NC>
-int class_threads(const Geo &g, int n) {
-    return NC != 18 || g.Q != 5 ? n : (n + 29) / 30 * 32;
 }
 
 // --------------------------------------------------------------------------
