@@ -14,6 +14,8 @@
 // (nu, s) units of a link also go to two or six lanes of their own.
 #pragma once
 
+#include <algorithm>
+
 #include "vs_stout.cuh"
 
 namespace vs {
@@ -471,6 +473,62 @@ __global__ void __launch_bounds__(kRowThreads, 3) k_subsweep_rows(SubsweepParams
             return;
         }
     rows_block<RECT, US>(a, mu, n_whole * row_links(1) + (b - n_whole) * row_links(US), a.n_threads, shared);
+}
+
+// A launch of n links as blocks of 42 links (one lane per row), 21 (two) and 7 (six), or a
+// thread per link.  A layer of one block per SM takes layer[] us of the FP64 pipe: whole
+// layers go to the first kind and what is left to the cheaper of the first two (they sum in
+// the same order, so that equal links of a launch come out bit-identical), unless blocks of
+// 7 are cheaper for all of it.  Measured (us per class launch, over-improved / plaquette
+// staples; a thread per link in blocks of 128, the last row):
+//   links       64      1024    3456    10368    18432    32768    36864    57600    262144
+//   one lane    94/30   97/31   98/32   170/49   253/73   491/135  495/137  773/213  3364/900
+//   two         55/21   57/23   94/31   182/58            472/140                    3479/1013
+//   six         26/14   27/14   74/36   173/72            505/203                    3919/1556
+//   thread      247/62  247/62  247/62  247/62   247/62   482/117  483/118  726/176      /793
+// A thread per link takes layers of 19,456 links and wins where the last one is nearly
+// full: thread_layers() compares the two by their layers' times and a launch's own (before,
+// the row kernel took every over-improved launch and every plaquette launch below 131,072
+// links: 38,400 links 533/149 where a thread per link takes 485/120).
+template <bool RECT>
+struct RowPlan {
+    static constexpr double layer[3] = {RECT ? 80.0 : 21.4, RECT ? 41.9 : 12.2, RECT ? 15.9 : 6.3};
+    int n_whole;       // blocks of 42 links
+    int rest;          // links left to blocks of 21, or all of them to blocks of 7
+    bool sixes;
+    double us;
+};
+
+template <bool RECT>
+inline RowPlan<RECT> row_plan(int n, int n_sm) {
+    using R = RowPlan<RECT>;
+    const auto blocks = [](int links, int us) { return (links + row_links(us) - 1) / row_links(us); };
+    const auto layers = [&](int links, int us) { return (blocks(links, us) + n_sm - 1) / n_sm; };
+    R r;
+    const int whole = n / (n_sm * row_links(1));   // whole layers
+    r.n_whole = whole * n_sm;
+    r.rest = n - r.n_whole * row_links(1);
+    const double c2 = R::layer[1] * layers(r.rest, 2), c6 = R::layer[2] * layers(n, 6);
+    r.us = R::layer[0] * whole + std::min(R::layer[0], c2);
+    r.sixes = c6 < r.us;
+    if (r.sixes) {
+        r.us = c6;
+        r.n_whole = 0;
+        r.rest = n;
+    } else if (R::layer[0] <= c2) {
+        r.n_whole += blocks(r.rest, 1);
+        r.rest = std::max(0, n - r.n_whole * row_links(1));
+    }
+    return r;
+}
+
+// Whether a thread per link is faster: 237.2 us per layer and 9.6 per launch over-improved,
+// 56.0 and 5.8 with plaquette staples, against the row kernel's plan and 12 or 8 us.
+template <bool RECT>
+inline bool thread_layers(int n, int n_sm) {
+    const int layers = (n + VS_SUBSWEEP_THREADS * n_sm - 1) / (VS_SUBSWEEP_THREADS * n_sm);
+    const double thread = (RECT ? 237.2 : 56.0) * layers + (RECT ? 9.6 : 5.8);
+    return thread < row_plan<RECT>(n, n_sm).us + (RECT ? 12.0 : 8.0);
 }
 
 }  // namespace vs

@@ -537,9 +537,9 @@ __global__ void __launch_bounds__(32) k_redecide(SubsweepParams a) {
     }
 }
 
-// FP64 with plaquette staples: one thread per link of the colour class (or of
-// direction MU when colour < 0), for launches that fill the chip several times.
-template <int MU>
+// FP64: one thread per link of the colour class (or of direction MU when colour < 0), for
+// launches that fill their last layer of blocks (thread_layers in vs_rows.cuh).
+template <bool RECT, int MU>
 __global__ void __launch_bounds__(VS_SUBSWEEP_THREADS) k_subsweep(SubsweepParams a) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const bool active = t < a.n_threads;
@@ -549,7 +549,7 @@ __global__ void __launch_bounds__(VS_SUBSWEEP_THREADS) k_subsweep(SubsweepParams
         Pt x = a.colour >= 0 ? class_site(g, MU, a.colour, t) : dir_site(g, MU, t);
         const int i = sidx(g, x);
         const double *Us = static_cast<const double *>(a.Usrc);
-        M3<double> sig = staple_sum<double, 18, false, MU>(g, Us, x, a.c0, a.c1);
+        M3<double> sig = staple_sum<double, 18, RECT, MU>(g, Us, x, a.c0, a.c1);
         M3<double> Ux = load_link<double, 18>(Us, g.P, MU, i);
         stout_store<double, 18>(a, MU, x, i, sig, Ux, u);
     }
