@@ -124,23 +124,25 @@ __device__ __forceinline__ void ape_finish(const ApeParams &a, int MU, const Pt 
     else if (a.U != a.Usrc) store_link<T, NC>(static_cast<T *>(a.U), g.P, MU, i, u);
 }
 
-// FP64 APE / AUS with unit circle projection: one thread per link of the colour
-// class (annealed, in place) or of direction MU (colour < 0, from Usrc).
-template <bool RECT, int MU>
-__global__ void __launch_bounds__(VS_SUBSWEEP_THREADS) k_ape(ApeParams a) {
+// APE / AUS with unit circle projection from plain loads: one thread per link of the
+// colour class (annealed, in place) or of direction MU (colour < 0, from Usrc).  FP64, and
+// FP32 plaquette staples where plain_ape() says so (four blocks per SM).
+template <class T, int NC, bool RECT, int MU>
+__global__ void __launch_bounds__(VS_SUBSWEEP_THREADS, sizeof(T) == 4 ? 4 : 1) k_ape(ApeParams a) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const bool active = t < a.n_threads;
-    Update<double> up;
+    Update<T> up;
     if (active) {
         const Geo &g = a.g;
         const Pt x = a.colour >= 0 ? class_site(g, MU, a.colour, t) : dir_site(g, MU, t);
         const int i = sidx(g, x);
-        const double *Us = static_cast<const double *>(a.Usrc);
-        const M3<double> Vb = staple_sum<double, 18, RECT, MU>(g, Us, x, a.c0, a.c1);
-        const M3<double> u = load_link<double, 18>(Us, g.P, MU, i);
-        ape_finish<double, 18>(a, MU, x, i, Vb, u, up);
+        const T *Us = static_cast<const T *>(a.Usrc);
+        const T c0 = sizeof(T) == 4 ? T(a.c0_f) : T(a.c0), c1 = sizeof(T) == 4 ? T(a.c1_f) : T(a.c1);
+        const M3<T> Vb = staple_sum<T, NC, RECT, MU>(g, Us, x, c0, c1);
+        const M3<T> u = load_link<T, NC>(Us, g.P, MU, i);
+        ape_finish<T, NC>(a, MU, x, i, Vb, u, up);
     }
-    count_update<double>(a.counters, up);
+    count_update<T>(a.counters, up);
 }
 
 // FP32 colour class, or every link of direction MU (colour < 0): the staple links

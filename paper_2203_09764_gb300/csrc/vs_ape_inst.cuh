@@ -7,13 +7,35 @@
 
 namespace vs {
 
+// Whether a colour class with plaquette staples takes plain loads (k_ape) instead of the
+// link ring.  Where a run of class sites has an odd number of positions, every 16-byte
+// chunk run ends in half a 32-byte sector: the ring's copies pass the L1 cache by and fetch
+// the other half again, plain loads find it there.  With four blocks per SM (58,369 to
+// 77,824 links) all of a launch is resident and that decides; in narrow rows it decides
+// elsewhere, too.  us per class launch, ring / plain loads, 18 reals: rows of 4, 33,792
+// links 13.9 / 12.4, 64,000 24.5 / 19.4, 139,968 46.9 / 40.2; rows of 12, 60,480 20.3 / 16.7, 96,000 25.7 / 28.1,
+// 139,968 39.0 / 37.0; rows of 36, 64,512 15.7 / 14.7, 96,768 20.8 / 25.4; rows of 28 (runs
+// of seven in lines of eight), 64,512 14.8 / 15.6.  12 reals: rows of 4, 109,440 27.4 /
+// 23.2; rows of 12, 67,584 16.2 / 14.5, 110,592 23.5 / 22.6; rows of 36, 64,512 13.4 / 14.4.
+inline bool plain_ape(int nc, int Qp, int links) {
+    int dev = 0, n_sm = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    const int per_sm = ((links + VS_SUBSWEEP_THREADS - 1) / VS_SUBSWEEP_THREADS + n_sm - 1) / n_sm;
+    if (Qp % 2 == 0 || per_sm < (Qp == 1 ? 2 : 4)) return false;
+    if (Qp == 1) return true;
+    if (nc == 12) return Qp == 3;
+    return per_sm == 4 || (Qp == 3 && per_sm % 4 == 0);
+}
+
 // A colour class of direction mu, or every link (mu < 0: simultaneous sweeps).
 template <class T, int NC>
 cudaError_t launch_ape_tpl(bool rect, int mu, const ApeParams &p, cudaStream_t st) {
     if (p.n_threads <= 0) return cudaSuccess;
     if constexpr (sizeof(T) == 8) {
-        static void (*const kernels[2][4])(ApeParams) = {{k_ape<false, 0>, k_ape<false, 1>, k_ape<false, 2>, k_ape<false, 3>},
-                                                         {k_ape<true, 0>, k_ape<true, 1>, k_ape<true, 2>, k_ape<true, 3>}};
+        static void (*const kernels[2][4])(ApeParams) = {
+            {k_ape<T, NC, false, 0>, k_ape<T, NC, false, 1>, k_ape<T, NC, false, 2>, k_ape<T, NC, false, 3>},
+            {k_ape<T, NC, true, 0>, k_ape<T, NC, true, 1>, k_ape<T, NC, true, 2>, k_ape<T, NC, true, 3>}};
         cudaError_t e = cudaSuccess;
         for (int d = mu < 0 ? 0 : mu; e == cudaSuccess && d <= (mu < 0 ? 3 : mu); ++d)
             e = launch_links(kernels[rect][d], p, st);
@@ -30,6 +52,10 @@ cudaError_t launch_ape_tpl(bool rect, int mu, const ApeParams &p, cudaStream_t s
         static void (*const kernels[2])(ApeParams) = {k_ape_all<NC, false>, k_ape_all<NC, true>};
         static std::atomic<unsigned long long> set{0};
         return launch_all<NC>(kernels, rect, p, set, st);
+    } else if (!rect && p.colour >= 0 && plain_ape(NC, p.g.Qp, p.n_threads)) {
+        static void (*const kernels[4])(ApeParams) = {k_ape<T, NC, false, 0>, k_ape<T, NC, false, 1>, k_ape<T, NC, false, 2>,
+                                                      k_ape<T, NC, false, 3>};
+        return launch_links(kernels[mu], p, st);
     } else {
         static void (*const kernels[2][4])(ApeParams) = {
             {k_ape_ring<NC, false, 0>, k_ape_ring<NC, false, 1>, k_ape_ring<NC, false, 2>, k_ape_ring<NC, false, 3>},
