@@ -13,10 +13,11 @@ namespace vs {
 // the other half again, plain loads find it there.  With four blocks per SM (58,369 to
 // 77,824 links) all of a launch is resident and that decides; in narrow rows it decides
 // elsewhere, too.  us per class launch, ring / plain loads, 18 reals: rows of 4, 33,792
-// links 13.9 / 12.4, 64,000 24.5 / 19.4, 139,968 46.9 / 40.2; rows of 12, 60,480 20.3 / 16.7, 96,000 25.7 / 28.1,
-// 139,968 39.0 / 37.0; rows of 36, 64,512 15.7 / 14.7, 96,768 20.8 / 25.4; rows of 28 (runs
-// of seven in lines of eight), 64,512 14.8 / 15.6.  12 reals: rows of 4, 109,440 27.4 /
-// 23.2; rows of 12, 67,584 16.2 / 14.5, 110,592 23.5 / 22.6; rows of 36, 64,512 13.4 / 14.4.
+// links 13.9 / 12.4, 64,000 24.5 / 19.4, 139,968 46.9 / 40.2; rows of 12, 60,480 20.3 /
+// 16.7, 96,000 25.7 / 28.1, 139,968 39.0 / 37.0; rows of 36, 64,512 15.7 / 14.7, 96,768
+// 20.8 / 25.4; rows of 28 (runs of seven in lines of eight), 64,512 14.8 / 15.6.  12 reals:
+// rows of 4, 109,440 27.4 / 23.2; rows of 12, 67,584 16.2 / 14.5, 110,592 23.5 / 22.6; rows
+// of 36, 64,512 13.4 / 14.4.
 inline bool plain_ape(int nc, int Qp, int links) {
     int dev = 0, n_sm = 1;
     cudaGetDevice(&dev);
