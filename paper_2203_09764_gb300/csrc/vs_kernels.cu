@@ -521,13 +521,14 @@ __global__ void k_correlation_finish(const double *__restrict__ partials, int nb
 // Vortex check
 // ---------------------------------------------------------------------------
 
-// One thread per site, its four links.  dz: per link (current - reference label)
+// One thread per site, its four links; in FP64 on fields of few sites (kLinkSites) one per
+// link, direction blockIdx.y.  dz: per link (current - reference label)
 // mod 3 in {0, 1, 2}, all that the charges need.  A warp's smallest margin goes
 // to the global minimum only if it is below the value read there: with one
 // 64-bit atomicMin per warp of links, all to one address, this kernel took
 // 0.21 ms at 32^3x64 whatever it read.  Without a gauge only the diagonals are
 // loaded (40 of 72 bytes per FP32 link, 335 MB: 0.05 ms at the copy rate).
-template <class T, int NC, bool GAUGE>
+template <class T, int NC, bool GAUGE, bool LINK>
 __global__ void __launch_bounds__(kThreads) k_vortex_links(Geo g, const T *__restrict__ U,
                                                             const int8_t *__restrict__ ref, int8_t *dz,
                                                             unsigned long long *counts, unsigned long long *mbits,
@@ -537,7 +538,8 @@ __global__ void __launch_bounds__(kThreads) k_vortex_links(Geo g, const T *__res
     int n_diff = 0, n_near = 0;
     double margin = 1e300;
 #pragma unroll
-    for (int mu = 0; mu < 4; ++mu) {
+    for (int j = 0; j < (LINK ? 1 : 4); ++j) {
+        const int mu = LINK ? (int)blockIdx.y : j;
         const M3<T> m = load_link<T, NC>(U, g.P, mu, i);
         T a, b;
         if constexpr (GAUGE) vp_trace<T>(G, g.P, i, i + shift_delta(g, x, mu, 1), m, a, b);
@@ -936,30 +938,38 @@ cudaError_t launch_correlation(const double *a, const double *b, long long n, do
 
 cudaError_t preload_vortex_kernels() {
     cudaFuncAttributes a;
-    cudaError_t e = cudaFuncGetAttributes(&a, k_vortex_links<double, 18, false>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_vortex_links<float, 18, false>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_vortex_links<float, 12, false>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_vortex_links<double, 18, true>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_vortex_links<float, 18, true>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_vortex_links<float, 12, true>);
+    cudaError_t e = cudaFuncGetAttributes(&a, k_vortex_links<double, 18, false, false>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_vortex_links<double, 18, false, true>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_vortex_links<float, 18, false, false>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_vortex_links<float, 12, false, false>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_vortex_links<double, 18, true, false>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_vortex_links<double, 18, true, true>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_vortex_links<float, 18, true, false>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_vortex_links<float, 12, true, false>);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k_vortex_charges);
     return e;
 }
 
-template <class T, int NC>
+// Up to this many sites an FP64 check takes a thread per link: a site's four atan2 in a row
+// then last longer than the links' loads (us per check, per site / per link: 4^4 42.0 / 29.7,
+// 12^3x24 67.1 / 55.3, 16^3x32 106.8 / 107.4, 24^3x48 403.6 / 458.0).
+constexpr int kLinkSites = 65536;
+
+template <class T, int NC, bool LINK = false>
 static void vortex_links(const Geo &g, const void *U, const int8_t *ref, int8_t *dz, unsigned long long *counts,
                          unsigned long long *mbits, cudaStream_t st, const void *G) {
-    const int b = nblocks(g.V);
+    const dim3 b(nblocks(g.V), LINK ? 4 : 1);
     if (G)
-        k_vortex_links<T, NC, true><<<b, kThreads, 0, st>>>(g, (const T *)U, ref, dz, counts, mbits, (const T *)G);
+        k_vortex_links<T, NC, true, LINK><<<b, kThreads, 0, st>>>(g, (const T *)U, ref, dz, counts, mbits, (const T *)G);
     else
-        k_vortex_links<T, NC, false><<<b, kThreads, 0, st>>>(g, (const T *)U, ref, dz, counts, mbits, nullptr);
+        k_vortex_links<T, NC, false, LINK><<<b, kThreads, 0, st>>>(g, (const T *)U, ref, dz, counts, mbits, nullptr);
 }
 
 cudaError_t launch_vortex(int prec, int nc, const Geo &g, const void *U, const int8_t *ref, int8_t *dz,
                           unsigned long long *counts, unsigned long long *mbits, cudaStream_t st,
                           const void *G) {
-    if (prec == 0) vortex_links<double, 18>(g, U, ref, dz, counts, mbits, st, G);
+    if (prec == 0 && g.V <= kLinkSites) vortex_links<double, 18, true>(g, U, ref, dz, counts, mbits, st, G);
+    else if (prec == 0) vortex_links<double, 18>(g, U, ref, dz, counts, mbits, st, G);
     else if (nc == 18) vortex_links<float, 18>(g, U, ref, dz, counts, mbits, st, G);
     else vortex_links<float, 12>(g, U, ref, dz, counts, mbits, st, G);
     k_vortex_charges<<<nblocks(g.V), kThreads, 0, st>>>(g, dz, counts);
