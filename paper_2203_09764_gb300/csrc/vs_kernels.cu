@@ -79,13 +79,34 @@ __device__ __forceinline__ M3<T> staged_matrix(const double *__restrict__ in, do
     return m;
 }
 
+// The matrix at q, read by its own thread.
+template <class T>
+__device__ __forceinline__ M3<T> direct_matrix(const double *__restrict__ q, double &tr, double &ti) {
+    M3<T> m;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        m.re[k] = T(q[2 * k]);
+        m.im[k] = T(q[2 * k + 1]);
+    }
+    tr = q[0] + q[8] + q[16];
+    ti = q[1] + q[9] + q[17];
+    return m;
+}
+
 // Links from FP64 host layout; the reference label is the sector of arg Tr U of the FP64 input.
-template <class T, int NC>
+// A thread's 18 reads of its matrix find the line of the first in L1, so staging pays only
+// for 18-real links in rows whose runs of 5 or 7 sites leave unused positions (FP64, us
+// staged / direct: 20^3x40 111.3 / 119.6, 28^3x56 309 / 336, but 24^3x48 139.1 / 131.3,
+// 12x40^3 154.5 / 143.5; 12 reals 16^3x32 29.3 / 27.8).
+template <class T, int NC, bool STAGED>
 __global__ void __launch_bounds__(kThreads) k_load_links(Geo g, const double *__restrict__ in, T *U, int8_t *ref) {
-    __shared__ __align__(16) double sm[kThreads * 18];
+    __shared__ __align__(16) double sm[STAGED ? kThreads * 18 : 1];
     const int mu = blockIdx.y, s0 = blockIdx.x * kThreads;
     double tr, ti;
-    const M3<T> m = staged_matrix<T>(in + ((long long)mu * g.V + s0) * 18, sm, tr, ti);
+    const double *first = in + ((long long)mu * g.V + s0) * 18;
+    M3<T> m;
+    if constexpr (STAGED) m = staged_matrix<T>(first, sm, tr, ti);
+    else m = direct_matrix<T>(first + 18 * threadIdx.x, tr, ti);
     const int i = sidx(g, site_of_lex(g, s0 + threadIdx.x));
     store_link<T, NC>(U, g.P, mu, i, m);
     ref[(long long)mu * g.P + i] = (int8_t)z3_label<double>(tr, ti);
@@ -826,9 +847,12 @@ cudaError_t launch_load_labels(int prec, int nc, const Geo &g, const int8_t *lab
 cudaError_t launch_load_links(int prec, int nc, const Geo &g, const double *in, void *U, int8_t *ref,
                               cudaStream_t st) {
     const dim3 b(nblocks(g.V), 4);
-    if (prec == 0) k_load_links<double, 18><<<b, kThreads, 0, st>>>(g, in, (double *)U, ref);
-    else if (nc == 18) k_load_links<float, 18><<<b, kThreads, 0, st>>>(g, in, (float *)U, ref);
-    else k_load_links<float, 12><<<b, kThreads, 0, st>>>(g, in, (float *)U, ref);
+    const bool staged = g.Qp != g.Q && g.Q % 2 && nc == 18;
+    if (prec == 0 && staged) k_load_links<double, 18, true><<<b, kThreads, 0, st>>>(g, in, (double *)U, ref);
+    else if (prec == 0) k_load_links<double, 18, false><<<b, kThreads, 0, st>>>(g, in, (double *)U, ref);
+    else if (staged) k_load_links<float, 18, true><<<b, kThreads, 0, st>>>(g, in, (float *)U, ref);
+    else if (nc == 18) k_load_links<float, 18, false><<<b, kThreads, 0, st>>>(g, in, (float *)U, ref);
+    else k_load_links<float, 12, false><<<b, kThreads, 0, st>>>(g, in, (float *)U, ref);
     count_launches(1);
     return cudaGetLastError();
 }
