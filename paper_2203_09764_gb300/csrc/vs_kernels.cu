@@ -328,11 +328,13 @@ template <> struct PlaqSum<float> {
 // L1/L2 rate of their link loads (1.5 and 6 KB per site), so what counts is warps
 // per SM: 16 for the action (120 registers), 12 for the observables (168), where
 // blocks of 256 threads left 8.  Per call at 32^3x64, FP32: action 395 -> 213 us
-// (five blocks per SM spill: 295), observables 1174 -> 880 us (four: 980).
-constexpr int kMeasThreads = 128, kActionPerSM = 4, kObsPerSM = 3;
+// (five blocks per SM spill: 295), observables 1174 -> 880 us (four: 980).  FP64: two
+// blocks per SM at a time (up to 255 registers); the action takes eight in all, so that the
+// last of its four rounds is short (28^3x56 2996 -> 2957 us).
+constexpr int kMeasThreads = 128, kActionPerSM = 4, kObsPerSM = 3, kMeasFp64PerSM = 2, kActionFp64Blocks = 8;
 
 template <class T, int NC>
-__global__ void __launch_bounds__(kMeasThreads, sizeof(T) == 4 ? kActionPerSM : 2)
+__global__ void __launch_bounds__(kMeasThreads, sizeof(T) == 4 ? kActionPerSM : kMeasFp64PerSM)
     k_action(Geo g, const T *__restrict__ U, double *partials) {
     double acc = 0;
     for (int d = blockIdx.x * blockDim.x + threadIdx.x; d < g.V; d += gridDim.x * blockDim.x) {
@@ -431,7 +433,7 @@ __device__ __forceinline__ T tr_herm(const T a[9], const T b[9]) {
 }
 
 template <class T, int NC>
-__global__ void __launch_bounds__(kMeasThreads, sizeof(T) == 4 ? kObsPerSM : 2)
+__global__ void __launch_bounds__(kMeasThreads, sizeof(T) == 4 ? kObsPerSM : kMeasFp64PerSM)
     k_observables(Geo g, const T *__restrict__ U, double *partials, double *S_site, double *SR_site,
                   double *q_site) {
     double aS = 0, aSR = 0, aQ = 0;
@@ -909,22 +911,21 @@ cudaError_t launch_centrifuge(int prec, int nc, const Geo &g, const int8_t *ref,
     return cudaGetLastError();
 }
 
-// One wave of the resident blocks of a measurement kernel, at most `most` (its partials).
-template <class K>
-static int meas_blocks(K kernel, const Geo &g, int most) {
-    int dev = 0, n_sm = 0, per_sm = 0;
+// Blocks of a measurement kernel: per_sm for each SM, at most `most` (its partials), or a
+// thread per site where `most` blocks suffice for that.
+static int meas_blocks(const Geo &g, int per_sm, int most) {
+    int dev = 0, n_sm = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kMeasThreads, 0);
-    const int wave = std::max(1, n_sm * std::max(per_sm, 1));
-    return std::min(nblocks(g.V, kMeasThreads), std::min(wave, most));
+    const int all = nblocks(g.V, kMeasThreads);
+    return all <= most ? all : std::min(n_sm * per_sm, most);
 }
 
 cudaError_t launch_action(int prec, int nc, const Geo &g, const void *U, double *partials, double *out,
                           cudaStream_t st) {
     int b = 0;
     const auto run = [&](auto kernel, auto *links) {
-        b = meas_blocks(kernel, g, kActionBlocks);
+        b = meas_blocks(g, prec == 0 ? kActionFp64Blocks : kActionPerSM, kActionBlocks);
         kernel<<<b, kMeasThreads, 0, st>>>(g, links, partials);
     };
     if (prec == 0) run(k_action<double, 18>, (const double *)U);
@@ -940,7 +941,7 @@ cudaError_t launch_observables(int prec, int nc, const Geo &g, const void *U, do
                                double *S_site, double *SR_site, double *q_site, cudaStream_t st) {
     int b = 0;
     const auto run = [&](auto kernel, auto *links) {
-        b = meas_blocks(kernel, g, kObsBlocks);
+        b = meas_blocks(g, prec == 0 ? kMeasFp64PerSM : kObsPerSM, kObsBlocks);
         kernel<<<b, kMeasThreads, 0, st>>>(g, links, partials, S_site, SR_site, q_site);
     };
     if (prec == 0) run(k_observables<double, 18>, (const double *)U);
