@@ -178,7 +178,7 @@ __global__ void __launch_bounds__(VS_RING_THREADS, RECT ? VS_RING_MINB : 4) k_ap
     count_update<float>(a.counters, up);
 }
 
-// The same for every link, from Usrc (simultaneous sweeps).
+// FP32, every link from Usrc (simultaneous sweeps).
 template <int NC, bool RECT>
 __global__ void __launch_bounds__(VS_RING_THREADS, RECT ? VS_RING_MINB : 4) k_ape_all(ApeParams a) {
     extern __shared__ float4 ape_dyn[];
@@ -257,9 +257,9 @@ __global__ void __launch_bounds__(VS_SUBSWEEP_THREADS) k_flow_stage(FlowParams a
     flow_count(a, used64);
 }
 
-// The same stage in FP32 with the staple links streamed through the per-thread cp.async ring: the one-pass stream of the class
-// kernel for over-improved staples, the plaquette-staple ring for eps = 1.
-// MU: every direction in one launch (-1), or this one.
+// A stage in FP32 with the staple links streamed through the per-thread cp.async ring: the
+// one-pass stream of the class kernel for over-improved staples, the plaquette-staple ring
+// for eps = 1.  MU: every direction in one launch (-1), or this one.
 template <int NC, bool RECT, int MU>
 __global__ void __launch_bounds__(VS_RING_THREADS, RECT ? VS_RING_MINB : 4) k_flow_stage_ring(FlowParams a) {
     extern __shared__ float4 flow_dyn[];

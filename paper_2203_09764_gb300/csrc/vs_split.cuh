@@ -171,12 +171,23 @@ __global__ void __launch_bounds__(kSplitThreads, 4) k_flow_split(FlowParams a, i
     flow_count(a, used64);
 }
 
-// Up to this many links per launch three warps share 32 links.  us per class launch
-// with one warp / three, 18 reals: over-improved 1024 links 12.3 / 5.5, 3456 15.7 /
-// 6.7, 10,368 16.3 / 16.0, 16,384 13.0 / 9.8, 24,576 15.9 / 14.3, 32,768 17.1 / 17.7
-// (12 reals 16.2 / 18.4); two warps, one per sign, run two code paths at a time and
-// lose to either (6.5, 8.1, 13.0, 14.0, 16.3, 22.1).  Plaquette staples 1024 5.0 /
-// 2.9, 6912 6.2 / 4.2, 10,368 6.2 / 5.5, 16,384 4.4 / 4.6.
+// Up to this many links per launch three warps share 32 links.  The time depends on the
+// row as well as on the links: a class is a run of Lx/4 sites per x-row, and the shorter
+// the run, the more lines every load visits.  us per class launch with one warp / three,
+// 18 reals:
+//   over-improved    rows of 12      16             20             32
+//     3072-5120      15.7 / 6.5                     12.0 / 7.8     9.6 / 5.8
+//     8192-9216      16.1 / 9.8      10.9 / 6.8                    10.0 / 6.4
+//     11,520-12,288  16.3 / 16.1     11.0 / 9.2     12.5 / 12.4    10.2 / 8.2
+//     15,360-16,384  16.5 / 16.4     11.3 / 9.7     12.9 / 12.7
+//     20,480-24,576  29.1 / 20.3     15.5 / 12.3    20.0 / 15.9    14.3 / 13.0
+//     28,672-32,768                  16.1 / 14.3                   14.7 / 17.7
+//   plaquette staples
+//     8192-11,520    6.2 / 4.3       4.3 / 3.3      5.0 / 4.7      4.0 / 3.1
+//     12,288         6.2 / 7.3       4.5 / 4.5                     4.1 / 4.1
+// (12 reals: 28,672 links in rows of 16 15.9 / 17.0, otherwise alike.)  Two warps, one per
+// sign, run two code paths at a time and lose to either (1024 links 6.5, 10,368 13.0,
+// 24,576 16.3).
 constexpr int kSplitMost = 28672, kSplitMostPlain = 12288;
 
 inline bool split_launch(bool rect, long long links) { return links <= (rect ? kSplitMost : kSplitMostPlain); }

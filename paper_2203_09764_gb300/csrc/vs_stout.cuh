@@ -338,8 +338,9 @@ __device__ __forceinline__ M3<T> stout_candidate(const M3<T> &sig, const M3<T> &
     return m3_mul(Mx, Ux);
 }
 
-// Threads of the plain-load FP64 kernels.  128 and not 256: an FP64 thread holds up to 255 registers, two blocks of 128 fit an SM
-// as one of 256 does, and the last, partial layer of blocks is half as long.
+// Threads of the plain-load kernels.  128 and not 256: an FP64 thread holds up to 255
+// registers, two blocks of 128 fit an SM as one of 256 does, and the last, partial layer of
+// blocks is half as long.
 #ifndef VS_SUBSWEEP_THREADS
 #define VS_SUBSWEEP_THREADS 128
 #endif
@@ -353,12 +354,15 @@ __device__ __forceinline__ M3<T> stout_candidate(const M3<T> &sig, const M3<T> &
 // 6.2 -> 2.9), 165,888 links 71.3 -> 68.7, 524,288 links 165.7 -> 163.4 (88.7 -> 85.6).
 // A launch lets its own successor in (dep_launch) never before its wait, so that no
 // more than two launches share the SMs (earlier, blocks of several launches pile up on
-// some SMs: 41 us instead of 16 for a launch of 81 blocks).  The over-improved kernels
-// with a thread per link do it after the staple sum: the successor's blocks, placed on
-// whatever SMs have room, then hold their places for the update only (32,768 links
+// some SMs: 41 us instead of 16 for a launch of 81 blocks).  The over-improved class
+// kernels with a thread per link do it after the staple sum: the successor's blocks, placed
+// on whatever SMs have room, then hold their places for the update only (32,768 links
 // 22.4 -> 17.1 us, 49,152 24.2 -> 23.6, 524,288 163.0 -> 162.4).  The short launches of
 // the other kernels do it at once (with three warps per 32 links 3456 links take 6.6 us
-// that way and 8.1 the other, plaquette staples at 32,768 links 6.1 and 7.3).
+// that way and 8.1 the other, plaquette staples at 32,768 links 6.1 and 7.3), and so do
+// the launches over every direction, where the place hardly matters (per direction, at
+// once / after the staple sum, over-improved: simultaneous stout at 24^4 111.5 / 111.5 us,
+// Runge-Kutta stage at 32^4 299.7 / 298.5).
 __device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void dep_wait_launch() {
@@ -1126,13 +1130,16 @@ __global__ void __launch_bounds__(VS_RING_THREADS, 4) k_aus_pring(AusParams a) {
 // of kAllGroup per direction, direction after direction, so that the directions of the
 // same sites run at the same time and share their links in L2.  Against a launch per
 // direction: small lattices save three launches of four and fill the chip (flow stage
-// with eps = 1, per direction: 1024 sites 4.6 -> 1.1 us, 16,384 sites 9.1 -> 6.5);
+// with eps = 1, per direction: 4096 sites 4.6 -> 1.1 us, 65,536 sites 9.1 -> 6.5);
 // from 262,144 sites on, the links' way from L2 into the SMs (1.4 KB per link, 17 TB/s)
 // is the bound and the order changes little (177.7 -> 177.3 us at 32^3x64).
 // Over-improved staples need every register, and a direction known at compile time
 // saves a few: above kAllMostRect sites they keep a launch per direction (1,048,576
 // sites, APE 362 us per direction against 356; 663,552 sites 245 against 249).
-constexpr int kAllGroup = 114;   // a quarter of the resident blocks
+// The group is a quarter of the blocks that are resident on 152 SMs at three per SM; the
+// plaquette kernels have four per SM, but groups of 152 change nothing there (simultaneous
+// stout 32^3x64, eps = 1: 176.3 / 176.1 us, 16^4 6.6 / 6.6).
+constexpr int kAllGroup = 114;
 inline bool all_launch(bool rect, int sites) { return !rect || sites <= kAllMostRect; }
 
 // Direction and first-to-last site number of this thread in such a launch; the blocks
@@ -1146,7 +1153,7 @@ __device__ __forceinline__ int all_directions(int threads, int &t) {
     return mu;
 }
 
-// The same for every link, from Usrc.
+// FP32 stout, every link from Usrc (simultaneous sweeps).
 template <int NC, bool RECT>
 __global__ void __launch_bounds__(VS_RING_THREADS, RECT ? VS_RING_MINB : 4) k_subsweep_all(SubsweepParams a) {
     extern __shared__ float4 all_dyn[];
