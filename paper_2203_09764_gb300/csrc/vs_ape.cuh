@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(VS_RING_THREADS, RECT ? VS_RING_MINB : 4) k_ap
     float4 *ring4 = ape_dyn;
     float2 *ring2 = reinterpret_cast<float2 *>(ape_dyn + 6 * (NC / 4) * VS_RING_THREADS);
     int t = blockIdx.x * blockDim.x + threadIdx.x;
-    t = class_thread<NC>(a.g, t, a.n_threads);
+    t = class_thread<NC>(a.colour, t, a.n_threads);
     const bool active = t < a.n_threads;
     Update<float> up;
     if (active) {

@@ -62,7 +62,7 @@ cudaError_t launch_ape_tpl(bool rect, int mu, const ApeParams &p, cudaStream_t s
             {k_ape_ring<NC, false, 0>, k_ape_ring<NC, false, 1>, k_ape_ring<NC, false, 2>, k_ape_ring<NC, false, 3>},
             {k_ape_ring<NC, true, 0>, k_ape_ring<NC, true, 1>, k_ape_ring<NC, true, 2>, k_ape_ring<NC, true, 3>}};
         static std::atomic<unsigned long long> set[2] = {{0}, {0}};
-        return launch_ring<NC>(kernels[rect], mu, p, p.colour >= 0, kRingPerSM[rect], set[rect], st);
+        return launch_ring<NC>(kernels[rect], mu, p, kRingPerSM[rect], set[rect], st);
     }
 }
 
@@ -91,7 +91,7 @@ cudaError_t launch_flow_tpl(bool rect, const FlowParams &p, cudaStream_t st) {
         if (all_launch(rect, p.n_threads)) return launch_all<NC>(all, rect, p, set[0], st);
         cudaError_t e = cudaSuccess;
         for (int d = 0; e == cudaSuccess && d < 4; ++d)
-            e = launch_ring<NC>(each, d, p, false, 0, set[1], st);
+            e = launch_ring<NC>(each, d, p, 0, set[1], st);
         return e;
     }
 }

@@ -27,7 +27,6 @@ struct Geo {
     int Qp;         // positions of that group in the layout (Q, or 8 for Q = 5, 6, 7)
     int Lxp;        // positions of an x-row: 4 Qp
     int V;          // sites
-    int runs;       // of a class launch: warps take whole runs of sites (class_thread)
     long long P;    // site positions per direction (plane stride): Lxp Ly Lz Lt >= V
 };
 
@@ -39,7 +38,6 @@ __host__ __device__ inline Geo make_geo(const int dims[4]) {
     g.Qp = (g.Q == 5 || g.Q == 6 || g.Q == 7) ? 8 : g.Q;
     g.Lxp = 4 * g.Qp;
     g.V = (int)((long long)dims[0] * dims[1] * dims[2] * dims[3]);
-    g.runs = 0;
     g.P = (long long)g.Lxp * dims[1] * dims[2] * dims[3];
     return g;
 }
@@ -150,11 +148,13 @@ __device__ __forceinline__ Pt class_site(const Geo &g, int MU, int c, int t) {
 }
 
 // Number of the class site that thread k of a class launch of n links takes, n or more
-// for an idle thread: site k, or with g.runs (set for a launch by class_threads in
-// vs_stout.cuh) six whole runs of five sites per warp and two idle lanes.
+// for an idle thread: site k, or if the launch's colour carries kRuns (class_threads in
+// vs_stout.cuh; a multiple of 4, which class_site does not see) six whole runs of five
+// sites per warp and two idle lanes.
+constexpr int kRuns = 256;
 template <int NC>
-__host__ __device__ __forceinline__ int class_thread(const Geo &g, int k, int n) {
-    if (NC != 18 || !g.runs) return k;
+__host__ __device__ __forceinline__ int class_thread(int colour, int k, int n) {
+    if (NC != 18 || colour < kRuns) return k;
     return (k & 31) < 30 ? k - 2 * (k >> 5) : n;
 }
 

@@ -16,7 +16,6 @@ struct SubsweepParams {
     const void *G;       // random gauge transformation (18 reals per site) or null
     int colour;          // 0..3, or -1: every site of direction mu
     int n_threads;
-    int crowded;         // a served job: launches of other jobs share the SMs (read on the host)
     double rho, c0, c1;
     float rho_f, c0_f, c1_f;   // the same, rounded once on the host for the FP32 kernels
     int vp;
@@ -28,6 +27,7 @@ struct SubsweepParams {
     unsigned *defer_n;    // entries appended by the class launch (may exceed defer_cap)
     unsigned *defer_done; // blocks of k_redecide that have finished (reset by the last)
     int defer_cap;
+    int crowded;         // a served job: launches of other jobs share the SMs (read on the host)
 };
 
 // Counter slots of one sweep, filled by the colour-class kernels of the
@@ -69,12 +69,12 @@ struct AusParams {
     const void *G;       // random gauge transformation or null
     int colour;
     int n_threads;
-    int crowded;         // as in SubsweepParams
     double alpha, c0, c1;
     float alpha_f, c0_f, c1_f;
     int n_hits;
     int vp;
     unsigned long long *counters;  // kSweepSlots counters of the sweep (kCnt*), or null
+    int crowded;         // as in SubsweepParams
 };
 
 // One colour class (or, colour < 0, every link of direction mu) of APE

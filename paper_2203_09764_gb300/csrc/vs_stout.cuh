@@ -30,6 +30,7 @@
 #include <algorithm>
 #include <atomic>
 #include <mutex>
+#include <type_traits>
 
 #include "vs_internal.h"
 
@@ -938,7 +939,7 @@ __global__ void __launch_bounds__(VS_RING_THREADS, 4) k_subsweep_pring(SubsweepP
     float4 *ring4 = pring_dyn;
     float2 *ring2 = reinterpret_cast<float2 *>(pring_dyn + 6 * (NC / 4) * VS_RING_THREADS);
     int t = blockIdx.x * blockDim.x + threadIdx.x;
-    t = class_thread<NC>(a.g, t, a.n_threads);
+    t = class_thread<NC>(a.colour, t, a.n_threads);
     const bool active = t < a.n_threads;
     Update<float> u;
     if (active) {
@@ -961,7 +962,7 @@ __global__ void __launch_bounds__(VS_RING_THREADS, VS_RING_MINB) k_subsweep_fuse
     float4 *ring4 = ring6_dyn;
     float2 *ring2 = reinterpret_cast<float2 *>(ring6_dyn + 6 * (NC / 4) * VS_RING_THREADS);
     int t = blockIdx.x * blockDim.x + threadIdx.x;
-    t = class_thread<NC>(a.g, t, a.n_threads);
+    t = class_thread<NC>(a.colour, t, a.n_threads);
     const bool active = t < a.n_threads;
     Update<float> u;
     if (active) {
@@ -1083,7 +1084,7 @@ __global__ void __launch_bounds__(VS_RING_THREADS, VS_RING_MINB) k_aus_ring(AusP
     float4 *ring4 = aus_dyn;
     float2 *ring2 = reinterpret_cast<float2 *>(aus_dyn + 6 * (NC / 4) * VS_RING_THREADS);
     int t = blockIdx.x * blockDim.x + threadIdx.x;
-    t = class_thread<NC>(a.g, t, a.n_threads);
+    t = class_thread<NC>(a.colour, t, a.n_threads);
     const bool active = t < a.n_threads;
     Update<float> up;
     if (active) {
@@ -1108,7 +1109,7 @@ __global__ void __launch_bounds__(VS_RING_THREADS, 4) k_aus_pring(AusParams a) {
     float4 *ring4 = ausp_dyn;
     float2 *ring2 = reinterpret_cast<float2 *>(ausp_dyn + 6 * (NC / 4) * VS_RING_THREADS);
     int t = blockIdx.x * blockDim.x + threadIdx.x;
-    t = class_thread<NC>(a.g, t, a.n_threads);
+    t = class_thread<NC>(a.colour, t, a.n_threads);
     const bool active = t < a.n_threads;
     Update<float> up;
     if (active) {
@@ -1218,31 +1219,35 @@ inline int even_smem(int blocks, int smem, int per_sm, int n_sm, int all, int re
     return need >= per_sm ? smem : std::max(smem, std::min(most, (all / need - reserved) & ~127));
 }
 
-// Threads of a launch of n links of a colour class (or of one direction), with g.runs set
-// for it.  18-real links in rows of 20 sites (Lx/4 = 5): a row's class sites are a run of
-// five positions in a line of eight, and a warp that takes 32 sites in order touches parts
-// of 7 or 8 runs with every load.  Six whole runs per warp are 7 % faster for a block, but
-// make a fifteenth more blocks, so they are taken where that costs no further layer of
-// blocks over the SMs, or one among many.  us per class launch, in order / whole runs:
+// Whether a launch of n links of a colour class takes whole runs of sites.  18-real links
+// in rows of 20 sites (Lx/4 = 5): a row's class sites are a run of five positions in a line
+// of eight, and a warp that takes 32 sites in order touches parts of 7 or 8 runs with every
+// load.  Six whole runs per warp are 7 % faster for a block, but make a fifteenth more
+// blocks, so they are taken where that costs no further layer of blocks over the SMs, or
+// one among many.  us per class launch, in order / whole runs:
 // 35,840 links 22.1 / 20.5, 38,400 22.1 / 29.1, 57,600 32.5 / 38.9, 64,000 41.9 / 39.0,
 // 96,000 52.2 / 56.1, 199,680 108.9 / 103.2, 599,040 302.7 / 295.5.  Not with 12 reals,
 // where the mapping gains 0.3 us of 40.3 at 80,000 links but costs the kernel registers
 // (165,888 links 61.1 -> 62.0).  Other rows: 24 sites (five runs of six to a warp) 68.6 ->
 // 69.6 at 165,888 links; 28 sites (four runs of seven) 27.0 -> 24.7 at 50,176 links but
 // 131.5 -> 137.2 at 307,328, whose further blocks cost more than the runs gain.
+constexpr int whole_run_threads(int n) { return (n + 29) / 30 * 32; }
+
 template <int NC>
-int class_threads(Geo &g, int n, bool one_class, int n_sm) {
-    const int whole = (n + 29) / 30 * 32;
+bool whole_runs(const Geo &g, int n, int n_sm) {
     const auto layers = [&](int threads) { return (threads + VS_RING_THREADS * n_sm - 1) / (VS_RING_THREADS * n_sm); };
-    g.runs = NC == 18 && one_class && g.Q == 5 && 14 * layers(whole) <= 15 * layers(n);
-    return g.runs ? whole : n;
+    return NC == 18 && g.Q == 5 && 14 * layers(whole_run_threads(n)) <= 15 * layers(n);
 }
+
+// The Runge-Kutta stages know no colour classes.
+template <class P, class = void> struct HasColour : std::false_type {};
+template <class P> struct HasColour<P, std::void_t<decltype(std::declval<P>().colour)>> : std::true_type {};
 
 // One launch of a link-ring kernel of direction mu out of its four instantiations, evenly
 // spread if it has less than per_sm blocks per SM (0: as they come).  attr_set: where the
 // shared-memory limit has been set, one flag per kernel family.
 template <int NC, class P>
-cudaError_t launch_ring(void (*const kernels[4])(P), int mu, P p, bool one_class, int per_sm,
+cudaError_t launch_ring(void (*const kernels[4])(P), int mu, P p, int per_sm,
                         std::atomic<unsigned long long> &attr_set, cudaStream_t st) {
     constexpr int smem = ring6_smem_bytes<NC>();
     int dev = 0, n_sm = 1, all = 0, reserved = 0, most = smem;
@@ -1255,7 +1260,13 @@ cudaError_t launch_ring(void (*const kernels[4])(P), int mu, P p, bool one_class
         for (int k = 0; k < 4; ++k)
             cudaFuncSetAttribute(kernels[k], cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     });
-    const int blocks = (class_threads<NC>(p.g, p.n_threads, one_class, n_sm) + VS_RING_THREADS - 1) / VS_RING_THREADS;
+    int threads = p.n_threads;
+    if constexpr (HasColour<P>::value)
+        if (p.colour >= 0 && whole_runs<NC>(p.g, p.n_threads, n_sm)) {
+            p.colour |= kRuns;
+            threads = whole_run_threads(p.n_threads);
+        }
+    const int blocks = (threads + VS_RING_THREADS - 1) / VS_RING_THREADS;
     return launch_dependent(kernels[mu], blocks, VS_RING_THREADS,
                             (size_t)even_smem(blocks, smem, per_sm, n_sm, all, reserved, most), st, p);
 }

@@ -45,7 +45,7 @@ cudaError_t launch_subsweep_tpl(bool rect, int mu, const SubsweepParams &p, cuda
             {k_subsweep_pring<NC, 0>, k_subsweep_pring<NC, 1>, k_subsweep_pring<NC, 2>, k_subsweep_pring<NC, 3>},
             {k_subsweep_fused<NC, 0>, k_subsweep_fused<NC, 1>, k_subsweep_fused<NC, 2>, k_subsweep_fused<NC, 3>}};
         static std::atomic<unsigned long long> set[2] = {{0}, {0}};
-        e = launch_ring<NC>(kernels[rect], mu, p, p.colour >= 0, p.crowded ? 0 : kRingPerSM[rect], set[rect], st);
+        e = launch_ring<NC>(kernels[rect], mu, p, p.crowded ? 0 : kRingPerSM[rect], set[rect], st);
     }
     if (e == cudaSuccess && p.defer_idx) {
         if (rect) launch_redecide<NC, true>(mu, p, st);
@@ -70,7 +70,7 @@ cudaError_t launch_aus_tpl(bool rect, int mu, const AusParams &p, cudaStream_t s
             {k_aus_pring<NC, 0>, k_aus_pring<NC, 1>, k_aus_pring<NC, 2>, k_aus_pring<NC, 3>},
             {k_aus_ring<NC, 0>, k_aus_ring<NC, 1>, k_aus_ring<NC, 2>, k_aus_ring<NC, 3>}};
         static std::atomic<unsigned long long> set[2] = {{0}, {0}};
-        return launch_ring<NC>(kernels[rect], mu, p, true, p.crowded ? 0 : kRingPerSM[rect], set[rect], st);
+        return launch_ring<NC>(kernels[rect], mu, p, p.crowded ? 0 : kRingPerSM[rect], set[rect], st);
     }
 }
 

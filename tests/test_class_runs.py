@@ -21,16 +21,17 @@ namespace vs { void count_launches(int) {} }
 template <int NC>
 void row(int lx, int n, bool one_class) {
     const int dims[4] = {lx, 4, 4, 4};
-    vs::Geo g = vs::make_geo(dims);
-    const int threads = vs::class_threads<NC>(g, n, one_class, 152);
+    const bool runs = one_class && vs::whole_runs<NC>(vs::make_geo(dims), n, 152);
+    const int threads = runs ? vs::whole_run_threads(n) : n;
+    const int colour = one_class ? (runs ? 3 | vs::kRuns : 3) : -1;
     std::vector<int> taken(n, 0);
     bool once = threads >= n;
     for (int k = 0; k < (threads + 127) / 128 * 128; ++k) {
-        const int t = vs::class_thread<NC>(g, k, n);
+        const int t = vs::class_thread<NC>(colour, k, n);
         if (t >= 0 && t < n) once &= ++taken[t] == 1;
     }
     for (int c : taken) once &= c == 1;
-    std::printf("%%d %%d %%d %%d %%d %%d %%d\\n", NC, lx, n, one_class, g.runs, threads, once);
+    std::printf("%%d %%d %%d %%d %%d %%d %%d\\n", NC, lx, n, one_class, runs, threads, once);
 }
 int main() {
     for (int n : {%s})
